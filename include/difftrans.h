@@ -449,10 +449,11 @@ dt_status dt_edge_loss_grad(const void* d_topo, int32_t nv, int32_t nf, const fl
  * the values current when it is made).  The traversal is persistent: each
  * lane carries one ray, a warp runs trace_steps node visits per round and
  * refills its idle lanes from the level's queue once trace_refill of them
- * are idle; trace_blocks_per_sm CTAs of 256 threads run per SM.
+ * are idle; trace_blocks_per_sm sizes its grid and register budget in units
+ * of 256 resident threads per SM (CTAs of 128 threads; 5 runs nine of them).
  * shade_blocks_per_sm sizes the grid of the shading and adjoint kernels.
  * bvh_width selects the node format the traversal reads: 2 (binary nodes,
- * 64 B) or 4 (4-wide nodes, 128 B: the binary nodes at even depth with
+ * 32 B: boxes in 16-bit codes, rounded outward) or 4 (4-wide nodes, 128 B: the binary nodes at even depth with
  * their grandchildren as children); both are kept current by build/refit.
  * bvh_builder selects the topology dt_build_bvh builds: 0 = LBVH (Morton
  * codes, radix sort, Karras 2012 hierarchy), 1 = top-down binned surface

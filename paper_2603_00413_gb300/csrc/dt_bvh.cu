@@ -313,6 +313,7 @@ __device__ __forceinline__ void load_box(const float4* box, float3& lo, float3& 
 __global__ void k_refit(const float* __restrict__ V, const int32_t* __restrict__ F, int32_t nf, BvhView B,
                         uint32_t* __restrict__ arrive) {
   const int n_int = B.hdr->n_int;
+  if (blockIdx.x == 0 && threadIdx.x == 0) B.hdr->coarse = 0;  // counted by k_node2_boxes
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nf; i += gridDim.x * blockDim.x) {
     const int tri = B.leaf_tri[i];
     const float3 v0 = load3(V + 3 * F[3 * tri]), v1 = load3(V + 3 * F[3 * tri + 1]), v2 = load3(V + 3 * F[3 * tri + 2]);
@@ -1032,28 +1033,61 @@ __global__ void k_node4_boxes(BvhView B) {
   }
 }
 
-// binary nodes for the 2-wide traversal, from the binary boxes (after each refit)
+// Binary nodes for the 2-wide traversal, from the binary boxes (after each
+// refit): the grid over the scene's box (the union of the root's two child
+// boxes) and every child box coded on it, rounded outward.  The 0.02 steps
+// cover the rounding of (x - lo) inv, at most 65000 steps times 2^-23.
+__device__ __forceinline__ uint32_t code_planes(float lo, float hi, float base, float inv) {
+  const float a = floorf((lo - base) * inv + (kQOffset - 0.02f)), b = ceilf((hi - base) * inv + (kQOffset + 0.02f));
+  return (uint32_t)fminf(fmaxf(a, 0.0f), 65535.0f) | ((uint32_t)fminf(fmaxf(b, 0.0f), 65535.0f) << 16);
+}
+__device__ __forceinline__ float longest_side(const float4* box) {
+  const float4 a = box[0], b = box[1];
+  return fmaxf(fmaxf(b.x - a.x, b.y - a.y), b.z - a.z);
+}
+__device__ __forceinline__ const float4* child_box(const BvhView& B, int c) {
+  return c >= 0 ? B.box_int + 2 * c : B.box_leaf + 2 * (~c);
+}
+
+constexpr int kQCluster = 6;  // levels: a cluster below the grid's resolution holds dozens of triangles
+
 __global__ void k_node2_boxes(BvhView B) {
   const int n_int = B.hdr->n_int;
+  float3 rlo = mk(INFINITY, INFINITY, INFINITY), rhi = mk(-INFINITY, -INFINITY, -INFINITY);
+  const int2 root = B.bin_child[0];
+  for (int k = 0; k < 2; ++k) {
+    const int c = k ? root.y : root.x;
+    if (c == kNoChild) continue;
+    const float4 a = child_box(B, c)[0], b = child_box(B, c)[1];
+    rlo = mk(fminf(rlo.x, a.x), fminf(rlo.y, a.y), fminf(rlo.z, a.z));
+    rhi = mk(fmaxf(rhi.x, b.x), fmaxf(rhi.y, b.y), fmaxf(rhi.z, b.z));
+  }
+  const float step = fmaxf(fmaxf(fmaxf(rhi.x - rlo.x, rhi.y - rlo.y), rhi.z - rlo.z), 1e-30f) * (1.0f / kQSteps);
+  const float inv = 1.0f / step;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n_int; j += gridDim.x * blockDim.x) {
-    const int2 ch = B.bin_child[j];
-    float3 lo[2], hi[2];
-    const int c2[2] = {ch.x, ch.y};
-    for (int k = 0; k < 2; ++k) {
-      lo[k] = mk(INFINITY, INFINITY, INFINITY);
-      hi[k] = mk(-INFINITY, -INFINITY, -INFINITY);
-      const int x = c2[k];
-      if (x != kNoChild) {
-        const float4* bx = x >= 0 ? B.box_int + 2 * x : B.box_leaf + 2 * (~x);
-        const float4 a = bx[0], b = bx[1];
-        lo[k] = mk(a.x, a.y, a.z);
-        hi[k] = mk(b.x, b.y, b.z);
-      }
+    if (j == 0) {
+      B.hdr->q[0] = rlo.x; B.hdr->q[1] = rlo.y; B.hdr->q[2] = rlo.z; B.hdr->q[3] = step;
+      B.hdr->hi[0] = rhi.x; B.hdr->hi[1] = rhi.y; B.hdr->hi[2] = rhi.z;
     }
-    B.node2[4 * j + 0] = make_float4(lo[0].x, hi[0].x, lo[0].y, hi[0].y);
-    B.node2[4 * j + 1] = make_float4(lo[1].x, hi[1].x, lo[1].y, hi[1].y);
-    B.node2[4 * j + 2] = make_float4(lo[0].z, hi[0].z, lo[1].z, hi[1].z);
-    reinterpret_cast<int4*>(B.node2)[4 * j + 3] = make_int4(ch.x, ch.y, 0, 0);
+    const int2 ch = B.bin_child[j];
+    uint32_t w[6];
+    for (int k = 0; k < 2; ++k) {
+      const int c = k ? ch.y : ch.x;
+      w[3 * k] = w[3 * k + 1] = w[3 * k + 2] = 0x0000ffffu;
+      if (c == kNoChild) continue;
+      const float4 a = child_box(B, c)[0], b = child_box(B, c)[1];
+      w[3 * k] = code_planes(a.x, b.x, rlo.x, inv);
+      w[3 * k + 1] = code_planes(a.y, b.y, rlo.y, inv);
+      w[3 * k + 2] = code_planes(a.z, b.z, rlo.z, inv);
+    }
+    B.node2[2 * j] = make_uint4(w[0], w[1], w[2], w[3]);
+    B.node2[2 * j + 1] = make_uint4(w[4], w[5], (uint32_t)ch.x, (uint32_t)ch.y);
+    // a node the grid cannot resolve, kQCluster levels below another one
+    if (n_int > 256 && longest_side(B.box_int + 2 * j) < 4.0f * step) {
+      int p = j;
+      for (int l = 0; l < kQCluster && p > 0; ++l) p = B.parent[p];
+      if (p > 0 && p < n_int && longest_side(B.box_int + 2 * p) < 4.0f * step) atomicAdd(&B.hdr->coarse, 1);
+    }
   }
 }
 
@@ -1089,6 +1123,7 @@ __global__ void k_bvh_header(BvhHeader* h, int32_t nf) {
   h->n_int = nf > 1 ? nf - 1 : 1;
   h->n4 = 0;
   h->corrupt = 0;
+  h->coarse = 0;
 }
 
 // scratch layout for build/refit

@@ -90,6 +90,7 @@ __device__ __forceinline__ uint32_t tiled_pixel(uint32_t q, uint32_t w, uint32_t
 // launch less per render than a clearing kernel of its own).
 __global__ void k_camera(WsView W, unsigned long long capacity) {
   const SceneEntry& E = W.ent[blockIdx.y];
+  if (blockIdx.x == 0 && threadIdx.x == 0 && E.bh->coarse > kQCoarse) atomicOr(&W.hdr->exact, 1u);
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
     W.hdr->capacity = capacity;
     W.hdr->ring = W.ring;
@@ -142,48 +143,59 @@ __device__ __forceinline__ float safe_inv(float v) {
   return 1.0f / (fabsf(v) > 1e-20f ? v : copysignf(1e-20f, v));
 }
 
-struct ClosestHit {
-  float t, b1, b2;
+// Where a traversal puts the hit it has found so far: t and the triangle
+// stay in registers (they bound the search), (t, b1, b2, triangle) goes to
+// the record whenever a nearer hit is found -- once or twice per ray, which
+// costs less than two more registers per lane would.
+struct HitSoFar {
+  float t;
   int tri;
+  float4* rec;
 };
 
 // Moller-Trumbore on a leaf; keeps the smallest t > tmin, ties to the smaller
-// triangle id, skipping the triangle the ray starts on.
+// triangle id, skipping the triangle the ray starts on.  No early returns:
+// the lanes of a warp test different triangles, and a branch per condition
+// runs the block's pieces one after another with a few lanes each (with the
+// branches in visit_node2 below gone as well: 13.2 -> 11.1 ms of traversal per
+// 48-view genus-2 step).
 __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, int leaf, float3 o, float3 d, int src,
-                                          float tmin, ClosestHit& h, uint32_t& ntest) {
+                                          float tmin, HitSoFar& h, uint32_t& ntest) {
   const float4 a = __ldg(tris + 3 * leaf), b = __ldg(tris + 3 * leaf + 1), c = __ldg(tris + 3 * leaf + 2);
   const int id = __float_as_int(a.w);
-  if (id == src) return;
-  ++ntest;
+  ntest += id != src ? 1u : 0u;
   // the arithmetic of intersect_known, written out (the checkpointed
   // backward calls that function on the same inputs and gets the same bits)
   const float3 v0 = xyz(a), e1 = xyz(b), e2 = xyz(c);
   const float3 p = cross(d, e2);
   const float det = dot(e1, p);
-  if (det == 0.0f) return;
-  const float inv = 1.0f / det;
+  const float inv = __frcp_rn(det);
   const float3 s = o - v0;
   const float b1 = dot(s, p) * inv;
   const float3 q = cross(s, e1);
   const float b2 = dot(d, q) * inv;
   const float t = dot(e2, q) * inv;
   const float b0 = 1.0f - b1 - b2;
-  if (!(t > tmin)) return;
-  if (b1 < 0.0f || b2 < 0.0f || b0 < 0.0f) return;
-  if (t < h.t || (t == h.t && id < h.tri)) {
-    h.t = t; h.b1 = b1; h.b2 = b2; h.tri = id;
+  const bool hit = id != src && det != 0.0f && t > tmin && !(b1 < 0.0f) && !(b2 < 0.0f) && !(b0 < 0.0f) &&
+                   (t < h.t || (t == h.t && id < h.tri));
+  if (hit) {
+    h.t = t;
+    h.tri = id;
+    *h.rec = make_float4(t, b1, b2, __int_as_float(id));
   }
 }
 
-// Reads of BVH nodes with 256-bit loads (sm_100 and later): a 64-byte
-// binary node is two loads instead of four 128-bit ones, which halves the
-// load instructions a visit issues through L1 (the traversal is bound by
-// instruction issue; measured 1.6 % faster than four 128-bit loads).  The
-// BVH buffer is 256-byte aligned and every node starts at a multiple of 64
-// bytes past it, so each load is 32-byte aligned.
+// 256-bit loads (sm_100 and later): a 32-byte binary node is one load, a
+// 4-wide node four.  The BVH buffer is 256-byte aligned and every node starts
+// at a multiple of 32 bytes past it.
 __device__ __forceinline__ void ld_nc_v8(const float4* p, float4& a, float4& b) {
   asm("ld.global.nc.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
       : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
+      : "l"(p));
+}
+__device__ __forceinline__ void ld_node2(const uint4* p, uint4& a, uint4& b) {
+  asm("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+      : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
       : "l"(p));
 }
 __device__ __forceinline__ float4 ld_nc_l1na(const float4* p) {
@@ -191,72 +203,175 @@ __device__ __forceinline__ float4 ld_nc_l1na(const float4* p) {
   asm("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p));
   return r;
 }
-__device__ __forceinline__ void ld_node2(const float4* Np, float4& n0, float4& n1, float4& n2, int4& n3) {
-  float4 c;
-  ld_nc_v8(Np, n0, n1);
-  ld_nc_v8(Np + 2, n2, c);
-  n3 = make_int4(__float_as_int(c.x), __float_as_int(c.y), __float_as_int(c.z), __float_as_int(c.w));
+
+// A ray as the coded boxes of the binary nodes see it.  Per axis the plane of
+// code c is met at t = fma(2^23 + c, s, b) with s = step / d: 2^23 + c is the
+// float whose bits are 0x4B000000 | c, so one byte permute both extracts a code
+// and converts it, and its selector picks the near plane (lower for d > 0,
+// upper for d < 0), so no min or max per axis is needed.  b = (lo - o) / d -
+// (2^23 + kQOffset) s is rounded down for the near planes and up for the far
+// ones; w covers the roundings of (lo - o) / d (three, the reciprocal's among
+// them: 2.4e-7 of it, and 0.008 steps) and of the plane's own fma (6e-8 of
+// it, and 0.004 steps), whatever the distance of the origin.  So a box that
+// the exact ray touches is never culled.
+struct RayAxis {
+  float s, b_near, b_far;
+  uint32_t sel;
+};
+struct RayQ {
+  RayAxis x, y, z;
+};
+__device__ __forceinline__ RayAxis ray_axis(float o, float d, float lo, float step) {
+  RayAxis a;
+  float inv;  // a zero component is taken as +-1e-20, so no 0 * inf appears
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(fabsf(d) > 1e-20f ? d : copysignf(1e-20f, d)));
+  a.s = step * inv;
+  const float r = (lo - o) * inv, w = fabsf(r) * 4e-7f + fabsf(a.s) * 0.02f;
+  a.b_near = __fmaf_rd(-8388608.0f - kQOffset, a.s, r - w);
+  a.b_far = __fmaf_ru(-8388608.0f - kQOffset, a.s, r + w);
+  a.sel = inv < 0.0f ? 0x7632u : 0x7610u;
+  return a;
+}
+__device__ __forceinline__ RayQ ray_q(float3 o, float3 d, const BvhHeader* __restrict__ bh) {
+  const float4 q = __ldg(reinterpret_cast<const float4*>(bh->q));
+  return RayQ{ray_axis(o.x, d.x, q.x, q.w), ray_axis(o.y, d.y, q.y, q.w), ray_axis(o.z, d.z, q.z, q.w)};
+}
+__device__ __forceinline__ float near_plane(const RayAxis& a, uint32_t w) {
+  return fmaf(__uint_as_float(__byte_perm(w, 0x4B000000u, a.sel)), a.s, a.b_near);
+}
+__device__ __forceinline__ float far_plane(const RayAxis& a, uint32_t w) {
+  return fmaf(__uint_as_float(__byte_perm(w, 0x4B000000u, a.sel ^ 0x22u)), a.s, a.b_far);
+}
+__device__ __forceinline__ bool slab_q(const RayQ& r, uint32_t x, uint32_t y, uint32_t z, float tmin, float tmax,
+                                       float& tnear) {
+  tnear = fmaxf(fmaxf(near_plane(r.x, x), near_plane(r.y, y)), fmaxf(near_plane(r.z, z), tmin));
+  return tnear <= fminf(fminf(far_plane(r.x, x), far_plane(r.y, y)), fminf(far_plane(r.z, z), tmax));
 }
 
-// One visit of binary node `node`: slab tests on its two children, leaf
-// children intersected at once, internal children that were hit entered
-// nearest first with the other pushed.  Returns the next node, or -1 when the
-// stack is empty.  (Used by the closest-hit tool; the persistent traversal
-// uses visit_node2_deferred.)
-__device__ __forceinline__ int visit_node2(const float4* __restrict__ node2, const float4* __restrict__ tris, int node,
-                                           float3 o, float3 d, float3 idir, int src, float tmin, ClosestHit& h,
-                                           int* stack, int& sp, bool& overflow, uint32_t& ntest) {
-  float4 n0, n1, n2;
-  int4 n3;
-  ld_node2(node2 + 4 * node, n0, n1, n2, n3);
-  float tn0, tn1;
-  bool h0 = slab(o, idir, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, tmin, h.t, tn0);
-  bool h1 = slab(o, idir, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, tmin, h.t, tn1);
-  if (h0 && n3.x < 0) { test_leaf(tris, ~n3.x, o, d, src, tmin, h, ntest); h0 = false; }
-  if (h1 && n3.y < 0) { test_leaf(tris, ~n3.y, o, d, src, tmin, h, ntest); h1 = false; }
-  if (h0 && h1) {
-    int nearc = n3.x, farc = n3.y;
-    if (tn1 < tn0) { nearc = n3.y; farc = n3.x; }
-    if (sp < kTraceStack) stack[sp++] = farc; else overflow = true;
-    return nearc;
-  }
-  if (h0) return n3.x;
-  if (h1) return n3.y;
-  return sp > 0 ? stack[--sp] : -1;
+// One visit of binary node `node`: both children's boxes; hit leaves join the
+// queue p0..p2 (newest first), of the internal children that were hit the
+// nearer is returned and the other pushed, and with none the stack is popped
+// (its bottom entry is -1, the end of the search).  Selects and predicated
+// accesses instead of branches, as in test_leaf.  The caller intersects every
+// lane's queued triangles together after a few visits, so that the triangle
+// test runs as one block per few visits for the warp, and visits only while
+// fewer than two are queued, so three slots suffice.
+__device__ __forceinline__ int visit_node2(const uint4* __restrict__ node2, int node, const RayQ& r, float tmin,
+                                           float tmax, int* stack, int& sp, int& p0, int& p1, int& p2) {
+  uint4 a, b;
+  ld_node2(node2 + 2 * node, a, b);
+  const int c0 = (int)b.z, c1 = (int)b.w;
+  float t0, t1;
+  const bool h0 = slab_q(r, a.x, a.y, a.z, tmin, tmax, t0), h1 = slab_q(r, a.w, b.x, b.y, tmin, tmax, t1);
+  const bool l0 = h0 && c0 < 0, l1 = h1 && c1 < 0, i0 = h0 && !l0, i1 = h1 && !l1;
+  p2 = l0 ? p1 : p2;
+  p1 = l0 ? p0 : p1;
+  p0 = l0 ? ~c0 : p0;
+  p2 = l1 ? p1 : p2;
+  p1 = l1 ? p0 : p1;
+  p0 = l1 ? ~c1 : p0;
+  const bool swap = !i0 || (i1 && t1 < t0);
+  int next = swap ? c1 : c0;
+  if (i0 && i1) stack[sp] = swap ? c0 : c1;
+  sp += i0 && i1 ? 1 : 0;
+  if (!i0 && !i1) next = stack[--sp];
+  return next;
 }
 
-// The binary visit of the persistent traversal: the same node test as
-// visit_node2, but a hit leaf is queued in the lane's pending slots rather
-// than intersected at once.  The kernel intersects every lane's pending
-// triangles together after a few visits, so the triangle test runs as one
-// block per few visits for the warp instead of one or two blocks per visit
-// in which a few lanes work while the rest wait.  The caller visits only
-// while fewer than two triangles are pending, so three slots always suffice.
-__device__ __forceinline__ void push_pending(int leaf, int& p0, int& p1, int& p2) {
-  if (p0 < 0) p0 = leaf;
-  else if (p1 < 0) p1 = leaf;
-  else p2 = leaf;
-}
-__device__ __forceinline__ int visit_node2_deferred(const float4* __restrict__ node2, int node, float3 o, float3 idir,
-                                                    float tmin, float tmax, int* stack, int& sp, bool& overflow,
-                                                    int& p0, int& p1, int& p2) {
-  float4 n0, n1, n2;
-  int4 n3;
-  ld_node2(node2 + 4 * node, n0, n1, n2, n3);
-  float tn0, tn1;
-  bool h0 = slab(o, idir, n0.x, n0.y, n0.z, n0.w, n2.x, n2.y, tmin, tmax, tn0);
-  bool h1 = slab(o, idir, n1.x, n1.y, n1.z, n1.w, n2.z, n2.w, tmin, tmax, tn1);
-  if (h0 && n3.x < 0) { push_pending(~n3.x, p0, p1, p2); h0 = false; }
-  if (h1 && n3.y < 0) { push_pending(~n3.y, p0, p1, p2); h1 = false; }
-  if (h0 && h1) {
-    int nearc = n3.x, farc = n3.y;
-    if (tn1 < tn0) { nearc = n3.y; farc = n3.x; }
-    if (sp < kTraceStack) stack[sp++] = farc; else overflow = true;
-    return nearc;
+// Up to kLeafEvery visits, then the triangles they queued; true once the
+// search is over.  stack: kTraceStack entries above the bottom one, and room
+// for one group's pushes, which are checked here.
+constexpr int kLeafEvery = 6;  // (8 visits: 1 % slower on the 52k-triangle mesh, 1 % faster on the 1M one)
+constexpr int kStackWords = 1 + kTraceStack + kLeafEvery;
+__device__ __forceinline__ bool visit_group(const uint4* __restrict__ node2, const float4* __restrict__ tris,
+                                            const RayQ& r, float3 o, float3 d, int src, float tmin, int* stack,
+                                            int& sp, int& node, HitSoFar& h, int& visits, uint32_t& ntest,
+                                            bool& overflow) {
+  int p0 = -1, p1 = -1, p2 = -1;
+  for (int j = 0; j < kLeafEvery && node >= 0 && p1 < 0; ++j, ++visits)
+    node = visit_node2(node2, node, r, tmin, h.t, stack, sp, p0, p1, p2);
+  while (p0 >= 0) {
+    test_leaf(tris, p0, o, d, src, tmin, h, ntest);
+    p0 = p1;
+    p1 = p2;
+    p2 = -1;
   }
-  if (h0) return n3.x;
-  if (h1) return n3.y;
-  return sp > 0 ? stack[--sp] : -1;
+  if (sp > kTraceStack + 1) {
+    overflow = true;
+    node = -1;
+  }
+  return node < 0;
+}
+
+// Closest hit through the exact boxes of the refit, for scenes that the coded
+// boxes' grid cannot resolve (BvhHeader::coarse); the same hits, slower.  A
+// tree traversal visits every node at most once, so more than max_iter = 2
+// n_int + 8 visits means a corrupt hierarchy: give up and flag it.
+__device__ __forceinline__ bool closest_hit_exact(const BvhHeader* bh, int32_t nf, float3 o, float3 d, int src,
+                                                  float tmin, int max_iter, HitSoFar& h, uint32_t& nvis,
+                                                  uint32_t& ntest) {
+  const BvhView B = bvh_view(bh, nf);
+  const float3 idir = mk(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
+  int stack[kTraceStack];
+  int sp = 0, node = 0, it = 0;
+  bool ok = true;
+  while (node >= 0) {
+    if (it >= max_iter) {
+      ok = false;
+      break;
+    }
+    ++it;
+    const int2 ch = B.bin_child[node];
+    int c[2] = {ch.x, ch.y};
+    float tn[2];
+    bool in[2];
+    for (int k = 0; k < 2; ++k) {
+      in[k] = false;
+      if (c[k] == kNoChild) continue;
+      const float4* bx = c[k] >= 0 ? B.box_int + 2 * c[k] : B.box_leaf + 2 * (~c[k]);
+      const float4 lo = bx[0], hi = bx[1];
+      const bool hb = slab(o, idir, lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, tmin, h.t, tn[k]);
+      if (hb && c[k] < 0) test_leaf(B.tris, ~c[k], o, d, src, tmin, h, ntest);
+      in[k] = hb && c[k] >= 0;
+    }
+    if (in[0] && in[1]) {
+      const int first = tn[1] < tn[0] ? 1 : 0;
+      if (sp < kTraceStack) stack[sp++] = c[1 - first]; else ok = false;
+      node = c[first];
+    } else {
+      node = in[0] ? c[0] : in[1] ? c[1] : sp > 0 ? stack[--sp] : -1;
+    }
+  }
+  nvis += (uint32_t)it;
+  return ok;
+}
+
+// Level k of a render one of whose scenes needs the exact boxes
+// (WsHeader::exact): a function of its own, called before the traversal's
+// loop, so that the loop's registers need not live across the call.
+__device__ __noinline__ void trace_level_exact(const WsView W, int k, int sorted) {
+  WsHeader* H = W.hdr;
+  const uint32_t n = level_size(H, k), start = H->level_start[k];
+  const int n_scenes = W.th->n;
+  uint32_t nvis = 0, ntest = 0;
+  bool ok = true;
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+    const uint32_t pos = sorted ? W.sflag[start + i] : i;
+    if (pos >= n) {
+      ok = false;
+      continue;
+    }
+    const uint32_t a = start + pos;
+    const float4 ro = W.ray_o[a], rd = W.ray_d[a], rw = W.ray_w[a];
+    const SceneEntry& E = W.ent[find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w))];
+    HitSoFar h{INFINITY, -1, W.hit + hit_slot(W, k, a, pos)};
+    if (E.bh->corrupt) ok = false;
+    else ok &= closest_hit_exact(E.bh, E.nf, xyz(ro), xyz(rd), __float_as_int(rw.w), E.t_min, E.max_iter, h, nvis, ntest);
+    if (h.tri < 0) *h.rec = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+  }
+  warp_add_u64(&H->counters[CNT_NODES], nvis);
+  warp_add_u64(&H->counters[CNT_TRIS], ntest);
+  if (__any_sync(kFull, !ok) && (threadIdx.x & 31) == 0) atomicOr(&H->status, ST_STACK_OVERFLOW);
 }
 
 // The 4-wide visit of the persistent traversal, with hit leaves queued as
@@ -310,45 +425,31 @@ __device__ __forceinline__ int visit_node4_deferred(const float4* __restrict__ n
 }
 
 
-// A tree traversal visits every node at most once, so more than max_iter
-// = 2 n_int + 8 visits means a corrupt hierarchy: give up and flag it.
-__device__ __forceinline__ ClosestHit closest_hit(const float4* __restrict__ node2, const float4* __restrict__ tris,
-                                                  float3 o, float3 d, int src, float tmin, int max_iter,
-                                                  uint32_t& nvis, uint32_t& ntest, bool& overflow) {
-  ClosestHit h{INFINITY, 0.f, 0.f, -1};
-  const float3 idir = mk(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
-  int stack[kTraceStack];
-  int sp = 0;
-  int node = 0;
-  for (int it = 0; node >= 0; ++it) {
-    if (it >= max_iter) {
-      overflow = true;
-      break;
-    }
-    ++nvis;
-    node = visit_node2(node2, tris, node, o, d, idir, src, tmin, h, stack, sp, overflow, ntest);
-  }
-  return h;
-}
-
 // Persistent traversal of level k with dynamic refill.  Every lane carries
 // its own ray; a warp runs up to `steps` node visits per round, then, when
 // at least `refill` lanes have finished, hands them new segments from a
 // batch of kTraceClaim it claimed from the level's cursor with one atomic.
-// Within a round, leaves hit by a visit are queued per lane and intersected
-// for the whole warp every kLeafEvery visits.  A warp stops when the level
+// A claim is one warp's width, so that the warps run out of work together:
+// with 64 the end of a level of 0.7M rays waited a quarter of its time for
+// the warps that had claimed last (12 views of 509x383: 2.88 -> 2.50 ms of
+// traversal).  Within a round, leaves hit by a visit are queued per lane and
+// intersected for the whole warp every kLeafEvery visits.  A warp stops when the level
 // is exhausted and its last ray is done.  sorted != 0: position i of the
 // level is the segment the traversal order put there (its flag word holds
 // it until the shading pass rewrites it).
 // kBatch = false: one scene, whose entry E0 arrives as a kernel parameter
 // (uniform constant-bank reads); true: each ray looks its scene up.
-constexpr int kTraceClaim = 64;  // segments a warp claims from the level cursor at once
-constexpr int kLeafEvery = 6;    // node visits between the warp's batched triangle tests
+constexpr int kTraceClaim = 32;  // segments a warp claims from the level cursor at once (at least its lanes)
+constexpr int kTraceThreads = 128;
 
 template <int kMinBlocks, int kWidth, bool kBatch>
-__global__ void __launch_bounds__(256, kMinBlocks) k_trace(WsView W, int k, int steps, int refill,
+__global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, int k, int steps, int refill,
                                                            const SceneEntry E0, int sorted) {
   WsHeader* H = W.hdr;
+  if (kWidth == 2 && H->exact) {
+    trace_level_exact(W, k, sorted);
+    return;
+  }
   uint32_t* cursor = &H->fetch[k];
   const int n_scenes = kBatch ? W.th->n : 1;
   const uint32_t n = level_size(H, k);
@@ -360,15 +461,18 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_trace(WsView W, int k, int 
   uint32_t nvis = 0, ntest = 0;
   bool overflow = false;
   bool active = false, exhausted = false;
-  uint32_t a = 0;
-  float3 o = mk(0.f, 0.f, 0.f), d = o, idir = o;
+  float3 o = mk(0.f, 0.f, 0.f), d = o, idir = o;  // idir: the 4-wide nodes' slab tests
+  RayQ rq = {};                                   // the binary nodes'
   int src = -1, node = 0, sp = 0, iters = 0;
   int max_iter = kBatch ? 0 : (E0.bh->corrupt ? 0 : E0.max_iter);  // a tree that failed validation is not traced
   float tmin = E0.t_min;
-  const float4* nodes = kWidth == 4 ? E0.node4 : E0.node2;
+  const BvhHeader* bh = E0.bh;
+  const uint4* node2 = E0.node2;
+  const float4* node4 = E0.node4;
   const float4* tris = E0.tris;
-  ClosestHit h{INFINITY, 0.f, 0.f, -1};
-  int stack[kTraceStack];
+  HitSoFar h{INFINITY, -1, nullptr};
+  int stack[kStackWords];
+  stack[0] = -1;
   // the warp's claimed batch [qb, qe) of the level's segments: one atomic on
   // the level cursor per kTraceClaim segments, not one per refill.  Warp w
   // starts with batch w of the level without an atomic, of B =
@@ -415,24 +519,27 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_trace(WsView W, int k, int 
         const uint32_t pos = order ? __ldg(order + i) : i;
         if (pos >= n) overflow = true;  // not a permutation of the level: reported, not traced
         else {
-          a = start + pos;
+          const uint32_t a = start + pos;
           // read once here: not allocated in L1, so they do not evict BVH
           // nodes (L2 keeps them for the shading pass that follows)
           const float4 ro = ld_nc_l1na(W.ray_o + a), rd = ld_nc_l1na(W.ray_d + a), rw = ld_nc_l1na(W.ray_w + a);
           if (kBatch) {
             const SceneEntry& E = W.ent[find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w))];
-            nodes = kWidth == 4 ? E.node4 : E.node2;
+            bh = E.bh;
+            node2 = E.node2;
+            node4 = E.node4;
             tris = E.tris;
-            max_iter = E.bh->corrupt ? 0 : E.max_iter;
+            max_iter = bh->corrupt ? 0 : E.max_iter;
             tmin = E.t_min;
           }
           o = xyz(ro);
           d = xyz(rd);
-          idir = mk(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
+          if (kWidth == 4) idir = mk(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
+          else rq = ray_q(o, d, bh);
           src = __float_as_int(rw.w);
-          h = ClosestHit{INFINITY, 0.f, 0.f, -1};
+          h = HitSoFar{INFINITY, -1, W.hit + hit_slot(W, k, a, pos)};
           node = 0;
-          sp = 0;
+          sp = kWidth == 4 ? 0 : 1;
           iters = 0;
           active = true;
         }
@@ -447,26 +554,13 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_trace(WsView W, int k, int 
     bool done = iters >= max_iter;
     if (!done) {
       if (kWidth == 2) {
-        // visits in groups of kLeafEvery, then the pending triangles of the
-        // whole warp at once (see visit_node2_deferred)
-        int p0 = -1, p1 = -1, p2 = -1;
-        while (st < steps) {
-          for (int j = 0; j < kLeafEvery && node >= 0 && p1 < 0; ++j, ++st)
-            node = visit_node2_deferred(nodes, node, o, idir, tmin, h.t, stack, sp, overflow, p0, p1, p2);
-          if (p0 >= 0) test_leaf(tris, p0, o, d, src, tmin, h, ntest);
-          if (p1 >= 0) test_leaf(tris, p1, o, d, src, tmin, h, ntest);
-          if (p2 >= 0) test_leaf(tris, p2, o, d, src, tmin, h, ntest);
-          p0 = p1 = p2 = -1;
-          if (node < 0) {
-            done = true;
-            break;
-          }
-        }
+        while (st < steps && !done)
+          done = visit_group(node2, tris, rq, o, d, src, tmin, stack, sp, node, h, st, ntest, overflow);
       } else {
         int p0 = -1, p1 = -1, p2 = -1, p3 = -1;
         while (st < steps) {
           for (int j = 0; j < kLeafEvery && node >= 0 && p0 < 0; ++j, ++st)
-            node = visit_node4_deferred(nodes, node, o, idir, tmin, h.t, stack, sp, overflow, p0, p1, p2, p3);
+            node = visit_node4_deferred(node4, node, o, idir, tmin, h.t, stack, sp, overflow, p0, p1, p2, p3);
           if (p0 >= 0) test_leaf(tris, p0, o, d, src, tmin, h, ntest);
           if (p1 >= 0) test_leaf(tris, p1, o, d, src, tmin, h, ntest);
           if (p2 >= 0) test_leaf(tris, p2, o, d, src, tmin, h, ntest);
@@ -484,8 +578,7 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_trace(WsView W, int k, int 
     }
     if (done) {
       if (node >= 0) overflow = true;  // stopped by the guard
-      W.hit[hit_slot(W, k, a, a - start)] = h.tri >= 0 ? make_float4(h.t, h.b1, h.b2, __int_as_float(h.tri))
-                                                       : make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+      if (h.tri < 0) *h.rec = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
       active = false;
     }
   }
@@ -507,11 +600,12 @@ __global__ void __launch_bounds__(256, kMinBlocks) k_trace(WsView W, int k, int 
 }
 
 // Closest hit of arbitrary rays (tooling and tests).
-__global__ void k_closest_hit_rays(const float4* __restrict__ nodes, const float4* __restrict__ tris,
-                                   const float* __restrict__ o, const float* __restrict__ d,
-                                   const int32_t* __restrict__ src, int32_t n, const BvhHeader* bh, float tmin,
-                                   int max_iter, int32_t* __restrict__ tri, float* __restrict__ tbb) {
-  const bool corrupt = bh->corrupt != 0;
+__global__ void __launch_bounds__(128) k_closest_hit_rays(const uint4* __restrict__ nodes,
+                                                          const float4* __restrict__ tris, const float* __restrict__ o,
+                                                          const float* __restrict__ d, const int32_t* __restrict__ src,
+                                                          int32_t n, const BvhHeader* bh, float tmin, int max_iter,
+                                                          int32_t* __restrict__ tri, float* __restrict__ tbb) {
+  const bool corrupt = bh->corrupt != 0, exact = bh->coarse > kQCoarse;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     uint32_t nv = 0, nt = 0;
     bool ovf = false;
@@ -519,12 +613,27 @@ __global__ void k_closest_hit_rays(const float4* __restrict__ nodes, const float
       tri[i] = -2;
       continue;
     }
-    const ClosestHit h = closest_hit(nodes, tris, load3(o + 3 * i), load3(d + 3 * i), src ? src[i] : -1, tmin,
-                                     max_iter, nv, nt, ovf);
+    const float3 ro = load3(o + 3 * i), rd = load3(d + 3 * i);
+    const int s = src ? src[i] : -1;
+    float4 rec = make_float4(0.f, 0.f, 0.f, 0.f);
+    HitSoFar h{INFINITY, -1, &rec};
+    if (exact) {
+      ovf = !closest_hit_exact(bh, bh->nf, ro, rd, s, tmin, max_iter, h, nv, nt);
+    } else {
+      const RayQ rq = ray_q(ro, rd, bh);
+      int stack[kStackWords];
+      stack[0] = -1;
+      int sp = 1, node = 0, visits = 0;
+      while (!visit_group(nodes, tris, rq, ro, rd, s, tmin, stack, sp, node, h, visits, nt, ovf))
+        if (visits >= max_iter) {
+          ovf = true;
+          break;
+        }
+    }
     tri[i] = ovf ? -2 : h.tri;
-    tbb[3 * i] = h.tri >= 0 ? h.t : 0.f;
-    tbb[3 * i + 1] = h.b1;
-    tbb[3 * i + 2] = h.b2;
+    tbb[3 * i] = rec.x;
+    tbb[3 * i + 1] = rec.y;
+    tbb[3 * i + 2] = rec.z;
   }
 }
 
@@ -561,7 +670,7 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeMinBlocks) k_shade(WsView
   // positions of level k+1 that can hold a bucket (its ring half, or the arena)
   const unsigned long long key_room = W.ring ? (unsigned long long)W.ring : H->capacity - next_start;
   float3 box_lo = mk(0.f, 0.f, 0.f), box_scale = box_lo;
-  if (!kBatch && order_bits) scene_order_box(E0.node2, box_lo, box_scale);
+  if (!kBatch && order_bits) scene_order_box(E0.bh, box_lo, box_scale);
   uint32_t c_hit = 0, c_miss = 0, c_disc = 0, c_back = 0, c_tir = 0, c_med = 0;
   bool overflow = false;
   // CTA-wide tiles, so that the children of a tile are appended with one
@@ -629,7 +738,7 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeMinBlocks) k_shade(WsView
             cwr = make_float4(Wt.x * h.R, Wt.y * h.R, Wt.z * h.R, __int_as_float(tri));
             nchild = 1;
             if (kBatch && order_bits) {
-              scene_order_box(E.node2, box_lo, box_scale);
+              scene_order_box(E.bh, box_lo, box_scale);
               scene_id = (uint32_t)scene;
             }
             if (!h.tir) {
@@ -849,18 +958,21 @@ void launch_order_clear(const WsView& W, int bits, cudaStream_t s);
 static int shade_blocks() { return g_tuning.shade_blocks_per_sm * num_sms(); }
 static int n_int_of(int32_t nf) { return nf > 1 ? nf - 1 : 1; }
 
-// The traversal is compiled for 2..8 resident CTAs of 256 threads per SM (the
-// register budget per thread follows) and for the 2- and 4-wide node
-// formats; the tuning picks the variant and the persistent grid is
-// trace_blocks_per_sm CTAs per SM.
+// The traversal runs in CTAs of 128 threads and is compiled for several
+// register budgets; trace_blocks_per_sm picks one in units of 256 resident
+// threads per SM.  The default 5 is the 56-register variant, nine CTAs (36
+// warps) per SM: at 48 registers and ten CTAs the ray's plane constants spill
+// (11.3 against 11.1 ms per 48-view genus-2 step, 23.0 against 22.4 ms on the
+// million-triangle step), at 64 and eight too few warps hide the node reads
+// (11.3 and 23.4 ms).
 template <int kWidth, bool kBatch, typename... A>
 static void launch_trace_w(int bps, cudaStream_t s, A... a) {
-  const int g = bps * num_sms();
+  const int sms = num_sms();
   switch (bps) {
-    case 1: case 2: case 3: k_trace<3, kWidth, kBatch><<<g, 256, 0, s>>>(a...); break;
-    case 4: k_trace<4, kWidth, kBatch><<<g, 256, 0, s>>>(a...); break;
-    case 5: k_trace<5, kWidth, kBatch><<<g, 256, 0, s>>>(a...); break;
-    default: k_trace<6, kWidth, kBatch><<<g, 256, 0, s>>>(a...); break;
+    case 1: case 2: case 3: k_trace<6, kWidth, kBatch><<<2 * bps * sms, kTraceThreads, 0, s>>>(a...); break;
+    case 4: k_trace<8, kWidth, kBatch><<<8 * sms, kTraceThreads, 0, s>>>(a...); break;
+    case 5: k_trace<9, kWidth, kBatch><<<9 * sms, kTraceThreads, 0, s>>>(a...); break;
+    default: k_trace<12, kWidth, kBatch><<<2 * bps * sms, kTraceThreads, 0, s>>>(a...); break;
   }
 }
 static int traversal_limit(int32_t nf) { return 2 * n_int_of(nf) + 8; }
