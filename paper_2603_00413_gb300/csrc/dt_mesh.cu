@@ -183,35 +183,141 @@ __device__ __forceinline__ void store3(float* p, float3 v) {
   p[2] = v.z;
 }
 
-// one atomic per CTA for each of three column sums (a warp-level atomic on
-// three addresses from every warp of a large mesh serialises); called by
-// every thread of the CTA after its loop
-__device__ __forceinline__ void block_add3(float* dst, float3 v) {
-  __shared__ float part[3][32];
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+// ---- conjugate gradients in one cooperative kernel ---------------------------
+// An iteration is two short passes over vectors that stay in L2, so as
+// launches of their own (three per iteration, 598 per optimiser step) they
+// cost a launch each: 145k vertices, 100 iterations, two solves took 2.9 ms.
+// Here one CTA per SM runs every iteration of the solve, with two sums over
+// the grid per iteration, and stops when all three columns have converged:
+// 2925 -> 868 us for the optimiser step of 72.6k vertices (100 iterations at
+// most, 60 to 100 taken), 12.3 -> 6.3 us per iteration for 2k to 72k vertices
+// and 30.0 -> 20.8 us for 540k.  Up to 78k vertices (one per thread) an
+// iteration is bound by its two grid sums, above that by the L2 traffic of the
+// neighbours' records.
+//
+// A grid sum doubles as the barrier: each CTA publishes its three partial
+// sums and the sum's number as one 16-byte word; CTA 0 polls those words,
+// adds them up and publishes the result, which the others poll (in one of
+// eight copies).  Two trips through L2, without atomics, and the sum has a
+// fixed order, so a solve gives the same bits on every run.  (Every CTA
+// reading every word is one trip, but 142 CTAs polling one another's words
+// took 5.0 us per sum against 3.0.)  A word is free again when its next value
+// is due: a CTA publishes sum n + 1 only after it has read the result of n, for
+// which CTA 0 had read every word.
+constexpr int kCgThreads = 512;
+constexpr int kCgMaxBlocks = 512;
+constexpr int kCgCopies = 8;          // of the result, a 128-byte line each
+constexpr int kCgWords = kCgMaxBlocks + 8 * kCgCopies;
+constexpr int kCgSpins = 1 << 21;     // polls before a wait is given up (about a second)
+constexpr int kCgListWords = 200 * 1024 / 4;  // shared memory for neighbour lists
+
+struct GridSum {
+  ulonglong2* word;  // [kCgMaxBlocks], then the copies of the result; cleared before the launch
+  uint32_t n;        // number of the last sum
+  bool failed;       // a wait ran out: the launch was not co-resident
+};
+
+template <bool kOrder>
+__device__ __forceinline__ void st_word(ulonglong2* p, float3 v, uint32_t n) {
+  const unsigned long long lo = (unsigned long long)__float_as_uint(v.x) | ((unsigned long long)__float_as_uint(v.y) << 32);
+  const unsigned long long hi = (unsigned long long)__float_as_uint(v.z) | ((unsigned long long)n << 32);
+  if (kOrder)
+    asm volatile("{ .reg .b128 w; mov.b128 w, {%1, %2}; st.release.gpu.global.b128 [%0], w; }" ::"l"(p), "l"(lo), "l"(hi) : "memory");
+  else
+    asm volatile("{ .reg .b128 w; mov.b128 w, {%1, %2}; st.relaxed.gpu.global.b128 [%0], w; }" ::"l"(p), "l"(lo), "l"(hi) : "memory");
+}
+template <bool kOrder>
+__device__ __forceinline__ uint32_t ld_word(const ulonglong2* p, float3& v) {
+  unsigned long long lo, hi;
+  if (kOrder)
+    asm volatile("{ .reg .b128 w; ld.acquire.gpu.global.b128 w, [%2]; mov.b128 {%0, %1}, w; }" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+  else
+    asm volatile("{ .reg .b128 w; ld.relaxed.gpu.global.b128 w, [%2]; mov.b128 {%0, %1}, w; }" : "=l"(lo), "=l"(hi) : "l"(p) : "memory");
+  v = mk(__uint_as_float((uint32_t)lo), __uint_as_float((uint32_t)(lo >> 32)), __uint_as_float((uint32_t)hi));
+  return (uint32_t)(hi >> 32);
+}
+
+// Polls *p until it holds value n; false when it gave up.
+template <bool kOrder>
+__device__ __forceinline__ bool wait_word(const ulonglong2* p, float3& v, uint32_t n) {
+  int spins = 0;
+  while (ld_word<kOrder>(p, v) != n)
+    if (++spins >= kCgSpins) return false;
+  return true;
+}
+
+// The grid's sum of v.  kOrder: what any thread wrote before it, every thread
+// can read after it (release and acquire of the words, with the CTA's own
+// barriers on both sides).  Without it only the sum passes, which saves the
+// wait for the CTA's stores; every CTA's reads before it are done all the
+// same, since its part of the sum is made of them.
+template <bool kOrder>
+__device__ __forceinline__ float3 grid_sum3(GridSum& g, float3 v, float (*part)[32]) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   v = mk(warp_sum(v.x), warp_sum(v.y), warp_sum(v.z));
   if (lane == 0) {
     part[0][wid] = v.x;
     part[1][wid] = v.y;
     part[2][wid] = v.z;
   }
+  ++g.n;
   __syncthreads();
+  bool ok = true;
   if (wid == 0) {
-    float3 t = lane < nw ? mk(part[0][lane], part[1][lane], part[2][lane]) : mk(0.f, 0.f, 0.f);
-    t = mk(warp_sum(t.x), warp_sum(t.y), warp_sum(t.z));
-    if (lane == 0) {
-      atomicAdd(dst, t.x);
-      atomicAdd(dst + 1, t.y);
-      atomicAdd(dst + 2, t.z);
+    const bool in = lane < kCgThreads / 32;
+    v = mk(warp_sum(in ? part[0][lane] : 0.f), warp_sum(in ? part[1][lane] : 0.f), warp_sum(in ? part[2][lane] : 0.f));
+    if (lane == 0 && blockIdx.x > 0) {
+      st_word<kOrder>(g.word + blockIdx.x, v, g.n);
+      ok = wait_word<kOrder>(g.word + kCgMaxBlocks + 8 * (blockIdx.x % kCgCopies), v, g.n);
     }
   }
+  if (blockIdx.x == 0 && wid * 32 < (int)gridDim.x) {  // the words of the other CTAs, 32 per warp, and its own sum
+    float3 w = mk(0.f, 0.f, 0.f);
+    if (threadIdx.x == 0) w = v;
+    else if (threadIdx.x < gridDim.x) ok = wait_word<kOrder>(g.word + threadIdx.x, w, g.n);
+    v = mk(warp_sum(w.x), warp_sum(w.y), warp_sum(w.z));
+  }
+  if (lane == 0) {
+    part[3][wid] = v.x;
+    part[4][wid] = v.y;
+    part[5][wid] = v.z;
+  }
+  if (__syncthreads_or(!ok)) g.failed = true;
+  v = mk(part[3][0], part[4][0], part[5][0]);
+  if (blockIdx.x == 0) {
+    for (int i = 1; i * 32 < (int)gridDim.x; ++i) v = v + mk(part[3][i], part[4][i], part[5][i]);
+    if (threadIdx.x < kCgCopies && gridDim.x > 1 && !g.failed) {
+      st_word<kOrder>(g.word + kCgMaxBlocks + 8 * threadIdx.x, v, g.n);
+    }
+  }
+  return v;
 }
 
-// CG scratch: r, z, p, Ap as [nv][3], then scalars rz[iters + 1][3] and
-// pAp[iters][3]
-struct CgView {
-  float *r, *z, *p, *ap, *rz, *pap;
+// CG scratch: the vertices' records (z, p) of 32 bytes, so that what an
+// iteration reads of a neighbour is one load of one sector, r and Ap as
+// [nv][3], and the grid sums' words.
+struct CgRecord {
+  float3 z, p;
 };
+struct CgView {
+  float4* rec;  // [2 nv]: (z.xyz, p.x), (p.yz, 0, 0)
+  float *r, *ap;
+  ulonglong2* word;
+};
+__device__ __forceinline__ CgRecord ld_record(const float4* rec, int v) {  // not .nc: rewritten by the kernel itself
+  float u0, u1;
+  CgRecord c;
+  asm volatile("ld.global.v8.f32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(c.z.x), "=f"(c.z.y), "=f"(c.z.z), "=f"(c.p.x), "=f"(c.p.y), "=f"(c.p.z), "=f"(u0), "=f"(u1)
+               : "l"(rec + 2 * (size_t)v)
+               : "memory");
+  return c;
+}
+__device__ __forceinline__ void st_record(float4* rec, int v, float3 z, float3 p) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%7};" ::"l"(rec + 2 * (size_t)v), "f"(z.x), "f"(z.y), "f"(z.z),
+               "f"(p.x), "f"(p.y), "f"(p.z), "f"(0.f)
+               : "memory");
+}
 
 __device__ __forceinline__ float safe_div(float a, float b) { return b != 0.0f ? a / b : 0.0f; }
 
@@ -220,104 +326,167 @@ __device__ __forceinline__ float safe_div(float a, float b) { return b != 0.0f ?
 // iterations change nothing (FP32 conjugate gradients run on in the
 // rounding noise would drift).
 constexpr float kCgTol2 = 1e-12f;
-__device__ __forceinline__ bool cg_live(const float* rz, int it, int c) {
-  return rz[3 * it + c] > kCgTol2 * rz[c];
+__device__ __forceinline__ bool cg_live(float rz, float rz0) { return rz > kCgTol2 * rz0; }
+__device__ __forceinline__ float cg_alpha(float rz, float rz0, float pap) {
+  return cg_live(rz, rz0) && pap > 0.0f ? rz / pap : 0.0f;
 }
-__device__ __forceinline__ float cg_alpha(const CgView& v, int it, int c) {
-  const float pap = v.pap[3 * it + c];
-  return cg_live(v.rz, it, c) && pap > 0.0f ? v.rz[3 * it + c] / pap : 0.0f;
-}
-
-
-static size_t cg_bytes(int32_t nv, int32_t iters) {
-  return 4 * align_up((size_t)nv * 3 * sizeof(float), 256) +
-         align_up(((size_t)iters * 2 + 1) * 3 * sizeof(float), 256);
+__device__ __forceinline__ float cg_beta(float rz, float old, float rz0) {
+  return cg_live(rz, rz0) ? safe_div(rz, old) : 0.0f;
 }
 
-static CgView cg_view(void* base, int32_t nv, int32_t iters) {
+static size_t cg_vec(int32_t nv, int width) { return align_up((size_t)nv * width * sizeof(float), 256); }
+
+static size_t cg_bytes(int32_t nv) {
+  return cg_vec(nv, 8) + 2 * cg_vec(nv, 3) + kCgWords * sizeof(ulonglong2);
+}
+
+static CgView cg_view(void* base, int32_t nv) {
   char* b = (char*)base;
-  const size_t vec = align_up((size_t)nv * 3 * sizeof(float), 256);
+  const size_t v8 = cg_vec(nv, 8), v3 = cg_vec(nv, 3);
   CgView c;
-  c.r = (float*)b;
-  c.z = (float*)(b + vec);
-  c.p = (float*)(b + 2 * vec);
-  c.ap = (float*)(b + 3 * vec);
-  c.rz = (float*)(b + 4 * vec);
-  c.pap = c.rz + 3 * ((size_t)iters + 1);
+  c.rec = (float4*)b;
+  c.r = (float*)(b + v8);
+  c.ap = (float*)(b + v8 + v3);
+  c.word = (ulonglong2*)(b + v8 + 2 * v3);
   return c;
 }
 
-// r = b - M x, z = r / diag, p = z, rz[0] = r . z
-__global__ void k_cg_init(const int32_t* __restrict__ row, const int32_t* __restrict__ col, int32_t nv, float lam,
-                          const float* __restrict__ b, const float* __restrict__ x, CgView c) {
-  float3 acc = mk(0.f, 0.f, 0.f);
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
-    const float3 r = load3(b + 3 * v) - apply_m(row, col, x, lam, v);
-    const float3 z = r * (1.0f / (1.0f + lam * (float)(row[v + 1] - row[v])));
-    store3(c.r + 3 * v, r);
-    store3(c.z + 3 * v, z);
-    store3(c.p + 3 * v, z);
+// M x = b, x holding the start on entry.  CTA i has the vertices [i chunk, (i +
+// 1) chunk), whose neighbour lists it copies to shared memory (where they
+// fit: the fences of the grid sums drop L1, and the lists are read every
+// iteration).  Pass A of an iteration: p = z + beta p_old (of the neighbours
+// too, from their records: their new p is formed again rather than waited
+// for), Ap = M p, sum p . Ap.  Pass B: x += alpha p, r -= alpha Ap, z = r / diag,
+// the record, sum r . z.  kOne: at most one vertex per thread, whose x, r, z, p
+// and Ap stay in registers.
+constexpr int kCgGather = 8;  // neighbours' records in flight per thread
+template <bool kOne>
+__global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int32_t* __restrict__ row, const int32_t* __restrict__ col,
+                                                      int32_t nv, int32_t chunk, int32_t list_room, float lam,
+                                                      const float* __restrict__ b, float* x, CgView c, int iters) {
+  __shared__ float part[6][32];
+  extern __shared__ int32_t lists[];  // [chunk + 1] list starts, then the lists
+  GridSum g{c.word, 0u, false};
+  const int v0 = min(blockIdx.x * chunk, nv), v1 = min(v0 + chunk, nv);
+  const int base = row[v0], len = row[v1] - base;
+  const bool fits = len <= list_room, starts = list_room >= 0;
+  int32_t* nb = lists + chunk + 1;
+  if (starts)
+    for (int v = v0 + threadIdx.x; v <= v1; v += blockDim.x) lists[v - v0] = row[v] - base;
+  if (fits)
+    for (int k = threadIdx.x; k < len; k += blockDim.x) nb[k] = col[base + k];
+  const int32_t* __restrict__ far = col + base;
+  __syncthreads();
+  auto start_of = [&](int v) { return starts ? lists[v - v0] : row[v] - base; };
+  auto inv_diag = [&](int v) { return 1.0f / (1.0f + lam * (float)(start_of(v + 1) - start_of(v))); };
+  // M applied at v to the vector whose entry j is value(read(j)), mine being its own
+  auto apply = [&](int v, float3 mine, auto read, auto value) {
+    const int e0 = start_of(v), e1 = start_of(v + 1);
+    float3 sum = mk(0.f, 0.f, 0.f);
+    for (int k = e0; k < e1; k += kCgGather) {
+      CgRecord rec[kCgGather];
+#pragma unroll
+      for (int q = 0; q < kCgGather; ++q)
+        if (k + q < e1) rec[q] = read(fits ? nb[k + q] : far[k + q]);
+#pragma unroll
+      for (int q = 0; q < kCgGather; ++q)
+        if (k + q < e1) sum = sum + value(rec[q]);
+    }
+    return mine + (mine * (float)(e1 - e0) - sum) * lam;
+  };
+  float3 acc = mk(0.f, 0.f, 0.f), kx, kr, kz, kp, kap;  // kOne: the thread's vertex
+  kx = kr = kz = kp = kap = acc;
+  // r = b - M x, z = r / diag, rz = r . z
+  for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
+    const float3 xv = load3(x + 3 * (size_t)v);
+    const float3 r = load3(b + 3 * (size_t)v) -
+                     apply(v, xv, [&](int j) { return CgRecord{load3(x + 3 * (size_t)j), mk(0.f, 0.f, 0.f)}; },
+                           [](const CgRecord& q) { return q.z; });
+    const float3 z = r * inv_diag(v);
+    if (kOne) {
+      kx = xv;
+      kr = r;
+      kz = z;
+    } else {
+      store3(c.r + 3 * (size_t)v, r);
+    }
+    st_record(c.rec, v, z, mk(0.f, 0.f, 0.f));
     acc = acc + mul(r, z);
   }
-  block_add3(c.rz, acc);
-}
-
-// Ap = M p, pAp[it] = p . Ap
-__global__ void k_cg_ap(const int32_t* __restrict__ row, const int32_t* __restrict__ col, int32_t nv, float lam,
-                        CgView c, int it) {
-  float3 acc = mk(0.f, 0.f, 0.f);
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
-    const float3 ap = apply_m(row, col, c.p, lam, v);
-    store3(c.ap + 3 * v, ap);
-    acc = acc + mul(load3(c.p + 3 * v), ap);
+  const float3 rz0 = grid_sum3<true>(g, acc, part);
+  float3 rz = rz0, beta = mk(0.f, 0.f, 0.f), keep = mk(1.f, 1.f, 1.f);
+  auto next_p = [&](const CgRecord& q) { return mul(keep, q.z) + mul(beta, q.p); };
+  for (int it = 0; it < iters && !g.failed; ++it) {
+    acc = mk(0.f, 0.f, 0.f);
+    for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
+      const float3 p = next_p(kOne ? CgRecord{kz, kp} : ld_record(c.rec, v));
+      const float3 ap = apply(v, p, [&](int j) { return ld_record(c.rec, j); }, next_p);
+      if (kOne) {
+        kp = p;
+        kap = ap;
+      } else {
+        store3(c.ap + 3 * (size_t)v, ap);
+      }
+      acc = acc + mul(p, ap);
+    }
+    const float3 pap = grid_sum3<false>(g, acc, part);  // pass A writes nothing that others read
+    const float3 alpha = mk(cg_alpha(rz.x, rz0.x, pap.x), cg_alpha(rz.y, rz0.y, pap.y), cg_alpha(rz.z, rz0.z, pap.z));
+    acc = mk(0.f, 0.f, 0.f);
+    for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
+      const float3 p = kOne ? kp : next_p(ld_record(c.rec, v));
+      const float3 r = (kOne ? kr : load3(c.r + 3 * (size_t)v)) - mul(alpha, kOne ? kap : load3(c.ap + 3 * (size_t)v));
+      const float3 z = r * inv_diag(v);
+      if (kOne) {
+        kx = kx + mul(alpha, p);
+        kr = r;
+        kz = z;
+      } else {
+        store3(x + 3 * (size_t)v, load3(x + 3 * (size_t)v) + mul(alpha, p));
+        store3(c.r + 3 * (size_t)v, r);
+      }
+      st_record(c.rec, v, z, p);
+      acc = acc + mul(r, z);
+    }
+    const float3 old = rz;
+    rz = grid_sum3<true>(g, acc, part);
+    // a converged column keeps its direction at zero
+    beta = mk(cg_beta(rz.x, old.x, rz0.x), cg_beta(rz.y, old.y, rz0.y), cg_beta(rz.z, old.z, rz0.z));
+    const bool lx = cg_live(rz.x, rz0.x), ly = cg_live(rz.y, rz0.y), lz = cg_live(rz.z, rz0.z);
+    keep = mk(lx ? 1.0f : 0.0f, ly ? 1.0f : 0.0f, lz ? 1.0f : 0.0f);
+    if (!lx && !ly && !lz) break;  // every later iteration would change nothing
   }
-  block_add3(c.pap + 3 * it, acc);
-}
-
-// alpha = rz[it] / pAp[it]; x += alpha p; r -= alpha Ap; z = r / diag;
-// rz[it + 1] = r . z
-__global__ void k_cg_step(const int32_t* __restrict__ row, int32_t nv, float lam, float* __restrict__ x, CgView c,
-                          int it) {
-  const float3 alpha = mk(cg_alpha(c, it, 0), cg_alpha(c, it, 1), cg_alpha(c, it, 2));
-  float3 acc = mk(0.f, 0.f, 0.f);
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x) {
-    store3(x + 3 * v, load3(x + 3 * v) + mul(alpha, load3(c.p + 3 * v)));
-    const float3 r = load3(c.r + 3 * v) - mul(alpha, load3(c.ap + 3 * v));
-    const float3 z = r * (1.0f / (1.0f + lam * (float)(row[v + 1] - row[v])));
-    store3(c.r + 3 * v, r);
-    store3(c.z + 3 * v, z);
-    acc = acc + mul(r, z);
+  for (int v = v0 + threadIdx.x; v < v1; v += blockDim.x) {
+    if (g.failed) store3(x + 3 * (size_t)v, mk(NAN, NAN, NAN));  // never in a co-resident launch; not to pass for a solution
+    else if (kOne) store3(x + 3 * (size_t)v, kx);
   }
-  block_add3(c.rz + 3 * (it + 1), acc);
 }
 
-// beta = rz[it + 1] / rz[it]; p = z + beta p
-__global__ void k_cg_dir(int32_t nv, CgView c, int it) {
-  // a converged column keeps its direction at zero
-  const float3 beta = mk(cg_live(c.rz, it + 1, 0) ? safe_div(c.rz[3 * (it + 1)], c.rz[3 * it]) : 0.0f,
-                         cg_live(c.rz, it + 1, 1) ? safe_div(c.rz[3 * (it + 1) + 1], c.rz[3 * it + 1]) : 0.0f,
-                         cg_live(c.rz, it + 1, 2) ? safe_div(c.rz[3 * (it + 1) + 2], c.rz[3 * it + 2]) : 0.0f);
-  const float3 keep = mk(cg_live(c.rz, it + 1, 0) ? 1.0f : 0.0f, cg_live(c.rz, it + 1, 1) ? 1.0f : 0.0f,
-                         cg_live(c.rz, it + 1, 2) ? 1.0f : 0.0f);
-  for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < nv; v += gridDim.x * blockDim.x)
-    store3(c.p + 3 * v, mul(keep, load3(c.z + 3 * v)) + mul(beta, load3(c.p + 3 * v)));
-}
-
-// M x = b, x holding the start on entry
 static void launch_cg(const TopoView& T, int32_t nv, float lam, const float* b, float* x, int iters, void* scratch,
                       cudaStream_t s) {
-  CgView c = cg_view(scratch, nv, iters);
-  cudaMemsetAsync(c.rz, 0, ((size_t)iters * 2 + 1) * 3 * sizeof(float), s);
-  const int g = blocks_for(nv, 256);
-  k_cg_init<<<g, 256, 0, s>>>(T.row, T.col, nv, lam, b, x, c);
-  for (int it = 0; it < iters; ++it) {
-    k_cg_ap<<<g, 256, 0, s>>>(T.row, T.col, nv, lam, c, it);
-    k_cg_step<<<g, 256, 0, s>>>(T.row, nv, lam, x, c, it);
-    if (it + 1 < iters) k_cg_dir<<<g, 256, 0, s>>>(nv, c, it);
-  }
+  CgView c = cg_view(scratch, nv);
+  cudaMemsetAsync(c.word, 0, kCgWords * sizeof(ulonglong2), s);
+  int blocks = (nv + kCgThreads - 1) / kCgThreads;
+  const int most = num_sms() < kCgMaxBlocks ? num_sms() : kCgMaxBlocks;
+  if (blocks > most) blocks = most;
+  int32_t chunk = (nv + blocks - 1) / blocks;
+  // list starts and room for lists of eight neighbours a vertex (a closed mesh
+  // has six on average), as far as they fit; the starts alone exceed shared
+  // memory past 7.7M vertices, and are then read where they are (room -1)
+  int64_t words = (int64_t)chunk * 9 + 1;
+  if (words > kCgListWords) words = kCgListWords;
+  int32_t room = words > chunk ? (int32_t)(words - (chunk + 1)) : -1;
+  if (room < 0) words = 0;
+  const int32_t *row = T.row, *col = T.col;
+  void* args[] = {&row, &col, &nv, &chunk, &room, &lam, &b, &x, &c, &iters};
+  const void* f = chunk <= kCgThreads ? (const void*)k_cg<true> : (const void*)k_cg<false>;
+  cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(words * sizeof(int32_t)));
+  cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(kCgThreads), args, (size_t)words * sizeof(int32_t), s);
 }
 
-size_t smooth_scratch_bytes(int32_t nv, int32_t iters) { return cg_bytes(nv, iters); }
+size_t smooth_scratch_bytes(int32_t nv, int32_t iters) {
+  (void)iters;
+  return cg_bytes(nv);
+}
 
 void launch_smooth_solve(const void* topo, int32_t nv, int32_t nf, float lam, const float* b, float* x, int iters,
                          void* scratch, cudaStream_t s) {
@@ -343,7 +512,8 @@ static size_t adam_state_bytes(int32_t nv) {
 }
 size_t large_steps_state_bytes(int32_t nv) { return adam_state_bytes(nv); }
 size_t large_steps_scratch_bytes(int32_t nv, int32_t iters) {
-  return 2 * align_up((size_t)nv * 3 * sizeof(float), 256) + cg_bytes(nv, iters);
+  (void)iters;
+  return 2 * align_up((size_t)nv * 3 * sizeof(float), 256) + cg_bytes(nv);
 }
 
 __global__ void k_apply_m(const int32_t* __restrict__ row, const int32_t* __restrict__ col, int32_t nv, float lam,

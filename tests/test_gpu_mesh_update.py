@@ -92,3 +92,45 @@ def test_edge_loss_matches_oracle():
     assert float(loss) == pytest.approx(ref_loss, rel=1e-4)
     got = dV.cpu().numpy().astype(np.float64)
     assert np.linalg.norm(got - ref_dV) <= 1e-4 * np.linalg.norm(ref_dV)
+
+
+@pytest.mark.parametrize("n,per", [(3, 1), (32, 1), (511, 1), (512, 2), (513, 3), (5000, 4), (5000, 1), (90000, 3)])
+def test_smooth_solve_sizes_and_long_lists(n, per):
+    """Vertex counts about a block's, several blocks, more than one vertex per
+    thread, and lists longer than a block's room for them (per random
+    triangles at every vertex): the solution's residual in FP64."""
+    rng = np.random.default_rng(n + per)
+    i = np.arange(n * per, dtype=np.int64) % n
+    F = np.stack([i, (i + 1) % n, rng.integers(0, n, n * per)], 1).astype(np.int32)
+    b = np.random.default_rng(n).normal(size=(n, 3)).astype(np.float32)
+    topo = dt.Topology(torch.from_numpy(F).cuda(), n)
+    x = dt.smooth_solve(topo, 4.0, torch.from_numpy(b).cuda(), iters=400)
+    _, _, row, col = topo.info()
+    row, col = row.cpu().numpy().astype(np.int64), col.cpu().numpy().astype(np.int64)
+    xd = x.cpu().numpy().astype(np.float64)
+    src = np.repeat(np.arange(n), np.diff(row))
+    Lx = np.diff(row)[:, None] * xd
+    np.subtract.at(Lx, src, xd[col])
+    r = (xd + 4.0 * Lx - b) / np.sqrt(1.0 + 4.0 * np.diff(row))[:, None]  # preconditioned residual
+    r0 = b / np.sqrt(1.0 + 4.0 * np.diff(row))[:, None]
+    # stopped at 1e-6, plus the rounding of M x in FP32 (its terms are up to 2 lambda deg |x|)
+    tol = 1e-6 * np.linalg.norm(r0) + 4 * 2.0 ** -24 * np.linalg.norm(
+        (1.0 + 8.0 * np.diff(row))[:, None] * xd / np.sqrt(1.0 + 4.0 * np.diff(row))[:, None]) * 8
+    assert np.linalg.norm(r) <= tol
+
+
+def test_large_steps_update_in_a_graph():
+    V, F = S.icosphere(4)
+    Ft, g = torch.from_numpy(F).cuda(), torch.from_numpy(np.random.default_rng(5).normal(size=V.shape).astype(np.float32)).cuda()
+    Va, Vb = torch.from_numpy(V.copy()).cuda(), torch.from_numpy(V.copy()).cuda()
+    opt_a, opt_b = dt.LargeStepsOptimizer(Va, Ft), dt.LargeStepsOptimizer(Vb, Ft)
+    graph = torch.cuda.CUDAGraph()
+    torch.cuda.synchronize()
+    with torch.cuda.graph(graph):
+        opt_a.step(g)
+    for _ in range(2):
+        graph.replay()
+        opt_b.step(g)
+    torch.cuda.synchronize()
+    assert torch.equal(Va, Vb)
+    assert (Va - torch.from_numpy(V).cuda()).abs().max() > 1e-4
