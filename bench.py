@@ -286,32 +286,16 @@ def run_reference(args):
 # kernels launched per profiled scope (a scope may hold more than one kernel)
 KERNELS_PER_SCOPE = {"k_vertex_normals": 2, "k_refit": 3, "k_camera": 1, "k_trace": 1,
                      "k_shade": 1, "k_order": 2, "order_clear": 0,
-                     "k_l2_loss_grad": 1, "k_adjoint": 1, "k_face_normals_backward": 1, "lbvh_build": 21,
+                     "k_l2_loss_grad": 1, "k_adjoint": 1, "k_face_normals_backward": 1, "lbvh_build": 27,
                      "k_write_table": 1, "k_zero_grads": 1}
-
-
-def sah_levels(nf: int) -> int:
-    """Large-task levels the binned-SAH builder launches for nf triangles:
-    tasks above 128 triangles are split level by level, with 24 levels of
-    free splits plus the median levels below them, at most 64."""
-    if nf <= 128:
-        return 0
-    lg = 0
-    while (128 << lg) < nf:
-        lg += 1
-    return min(24 + lg + 2, 64)
 
 
 def scope_kernels(scope: str, nf: int) -> int:
     """Kernels launched per entry of a profiled scope; the SAH build's scopes
-    nest (sah_build holds sah_large_levels and sah_small), so each counts only
-    its own launches."""
-    if scope == "sah_build":
-        return 10  # header, bounds x2, primitives, root, 4-wide topology x4, validation
-    if scope == "sah_large_levels":
-        return 4 * sah_levels(nf)
-    if scope == "sah_small":
-        return 1
+    nest (sah_build holds sah_large_levels and sah_small, one kernel each), so
+    each counts only its own launches."""
+    if scope == "sah_build":  # header, primitives, 4-wide topology x3, validation; a scan of one or two
+        return 7 if nf <= 2049 else 8
     return KERNELS_PER_SCOPE.get(scope, 1)
 
 

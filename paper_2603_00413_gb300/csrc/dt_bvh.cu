@@ -90,12 +90,6 @@ __device__ __forceinline__ float ord2f(uint32_t o) {
   return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
 }
 
-// scratch: bounds of the centroids as ordered uints [lo xyz, hi xyz]
-__global__ void k_init_bounds(uint32_t* b) {
-  if (threadIdx.x < 3) b[threadIdx.x] = 0xffffffffu;
-  else if (threadIdx.x < 6) b[threadIdx.x] = 0u;
-}
-
 __device__ __forceinline__ float3 centroid_of(const float* V, const int32_t* F, int f) {
   const float3 v0 = load3(V + 3 * F[3 * f]), v1 = load3(V + 3 * F[3 * f + 1]), v2 = load3(V + 3 * F[3 * f + 2]);
   return (v0 + v1 + v2) * (1.0f / 3.0f);
@@ -167,27 +161,99 @@ __global__ void k_radix_hist(const uint32_t* __restrict__ keys, int32_t n, int s
   hist[threadIdx.x * gridDim.x + blockIdx.x] = cnt[threadIdx.x];
 }
 
-// exclusive scan of m entries in one block of 1024 threads
-__global__ void k_scan_exclusive(uint32_t* __restrict__ a, int32_t m) {
-  __shared__ uint32_t part[1024];
-  const int per = (m + 1023) / 1024;
-  const int lo = threadIdx.x * per;
-  const int hi = min(lo + per, m);
-  uint32_t s = 0;
-  for (int i = lo; i < hi; ++i) s += a[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int o = 1; o < 1024; o <<= 1) {  // Hillis-Steele inclusive scan of the partial sums
-    uint32_t v = threadIdx.x >= o ? part[threadIdx.x - o] : 0u;
-    __syncthreads();
-    part[threadIdx.x] += v;
-    __syncthreads();
+// ---- exclusive scan -----------------------------------------------------------
+// At most kScanBlocks CTAs have a contiguous span each: one launch sums the
+// spans, the second adds up the spans before its own and scans its span tile
+// by tile (eight entries per thread, two 16-byte loads).  An array of one tile
+// needs the second launch only.  A scan of one CTA, each thread walking its
+// own thousandth of the array, took 1.0 ms for 1.08M entries and 103 us for
+// 120k; this takes 8 us for 120k and 18
+// us for 1.08M.
+constexpr int kScanThreads = 256;
+constexpr int kScanItems = 8;
+constexpr int kScanTile = kScanThreads * kScanItems;
+
+// inclusive sum over the CTA's threads before this one (exclusive), and the total
+__device__ __forceinline__ uint32_t cta_exclusive_sum(uint32_t v, uint32_t* s_warp, uint32_t& total) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  uint32_t x = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, x, o);
+    if (lane >= o) x += y;
   }
-  uint32_t run = threadIdx.x ? part[threadIdx.x - 1] : 0u;
-  for (int i = lo; i < hi; ++i) {
-    const uint32_t v = a[i];
-    a[i] = run;
-    run += v;
+  __syncthreads();  // the previous use of s_warp is over
+  if (lane == 31) s_warp[wid] = x;
+  __syncthreads();
+  uint32_t before = 0, all = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    const uint32_t t = s_warp[w];
+    if (w < wid) before += t;
+    all += t;
+  }
+  total = all;
+  return before + x - v;
+}
+
+// entries i .. i + 7 of a[0, m) (zeros past the end); i is a multiple of 8 and a 16-byte aligned
+__device__ __forceinline__ void scan_load(const uint32_t* a, int64_t i, int64_t m, uint32_t (&v)[kScanItems]) {
+  if (i + kScanItems <= m) {
+    const uint4 x = *reinterpret_cast<const uint4*>(a + i), y = *reinterpret_cast<const uint4*>(a + i + 4);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
+    v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+  } else {
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) v[k] = i + k < m ? a[i + k] : 0u;
+  }
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_totals(const uint32_t* __restrict__ a, int64_t m, int64_t span,
+                                                              uint32_t* __restrict__ totals) {
+  __shared__ uint32_t s_warp[kScanThreads / 32];
+  const int64_t lo = blockIdx.x * span, hi = min(lo + span, m);
+  uint32_t sum = 0, total;
+  for (int64_t i = lo + threadIdx.x * kScanItems; i < hi; i += kScanTile) {
+    uint32_t v[kScanItems];
+    scan_load(a, i, hi, v);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) sum += v[k];
+  }
+  cta_exclusive_sum(sum, s_warp, total);
+  if (threadIdx.x == 0) totals[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(kScanThreads) k_scan_apply(const uint32_t* src, uint32_t* dst, int64_t m, int64_t span,
+                                                             const uint32_t* __restrict__ totals) {
+  __shared__ uint32_t s_warp[kScanThreads / 32];
+  const int64_t lo = blockIdx.x * span, hi = min(lo + span, m);
+  uint32_t carry = 0, total;
+  if (gridDim.x > 1) {
+    uint32_t sum = 0;
+    for (uint32_t b = threadIdx.x; b < blockIdx.x; b += blockDim.x) sum += totals[b];
+    cta_exclusive_sum(sum, s_warp, carry);
+  }
+  for (int64_t t = lo; t < hi; t += kScanTile) {
+    const int64_t i = t + threadIdx.x * kScanItems;
+    uint32_t v[kScanItems], sum = 0;
+    scan_load(src, i, hi, v);
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) {
+      const uint32_t x = v[k];
+      v[k] = sum;
+      sum += x;
+    }
+    const uint32_t base = carry + cta_exclusive_sum(sum, s_warp, total);
+    carry += total;
+#pragma unroll
+    for (int k = 0; k < kScanItems; ++k) v[k] += base;
+    if (i + kScanItems <= hi) {
+      *reinterpret_cast<uint4*>(dst + i) = make_uint4(v[0], v[1], v[2], v[3]);
+      *reinterpret_cast<uint4*>(dst + i + 4) = make_uint4(v[4], v[5], v[6], v[7]);
+    } else {
+#pragma unroll
+      for (int k = 0; k < kScanItems; ++k)
+        if (i + k < hi) dst[i + k] = v[k];
+    }
   }
 }
 
@@ -353,11 +419,17 @@ __global__ void k_refit(const float* __restrict__ V, const int32_t* __restrict__
 // surface area cost area(left box) * left count + area(right box) * right
 // count, and the range
 // is partitioned stably into [left | right].  Tasks larger than kSahSmall
-// take four launches per tree level, each spread over chunks of kSahChunk
-// positions so that the few huge tasks near the root use the whole GPU: bin
-// (per-chunk shared-memory bins added into the task's bins), split (one warp
-// per task), count (left primitives per chunk) and scatter (stable, each
-// chunk at the offset of the chunks before it).  Smaller tasks are built
+// are split level by level in one cooperative launch (k_sah_levels), in
+// chunks of kSahChunk positions so that the few huge tasks near the root use
+// the whole GPU: each chunk's bins are summed in shared memory and added to its
+// task's, and the CTA that adds the last chunk of a task chooses the split;
+// after a barrier of the grid each chunk is scattered, stably, past the left
+// counts of the task's chunks before it (from their own bin counts).  A task
+// of one chunk is binned, split and scattered by its CTA at once.  (As four
+// launches per level, and as many levels as a tree could have, the host not
+// knowing how many there are, this took 1.18 ms for 120k triangles and 0.67
+// ms for 5k, most of it launches; now 212
+// and 89 us.)  Smaller tasks are built
 // down to their leaves by one warp each, in shared memory.  An internal node
 // is numbered by its split position s (the last position of its left child),
 // which is unique in [0, nf - 2]; the root's number is swapped with 0 so the
@@ -373,14 +445,15 @@ constexpr int kSahSmall = 128;
 constexpr int kSahFreeDepth = 24;
 constexpr int kSahSmallFreeDepth = 56;
 constexpr int kSahMaxLevels = 64;
-constexpr int kSahChunk = 4096;
+constexpr int kSahChunk = 1024;
 constexpr int kSahThreads = 256;
+constexpr int kSahBlocksPerSm = 3;  // resident CTAs of the level kernel
 constexpr int kSahSmallWarps = 4;
 
 struct SahTask {
   int a, n, parent, sd;       // range, parent node, side | depth << 1
   int chunk0, axis, bin, nl;  // first chunk of the level; the split (axis < 0: median)
-  float4 lo, hi;              // binning bounds (xyz), a superset of the centroids
+  float4 lo, hi;              // binning bounds (xyz), a superset of the centroids; lo.w: bits of the chunks binned
 };
 template <int kB>
 struct SahBinsT {  // order-preserving uints for the float bounds
@@ -394,6 +467,7 @@ struct SahState {
   unsigned long long packed[kSahMaxLevels + 2];  // per level: tasks << 32 | chunks
   int n_small;
   int sroot;
+  uint32_t barrier[kBarrierWords];
 };
 struct SahView {
   float4* cen;
@@ -401,7 +475,8 @@ struct SahView {
   uint32_t* idx[2];
   SahTask* tasks[2];
   SahBins* bins[2];
-  uint32_t* chunk_left;
+  int* chunk_task[2];   // [max_chunks]: the task of each chunk of a level
+  uint32_t* chunk_cnt;  // [max_chunks][3][kSahBins]: bin counts of a chunk of a task of several
   int4* small;  // (a, n, parent, side | depth << 1 | buffer << 30)
   SahState* st;
   int max_large, max_small, max_chunks;
@@ -428,15 +503,22 @@ __device__ __forceinline__ void sah_set_child(BvhView& B, int node, int side, in
 __device__ __forceinline__ float comp(const float4& v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : v.z); }
 __device__ __forceinline__ float comp3(const float3& v, int k) { return k == 0 ? v.x : (k == 1 ? v.y : v.z); }
 
-// primitive boxes and centroids, the identity permutation, bin_child cleared
-// to kNoChild and internal parents to -1 (validation catches any link a build
-// leaves unset, and the depth walks stop at an unset parent)
-__global__ void k_sah_prims(const float* __restrict__ V, const int32_t* __restrict__ F, int32_t nf, SahView S,
-                            BvhView B) {
+// Primitive boxes and centroids, the bounds of the centroids, the identity
+// permutation, bin_child cleared to kNoChild and internal parents to -1
+// (validation catches any link a build leaves unset, and the depth walks stop
+// at an unset parent).
+__global__ void __launch_bounds__(256) k_sah_prims(const float* __restrict__ V, const int32_t* __restrict__ F, int32_t nf,
+                                                   uint32_t* __restrict__ bounds, SahView S, BvhView B) {
+  __shared__ uint32_t s_b[6];
+  if (threadIdx.x < 6) s_b[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
+  __syncthreads();
   const int n_int = nf - 1;
+  float3 lo = mk(INFINITY, INFINITY, INFINITY), hi = mk(-INFINITY, -INFINITY, -INFINITY);
   for (int f = blockIdx.x * blockDim.x + threadIdx.x; f < nf; f += gridDim.x * blockDim.x) {
     const float3 v0 = load3(V + 3 * F[3 * f]), v1 = load3(V + 3 * F[3 * f + 1]), v2 = load3(V + 3 * F[3 * f + 2]);
     const float3 c = (v0 + v1 + v2) * (1.0f / 3.0f);
+    lo = mk(fminf(lo.x, c.x), fminf(lo.y, c.y), fminf(lo.z, c.z));
+    hi = mk(fmaxf(hi.x, c.x), fmaxf(hi.y, c.y), fmaxf(hi.z, c.z));
     S.cen[f] = make_float4(c.x, c.y, c.z, 0.f);
     S.pbox[2 * f] =
         make_float4(fminf(v0.x, fminf(v1.x, v2.x)), fminf(v0.y, fminf(v1.y, v2.y)), fminf(v0.z, fminf(v1.z, v2.z)), 0.f);
@@ -448,6 +530,19 @@ __global__ void k_sah_prims(const float* __restrict__ V, const int32_t* __restri
       B.parent[f] = -1;
     }
   }
+  const uint32_t m[6] = {__reduce_min_sync(kFull, f2ord(lo.x)), __reduce_min_sync(kFull, f2ord(lo.y)),
+                         __reduce_min_sync(kFull, f2ord(lo.z)), __reduce_max_sync(kFull, f2ord(hi.x)),
+                         __reduce_max_sync(kFull, f2ord(hi.y)), __reduce_max_sync(kFull, f2ord(hi.z))};
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      atomicMin(&s_b[k], m[k]);
+      atomicMax(&s_b[3 + k], m[3 + k]);
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) atomicMin(bounds + threadIdx.x, s_b[threadIdx.x]);
+  else if (threadIdx.x < 6) atomicMax(bounds + threadIdx.x, s_b[threadIdx.x]);
 }
 
 __device__ __forceinline__ int sah_chunks(int n) { return (n + kSahChunk - 1) / kSahChunk; }
@@ -468,13 +563,14 @@ __device__ __forceinline__ void sah_zero_bins(SahBinsT<kB>* g, int i0, int strid
 }
 
 // the root task: large (level 0) or, for at most kSahSmall triangles, small
-__global__ void k_sah_root(int32_t nf, const uint32_t* __restrict__ bounds, SahView S) {
-  for (int i = threadIdx.x; i < kSahMaxLevels + 2; i += blockDim.x) S.st->packed[i] = 0ull;
-  if (nf > kSahSmall) sah_zero_bins(&S.bins[0][0], threadIdx.x, blockDim.x);
-  __syncthreads();
+// (one CTA; the state starts out zero)
+__device__ void sah_root(int32_t nf, const uint32_t* bounds, const SahView& S) {
+  if (nf > kSahSmall) {
+    sah_zero_bins(&S.bins[0][0], threadIdx.x, blockDim.x);
+    for (int c = threadIdx.x; c < sah_chunks(nf); c += blockDim.x) S.chunk_task[0][c] = 0;
+  }
   if (threadIdx.x == 0) {
     S.st->sroot = -1;
-    S.st->n_small = 0;
     if (nf > kSahSmall) {
       SahTask t;
       t.a = 0; t.n = nf; t.parent = -1; t.sd = 0;
@@ -497,69 +593,8 @@ __device__ __forceinline__ void sah_flush(SahBinsT<kB>& sb, int k, int b, uint32
   atomicMax(&sb.hi[k][b][0], f2ord(hi.x)); atomicMax(&sb.hi[k][b][1], f2ord(hi.y)); atomicMax(&sb.hi[k][b][2], f2ord(hi.z));
 }
 
-// best split of one axis from its bins: boundary i puts bins 0..i left
-struct SahSplit {
-  float cost;
-  int axis, bin, nl;
-  float3 llo, lhi, rlo, rhi;
-};
-template <int kB>
-__device__ SahSplit sah_sweep(const SahBinsT<kB>& sb, int k) {
-  SahSplit best;
-  best.cost = INFINITY; best.axis = k; best.bin = -1; best.nl = 0;
-  float rarea[kB];
-  uint32_t rcnt[kB];
-  float3 rl = mk(INFINITY, INFINITY, INFINITY), rh = mk(-INFINITY, -INFINITY, -INFINITY);
-  uint32_t c = 0;
-  for (int i = kB - 1; i >= 1; --i) {
-    if (sb.cnt[k][i]) {
-      rl = mk(fminf(rl.x, ord2f(sb.lo[k][i][0])), fminf(rl.y, ord2f(sb.lo[k][i][1])), fminf(rl.z, ord2f(sb.lo[k][i][2])));
-      rh = mk(fmaxf(rh.x, ord2f(sb.hi[k][i][0])), fmaxf(rh.y, ord2f(sb.hi[k][i][1])), fmaxf(rh.z, ord2f(sb.hi[k][i][2])));
-    }
-    c += sb.cnt[k][i];
-    rcnt[i] = c;
-    rarea[i] = c ? sah_area(rl, rh) : 0.f;
-  }
-  float3 ll = mk(INFINITY, INFINITY, INFINITY), lh = mk(-INFINITY, -INFINITY, -INFINITY);
-  uint32_t lc = 0;
-  for (int i = 0; i < kB - 1; ++i) {
-    if (sb.cnt[k][i]) {
-      ll = mk(fminf(ll.x, ord2f(sb.lo[k][i][0])), fminf(ll.y, ord2f(sb.lo[k][i][1])), fminf(ll.z, ord2f(sb.lo[k][i][2])));
-      lh = mk(fmaxf(lh.x, ord2f(sb.hi[k][i][0])), fmaxf(lh.y, ord2f(sb.hi[k][i][1])), fmaxf(lh.z, ord2f(sb.hi[k][i][2])));
-    }
-    lc += sb.cnt[k][i];
-    const uint32_t rc = rcnt[i + 1];
-    if (lc == 0 || rc == 0) continue;
-    const float cost = sah_area(ll, lh) * (float)lc + rarea[i + 1] * (float)rc;
-    if (cost < best.cost) {
-      best.cost = cost; best.bin = i; best.nl = (int)lc;
-      best.llo = ll; best.lhi = lh;
-    }
-  }
-  if (best.bin >= 0) {  // the right box of the chosen boundary
-    float3 a = mk(INFINITY, INFINITY, INFINITY), b = mk(-INFINITY, -INFINITY, -INFINITY);
-    for (int i = best.bin + 1; i < kB; ++i)
-      if (sb.cnt[k][i]) {
-        a = mk(fminf(a.x, ord2f(sb.lo[k][i][0])), fminf(a.y, ord2f(sb.lo[k][i][1])), fminf(a.z, ord2f(sb.lo[k][i][2])));
-        b = mk(fmaxf(b.x, ord2f(sb.hi[k][i][0])), fmaxf(b.y, ord2f(sb.hi[k][i][1])), fmaxf(b.z, ord2f(sb.hi[k][i][2])));
-      }
-    best.rlo = a; best.rhi = b;
-  }
-  return best;
-}
-
-// the task that owns chunk c (tasks are in chunk order: slot and chunks come
-// from one 64-bit atomic)
-__device__ __forceinline__ int sah_find_task(const SahTask* tasks, int ntask, int c) {
-  int lo = 0, hi = ntask - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (tasks[mid].chunk0 <= c) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
+// Everything below is read after another CTA of the same launch wrote it, so
+// the loads are plain ones (never the read-only path).
 struct SahLevel {
   int ntask, nchunk;
 };
@@ -578,374 +613,585 @@ __device__ __forceinline__ bool sah_free(const SahTask& T, float sc[3]) {
   return (T.sd >> 1) < kSahFreeDepth && (sc[0] > 0.f || sc[1] > 0.f || sc[2] > 0.f);
 }
 
-__device__ __forceinline__ bool sah_goes_left(const SahView& S, const SahTask& T, const float sc[3], uint32_t p, int i) {
-  if (T.axis < 0) return i < T.nl;
-  const float4 c = S.cen[p];
-  return sah_bin(comp(c, T.axis), comp(T.lo, T.axis), sc[T.axis]) <= T.bin;
-}
+// A task's split, and what its children need.
+struct SahChoice {
+  int axis, bin, nl;
+  float3 llo, lhi, rlo, rhi;
+};
 
-// 1/4 of a level: the bins of every task, chunk by chunk
-__global__ void __launch_bounds__(kSahThreads) k_sah_bin(int level, SahView S) {
-  __shared__ SahBins sb;
-  const SahLevel L = sah_level(S, level);
-  const SahTask* tasks = S.tasks[level & 1];
-  const uint32_t* __restrict__ in = S.idx[level & 1];
-  const int tid = threadIdx.x;
-  for (int c = blockIdx.x; c < L.nchunk; c += gridDim.x) {
-    const int t = sah_find_task(tasks, L.ntask, c);
-    const SahTask T = tasks[t];
-    float sc[3];
-    if (!sah_free(T, sc)) continue;  // uniform over the block
-    sah_zero_bins(&sb, tid, blockDim.x);
-    __syncthreads();
-    const int q0 = T.a + (c - T.chunk0) * kSahChunk, q1 = min(T.a + T.n, q0 + kSahChunk);
-    // each thread bins a contiguous run, adding runs of equal bins at once
-    const int run = (q1 - q0 + blockDim.x - 1) / blockDim.x;
-    const int p0 = q0 + tid * run, p1 = min(q1, p0 + run);
-    int cb[3] = {-1, -1, -1};
-    uint32_t cn[3] = {0u, 0u, 0u};
-    float3 clo[3], chi[3];
-    for (int pos = p0; pos < p1; ++pos) {
-      const uint32_t p = in[pos];
-      const float4 c4 = S.cen[p], lo = S.pbox[2 * p], hi = S.pbox[2 * p + 1];
+// The split of a task from its bins in shared memory, by the whole CTA: warp k
+// has axis k and lane i bin i.  Boundary i puts bins 0..i left; the boxes
+// and counts left of every boundary are an inclusive scan over the lanes, those
+// right of it one from the other end.  The least cost wins, ties to the
+// lower boundary and then to the lower axis.
+__device__ __forceinline__ void sah_choose(const SahBins& sb, const SahTask& T, const float sc[3], bool free,
+                                           SahChoice* s_axis, float* s_cost, SahChoice& out) {
+  static_assert(kSahBins == 32, "a lane per bin");
+  const int lane = threadIdx.x & 31, k = threadIdx.x >> 5;
+  if (k < 3) {
+    float best = INFINITY;
+    SahChoice c;
+    c.axis = k; c.bin = -1; c.nl = T.n / 2;
+    c.llo = c.rlo = mk(T.lo.x, T.lo.y, T.lo.z);
+    c.lhi = c.rhi = mk(T.hi.x, T.hi.y, T.hi.z);
+    if (free && sc[k] > 0.f) {
+      const uint32_t cnt = sb.cnt[k][lane];
+      float3 ll = mk(INFINITY, INFINITY, INFINITY), lh = mk(-INFINITY, -INFINITY, -INFINITY);
+      if (cnt) {
+        ll = mk(ord2f(sb.lo[k][lane][0]), ord2f(sb.lo[k][lane][1]), ord2f(sb.lo[k][lane][2]));
+        lh = mk(ord2f(sb.hi[k][lane][0]), ord2f(sb.hi[k][lane][1]), ord2f(sb.hi[k][lane][2]));
+      }
+      float3 rl = ll, rh = lh;
+      uint32_t lc = cnt, rc = cnt;
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        if (sc[k] <= 0.f) continue;
-        const int b = sah_bin(comp(c4, k), comp(T.lo, k), sc[k]);
-        if (b != cb[k]) {
-          if (cb[k] >= 0) sah_flush(sb, k, cb[k], cn[k], clo[k], chi[k]);
-          cb[k] = b; cn[k] = 0u;
-          clo[k] = mk(INFINITY, INFINITY, INFINITY);
-          chi[k] = mk(-INFINITY, -INFINITY, -INFINITY);
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t a = __shfl_up_sync(kFull, lc, o), b = __shfl_down_sync(kFull, rc, o);
+        const float3 al = mk(__shfl_up_sync(kFull, ll.x, o), __shfl_up_sync(kFull, ll.y, o), __shfl_up_sync(kFull, ll.z, o));
+        const float3 ah = mk(__shfl_up_sync(kFull, lh.x, o), __shfl_up_sync(kFull, lh.y, o), __shfl_up_sync(kFull, lh.z, o));
+        const float3 bl = mk(__shfl_down_sync(kFull, rl.x, o), __shfl_down_sync(kFull, rl.y, o), __shfl_down_sync(kFull, rl.z, o));
+        const float3 bh = mk(__shfl_down_sync(kFull, rh.x, o), __shfl_down_sync(kFull, rh.y, o), __shfl_down_sync(kFull, rh.z, o));
+        if (lane >= o) {
+          lc += a;
+          ll = mk(fminf(ll.x, al.x), fminf(ll.y, al.y), fminf(ll.z, al.z));
+          lh = mk(fmaxf(lh.x, ah.x), fmaxf(lh.y, ah.y), fmaxf(lh.z, ah.z));
         }
-        ++cn[k];
-        clo[k] = mk(fminf(clo[k].x, lo.x), fminf(clo[k].y, lo.y), fminf(clo[k].z, lo.z));
-        chi[k] = mk(fmaxf(chi[k].x, hi.x), fmaxf(chi[k].y, hi.y), fmaxf(chi[k].z, hi.z));
+        if (lane + o < 32) {
+          rc += b;
+          rl = mk(fminf(rl.x, bl.x), fminf(rl.y, bl.y), fminf(rl.z, bl.z));
+          rh = mk(fmaxf(rh.x, bh.x), fmaxf(rh.y, bh.y), fmaxf(rh.z, bh.z));
+        }
+      }
+      // right of boundary `lane` begins at the next lane
+      rc = __shfl_down_sync(kFull, rc, 1);
+      rl = mk(__shfl_down_sync(kFull, rl.x, 1), __shfl_down_sync(kFull, rl.y, 1), __shfl_down_sync(kFull, rl.z, 1));
+      rh = mk(__shfl_down_sync(kFull, rh.x, 1), __shfl_down_sync(kFull, rh.y, 1), __shfl_down_sync(kFull, rh.z, 1));
+      const bool cut = lane < 31 && lc > 0 && rc > 0;
+      const float cost = cut ? sah_area(ll, lh) * (float)lc + sah_area(rl, rh) * (float)rc : INFINITY;
+      // (costs are not negative: their bits order like the numbers; a NaN never wins)
+      const uint32_t key = cut && cost < INFINITY ? __float_as_uint(cost) : 0x7f800000u;
+      const uint32_t least = __reduce_min_sync(kFull, key);
+      if (least < 0x7f800000u) {
+        const int at = __ffs(__ballot_sync(kFull, key == least)) - 1;
+        best = __uint_as_float(least);
+        c.bin = at;
+        c.nl = (int)__shfl_sync(kFull, lc, at);
+        c.llo = mk(__shfl_sync(kFull, ll.x, at), __shfl_sync(kFull, ll.y, at), __shfl_sync(kFull, ll.z, at));
+        c.lhi = mk(__shfl_sync(kFull, lh.x, at), __shfl_sync(kFull, lh.y, at), __shfl_sync(kFull, lh.z, at));
+        c.rlo = mk(__shfl_sync(kFull, rl.x, at), __shfl_sync(kFull, rl.y, at), __shfl_sync(kFull, rl.z, at));
+        c.rhi = mk(__shfl_sync(kFull, rh.x, at), __shfl_sync(kFull, rh.y, at), __shfl_sync(kFull, rh.z, at));
       }
     }
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      if (cb[k] >= 0) sah_flush(sb, k, cb[k], cn[k], clo[k], chi[k]);
-    __syncthreads();
-    SahBins& G = S.bins[level & 1][t];
-    for (int i = tid; i < 3 * kSahBins; i += blockDim.x) {
-      const int k = i / kSahBins, b = i % kSahBins;
-      if (!sb.cnt[k][b]) continue;
-      atomicAdd(&G.cnt[k][b], sb.cnt[k][b]);
-      for (int q = 0; q < 3; ++q) {
-        atomicMin(&G.lo[k][b][q], sb.lo[k][b][q]);
-        atomicMax(&G.hi[k][b][q], sb.hi[k][b][q]);
-      }
+    if (lane == 0) {
+      s_axis[k] = c;
+      s_cost[k] = best;
     }
-    __syncthreads();
+  }
+  __syncthreads();
+  int k0 = -1;
+  float least = INFINITY;
+  for (int a = 0; a < 3; ++a)
+    if (s_axis[a].bin >= 0 && s_cost[a] < least) {
+      least = s_cost[a];
+      k0 = a;
+    }
+  if (k0 >= 0) {
+    out = s_axis[k0];
+  } else {  // the median
+    out.axis = out.bin = -1;
+    out.nl = T.n / 2;
+    out.llo = out.rlo = mk(T.lo.x, T.lo.y, T.lo.z);
+    out.lhi = out.rhi = mk(T.hi.x, T.hi.y, T.hi.z);
   }
 }
 
-// 2/4: one warp per task chooses the split, numbers the node, links it to
-// its parent and queues the children (large ones for the next level with
-// cleared bins, the rest for the warp builder)
-__global__ void __launch_bounds__(128) k_sah_split(int level, SahView S, BvhView B) {
-  const SahLevel L = sah_level(S, level);
-  SahTask* tasks = S.tasks[level & 1];
-  const int lane = threadIdx.x & 31;
-  const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
-  for (int t = gw; t < L.ntask; t += nw) {
-    SahTask T = tasks[t];
-    const int depth = T.sd >> 1;
-    float sc[3];
-    int axis = -1, bin = -1, nl = T.n / 2;
-    float3 llo = mk(T.lo.x, T.lo.y, T.lo.z), lhi = mk(T.hi.x, T.hi.y, T.hi.z), rlo = llo, rhi = lhi;
-    if (sah_free(T, sc)) {
-      const SahBins& G = S.bins[level & 1][t];
-      SahSplit sp;
-      sp.cost = INFINITY; sp.bin = -1; sp.axis = lane; sp.nl = 0;
-      if (lane < 3 && sc[lane] > 0.f) sp = sah_sweep(G, lane);
-      float bc = INFINITY;
-      for (int k = 0; k < 3; ++k) {
-        const float ck = __shfl_sync(kFull, sp.cost, k);
-        const int bk = __shfl_sync(kFull, sp.bin, k);
-        if (bk >= 0 && ck < bc) { bc = ck; axis = k; }
-      }
-      if (axis >= 0) {
-        bin = __shfl_sync(kFull, sp.bin, axis);
-        nl = __shfl_sync(kFull, sp.nl, axis);
-        llo = mk(__shfl_sync(kFull, sp.llo.x, axis), __shfl_sync(kFull, sp.llo.y, axis), __shfl_sync(kFull, sp.llo.z, axis));
-        lhi = mk(__shfl_sync(kFull, sp.lhi.x, axis), __shfl_sync(kFull, sp.lhi.y, axis), __shfl_sync(kFull, sp.lhi.z, axis));
-        rlo = mk(__shfl_sync(kFull, sp.rlo.x, axis), __shfl_sync(kFull, sp.rlo.y, axis), __shfl_sync(kFull, sp.rlo.z, axis));
-        rhi = mk(__shfl_sync(kFull, sp.rhi.x, axis), __shfl_sync(kFull, sp.rhi.y, axis), __shfl_sync(kFull, sp.rhi.z, axis));
-      }
-    }
-    int child_slot[2] = {-1, -1};
+// Numbers the split's node, links it to its parent and queues the children:
+// large ones for the next level (with cleared bins where several CTAs will add
+// to them), the rest for the small builder.  By the whole CTA, a warp per child
+// (each waits on an atomic).
+__device__ __forceinline__ void sah_emit(int level, const SahTask& T, const SahChoice& c, int sroot, const SahView& S,
+                                         BvhView& B) {
+  const int q = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (q >= 2) return;
+  const int depth = T.sd >> 1;
+  const int s = T.a + c.nl - 1;
+  if (T.parent < 0) sroot = s;
+  const int id = sah_split_id(s, sroot);
+  const int ca = q ? T.a + c.nl : T.a, cn = q ? T.n - c.nl : c.nl, nc = sah_chunks(cn);
+  if (threadIdx.x == 0) {
+    if (T.parent < 0) S.st->sroot = s;
+    B.parent[id] = T.parent;
+    if (T.parent >= 0) sah_set_child(B, T.parent, T.sd & 1, id);
+  }
+  if (cn <= kSahSmall) {  // (one triangle: the small builder writes the leaf)
     if (lane == 0) {
-      tasks[t].axis = axis;
-      tasks[t].bin = bin;
-      tasks[t].nl = nl;
-      const int s = T.a + nl - 1;
-      int sroot;
-      if (T.parent < 0) {
-        sroot = s;
-        S.st->sroot = s;
-      } else {
-        sroot = S.st->sroot;
+      const int slot = atomicAdd(&S.st->n_small, 1);
+      if (slot < S.max_small) S.small[slot] = make_int4(ca, cn, id, q | ((depth + 1) << 1) | (((level + 1) & 1) << 30));
+      else atomicExch(&B.hdr->corrupt, 1);  // more tasks than disjoint ranges: never expected
+    }
+    return;
+  }
+  unsigned long long old = 0;
+  if (lane == 0) old = atomicAdd(&S.st->packed[level + 1], (1ull << 32) | (unsigned long long)nc);
+  old = __shfl_sync(kFull, old, 0);
+  const int slot = (int)(old >> 32), chunk0 = (int)(old & 0xffffffffull);
+  if (slot >= S.max_large || chunk0 + nc > S.max_chunks) {
+    if (lane == 0) atomicExch(&B.hdr->corrupt, 1);
+    return;
+  }
+  if (lane == 0) {
+    SahTask ct;
+    ct.a = ca; ct.n = cn; ct.parent = id; ct.sd = q | ((depth + 1) << 1);
+    ct.chunk0 = chunk0; ct.axis = -1; ct.bin = -1; ct.nl = 0;
+    const float3 lo = q ? c.rlo : c.llo, hi = q ? c.rhi : c.lhi;
+    ct.lo = make_float4(lo.x, lo.y, lo.z, 0.f);
+    ct.hi = make_float4(hi.x, hi.y, hi.z, 0.f);
+    S.tasks[(level + 1) & 1][slot] = ct;
+  }
+  for (int i = lane; i < nc; i += 32) S.chunk_task[(level + 1) & 1][chunk0 + i] = slot;
+  if (nc > 1) sah_zero_bins(&S.bins[(level + 1) & 1][slot], lane, 32);
+}
+
+// A chunk's positions, kSahPer consecutive ones per thread: the primitive
+// and, packed five bits each, its bins along the three axes.
+constexpr int kSahPer = kSahChunk / kSahThreads;
+struct SahItems {
+  uint32_t p[kSahPer], bins[kSahPer];
+};
+
+// Stable scatter of a chunk's items to [left | right] of its task, i0 the
+// chunk's first position in the task and `before` the left ones of the
+// chunks before it.
+__device__ __forceinline__ void sah_scatter(const SahTask& T, const SahItems& it, uint32_t* out, int i0, int before,
+                                            BvhView& B, uint32_t* s_warp) {
+  const int i = i0 + (int)threadIdx.x * kSahPer;
+  const int i1 = min(T.n, i0 + kSahChunk);
+  bool left[kSahPer];
+  uint32_t nleft = 0, total;
+#pragma unroll
+  for (int j = 0; j < kSahPer; ++j) {
+    left[j] = i + j < i1 && (T.axis < 0 ? i + j < T.nl : (int)((it.bins[j] >> (5 * T.axis)) & 31u) <= T.bin);
+    nleft += left[j] ? 1u : 0u;
+  }
+  int l = before + (int)cta_exclusive_sum(nleft, s_warp, total);
+#pragma unroll
+  for (int j = 0; j < kSahPer; ++j) {
+    if (i + j >= i1) break;
+    // a right one follows the task's left ones and the right ones before it; positions stay
+    // inside the task even if bins and partition disagreed
+    const int q = left[j] ? l : T.nl + (i + j - l);
+    if (q < T.n) out[T.a + q] = it.p[j];
+    l += left[j] ? 1 : 0;
+  }
+  if (threadIdx.x == 0 && i1 == T.n && before + (int)total != T.nl) atomicExch(&B.hdr->corrupt, 1);  // never expected
+}
+
+__global__ void __launch_bounds__(kSahThreads, kSahBlocksPerSm) k_sah_levels(int32_t nf, int levels,
+                                                                             const uint32_t* __restrict__ bounds,
+                                                                             SahView S, BvhView B) {
+  __shared__ SahBins sb;
+  __shared__ SahChoice s_axis[3];
+  __shared__ float s_cost[3];
+  __shared__ int s_last, s_before;
+  __shared__ uint32_t s_warp[kSahThreads / 32];
+  const int tid = threadIdx.x;
+  GridBarrier bar{S.st->barrier, 0u, false};
+  if (blockIdx.x == 0) sah_root(nf, bounds, S);
+  grid_barrier(bar);
+  for (int level = 0; level < levels && !bar.failed; ++level) {
+    const SahLevel L = sah_level(S, level);
+    if (L.ntask == 0) break;  // the same in every CTA
+    SahTask* tasks = S.tasks[level & 1];
+    const uint32_t* in = S.idx[level & 1];
+    uint32_t* out = S.idx[(level + 1) & 1];
+    const int sroot = S.st->sroot;  // (level 0 sets it)
+    // bins, splits, and the scatter of tasks of one chunk
+    for (int c = blockIdx.x; c < L.nchunk; c += gridDim.x) {
+      const int t = S.chunk_task[level & 1][c];
+      SahTask T = tasks[t];
+      const int nc = sah_chunks(T.n), i0 = (c - T.chunk0) * kSahChunk, i1 = min(T.n, i0 + kSahChunk);
+      float sc[3];
+      const bool free = sah_free(T, sc);  // uniform over the CTA
+      SahItems it;
+      const int i = i0 + tid * kSahPer;
+#pragma unroll
+      for (int j = 0; j < kSahPer; ++j) {
+        it.p[j] = i + j < i1 ? in[T.a + i + j] : 0u;
+        it.bins[j] = 0u;
       }
-      const int id = sah_split_id(s, sroot);
-      B.parent[id] = T.parent;
-      if (T.parent >= 0) sah_set_child(B, T.parent, T.sd & 1, id);
-      for (int c = 0; c < 2; ++c) {
-        const int ca = c ? T.a + nl : T.a, cn = c ? T.n - nl : nl;
-        if (cn <= kSahSmall) {  // (one triangle: the warp builder writes the leaf)
-          const int slot = atomicAdd(&S.st->n_small, 1);
-          if (slot < S.max_small) S.small[slot] = make_int4(ca, cn, id, c | ((depth + 1) << 1) | (((level + 1) & 1) << 30));
-          else atomicExch(&B.hdr->corrupt, 1);  // more tasks than disjoint ranges: never expected
-        } else {
-          const unsigned long long old =
-              atomicAdd(&S.st->packed[level + 1], (1ull << 32) | (unsigned long long)sah_chunks(cn));
-          const int slot = (int)(old >> 32), chunk0 = (int)(old & 0xffffffffull);
-          if (slot < S.max_large && chunk0 + sah_chunks(cn) <= S.max_chunks) {
-            SahTask ct;
-            ct.a = ca; ct.n = cn; ct.parent = id; ct.sd = c | ((depth + 1) << 1);
-            ct.chunk0 = chunk0; ct.axis = -1; ct.bin = -1; ct.nl = 0;
-            const float3 lo = c ? rlo : llo, hi = c ? rhi : lhi;
-            ct.lo = make_float4(lo.x, lo.y, lo.z, 0.f);
-            ct.hi = make_float4(hi.x, hi.y, hi.z, 0.f);
-            S.tasks[(level + 1) & 1][slot] = ct;
-            child_slot[c] = slot;
-          } else {
-            atomicExch(&B.hdr->corrupt, 1);
+      sah_zero_bins(&sb, tid, blockDim.x);
+      __syncthreads();
+      if (free && i < i1) {
+        float4 c4[kSahPer], lo[kSahPer], hi[kSahPer];
+#pragma unroll
+        for (int j = 0; j < kSahPer; ++j) {
+          c4[j] = S.cen[it.p[j]];
+          lo[j] = S.pbox[2 * it.p[j]];
+          hi[j] = S.pbox[2 * it.p[j] + 1];
+        }
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          if (sc[k] <= 0.f) continue;
+          // a run of equal bins is added at once
+          int cb = -1;
+          uint32_t cn = 0u;
+          float3 clo, chi;
+#pragma unroll
+          for (int j = 0; j < kSahPer; ++j) {
+            if (i + j >= i1) break;
+            const int b = sah_bin(comp(c4[j], k), comp(T.lo, k), sc[k]);
+            it.bins[j] |= (uint32_t)b << (5 * k);
+            if (b != cb) {
+              if (cb >= 0) sah_flush(sb, k, cb, cn, clo, chi);
+              cb = b;
+              cn = 0u;
+              clo = mk(INFINITY, INFINITY, INFINITY);
+              chi = mk(-INFINITY, -INFINITY, -INFINITY);
+            }
+            ++cn;
+            clo = mk(fminf(clo.x, lo[j].x), fminf(clo.y, lo[j].y), fminf(clo.z, lo[j].z));
+            chi = mk(fmaxf(chi.x, hi[j].x), fmaxf(chi.y, hi[j].y), fmaxf(chi.z, hi[j].z));
+          }
+          if (cb >= 0) sah_flush(sb, k, cb, cn, clo, chi);
+        }
+      }
+      __syncthreads();
+      bool last = true;
+      if (nc > 1) {  // into the task's bins; the CTA that completes them goes on
+        SahBins& G = S.bins[level & 1][t];
+        for (int i = tid; i < 3 * kSahBins; i += blockDim.x) {
+          const int k = i / kSahBins, b = i % kSahBins;
+          const uint32_t n = sb.cnt[k][b];
+          S.chunk_cnt[(size_t)c * (3 * kSahBins) + i] = n;
+          if (!n) continue;
+          atomicAdd(&G.cnt[k][b], n);
+          for (int q = 0; q < 3; ++q) {
+            atomicMin(&G.lo[k][b][q], sb.lo[k][b][q]);
+            atomicMax(&G.hi[k][b][q], sb.hi[k][b][q]);
           }
         }
+        __threadfence();
+        __syncthreads();
+        if (tid == 0) s_last = atomicAdd(reinterpret_cast<uint32_t*>(&tasks[t].lo.w), 1u) == (uint32_t)nc - 1u;
+        __syncthreads();
+        last = s_last != 0;
+        if (last) {
+          __threadfence();
+          for (int i = tid; i < 3 * kSahBins; i += blockDim.x) {
+            const int k = i / kSahBins, b = i % kSahBins;
+            sb.cnt[k][b] = __ldcg(&G.cnt[k][b]);
+            for (int q = 0; q < 3; ++q) {
+              sb.lo[k][b][q] = __ldcg(&G.lo[k][b][q]);
+              sb.hi[k][b][q] = __ldcg(&G.hi[k][b][q]);
+            }
+          }
+          __syncthreads();
+        }
+      }
+      if (last) {
+        SahChoice ch;
+        sah_choose(sb, T, sc, free, s_axis, s_cost, ch);
+        T.axis = ch.axis;
+        T.bin = ch.bin;
+        T.nl = ch.nl;
+        if (nc > 1 && tid == 0) {
+          tasks[t].axis = ch.axis;
+          tasks[t].bin = ch.bin;
+          tasks[t].nl = ch.nl;
+        }
+        sah_emit(level, T, ch, sroot, S, B);
+        if (nc == 1) sah_scatter(T, it, out, 0, 0, B, s_warp);
+      }
+      __syncthreads();  // the shared arrays are used again
+    }
+    // the scatter of tasks of several chunks, once they are split
+    if (L.nchunk > L.ntask) {
+      grid_barrier(bar);
+      if (bar.failed) break;
+      for (int c = blockIdx.x; c < L.nchunk; c += gridDim.x) {
+        const SahTask T = tasks[S.chunk_task[level & 1][c]];
+        if (sah_chunks(T.n) == 1) continue;
+        float sc[3];
+        sah_free(T, sc);
+        const int i0 = (c - T.chunk0) * kSahChunk, i1 = min(T.n, i0 + kSahChunk), i = i0 + tid * kSahPer;
+        SahItems it;
+#pragma unroll
+        for (int j = 0; j < kSahPer; ++j) it.p[j] = i + j < i1 ? in[T.a + i + j] : 0u;
+#pragma unroll
+        for (int j = 0; j < kSahPer; ++j) {
+          it.bins[j] = 0u;
+          if (T.axis >= 0 && i + j < i1)
+            it.bins[j] = (uint32_t)sah_bin(comp(S.cen[it.p[j]], T.axis), comp(T.lo, T.axis), sc[T.axis]) << (5 * T.axis);
+        }
+        if (tid == 0) s_before = 0;
+        __syncthreads();
+        if (T.axis < 0) {
+          if (tid == 0) s_before = min(i0, T.nl);
+        } else {
+          uint32_t sum = 0;
+          const int bins = T.bin + 1, n = (c - T.chunk0) * bins;
+          for (int i = tid; i < n; i += blockDim.x)
+            sum += S.chunk_cnt[(size_t)(T.chunk0 + i / bins) * (3 * kSahBins) + T.axis * kSahBins + i % bins];
+          sum = __reduce_add_sync(kFull, sum);
+          if ((tid & 31) == 0 && sum) atomicAdd(&s_before, (int)sum);
+        }
+        __syncthreads();
+        sah_scatter(T, it, out, i0, s_before, B, s_warp);
+        __syncthreads();
       }
     }
-    for (int c = 0; c < 2; ++c) {
-      const int slot = __shfl_sync(kFull, child_slot[c], 0);
-      if (slot >= 0) sah_zero_bins(&S.bins[(level + 1) & 1][slot], lane, 32);
+    grid_barrier(bar);
+  }
+  if (bar.failed && tid == 0) atomicExch(&B.hdr->corrupt, 1);  // not co-resident: never expected
+}
+
+// Small tasks: one CTA builds a whole subtree (at most kSahSmall triangles)
+// with the same binned SAH, its triangles in shared memory, level by level: a
+// warp splits a range, a group of four lanes a range of at most kSahTiny (most
+// of the nodes).  What bounds it is the chain of splits of one task: a warp per
+// task, one split after another and three lanes sweeping the bins, took 271 us
+// for 5k triangles (1.40 ms for 1.08M); this takes 37 us (468 us).
+struct SahRange {
+  int a, n, parent, sd;  // positions within the task, parent node, side | depth << 1
+};
+struct SahSmallShared {
+  float cen[3][kSahSmall], lo[3][kSahSmall], hi[3][kSahSmall];
+  uint32_t prim[kSahSmall];
+  uint8_t ids[kSahSmall];  // local triangles in position order
+  SahRange big[2][kSahSmall / 4], tiny[2][kSahSmall / 2];
+  int n_big[2], n_tiny[2], sroot;
+  SahSmallBins bins[kSahSmallWarps];
+};
+
+// Node of a split range at its split position s: numbered, linked to its
+// parent, its children queued for the next level or, single triangles, linked.
+__device__ __forceinline__ void sah_small_node(SahSmallShared& sh, int cur, const SahRange& r, int nl, int a, int n_int,
+                                               const SahView& S, BvhView& B) {
+  const int s = a + r.a + nl - 1;
+  int sroot = sh.sroot;
+  if (r.parent < 0) {  // the whole tree is this one task
+    sroot = sh.sroot = s;
+    S.st->sroot = s;
+  }
+  const int id = sah_split_id(s, sroot);
+  B.parent[id] = r.parent;
+  if (r.parent >= 0) sah_set_child(B, r.parent, r.sd & 1, id);
+  for (int c = 0; c < 2; ++c) {
+    const SahRange ch{c ? r.a + nl : r.a, c ? r.n - nl : nl, id, c | (((r.sd >> 1) + 1) << 1)};
+    if (ch.n == 1) {
+      sah_set_child(B, id, c, ~(a + ch.a));
+      B.parent[n_int + a + ch.a] = id;
+    } else if (ch.n <= kSahTiny) {
+      sh.tiny[cur ^ 1][atomicAdd(&sh.n_tiny[cur ^ 1], 1)] = ch;
+    } else {
+      sh.big[cur ^ 1][atomicAdd(&sh.n_big[cur ^ 1], 1)] = ch;
     }
   }
 }
 
-// 3/4: left primitives of every chunk
-__global__ void __launch_bounds__(kSahThreads) k_sah_count(int level, SahView S) {
-  __shared__ int s_sum;
-  const SahLevel L = sah_level(S, level);
-  const SahTask* tasks = S.tasks[level & 1];
-  const uint32_t* __restrict__ in = S.idx[level & 1];
-  for (int c = blockIdx.x; c < L.nchunk; c += gridDim.x) {
-    const SahTask T = tasks[sah_find_task(tasks, L.ntask, c)];
-    float sc[3];
-    sah_free(T, sc);
-    if (threadIdx.x == 0) s_sum = 0;
-    __syncthreads();
-    const int i0 = (c - T.chunk0) * kSahChunk, i1 = min(T.n, i0 + kSahChunk);
-    int cnt = 0;
-    for (int i = i0 + threadIdx.x; i < i1; i += blockDim.x) cnt += sah_goes_left(S, T, sc, in[T.a + i], i) ? 1 : 0;
-    for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(kFull, cnt, o);
-    if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum, cnt);
-    __syncthreads();
-    if (threadIdx.x == 0) S.chunk_left[c] = (uint32_t)s_sum;
-    __syncthreads();
+// The split of a range of more than kSahTiny triangles, by one warp.
+__device__ __forceinline__ void sah_small_split(SahSmallShared& sh, SahSmallBins& sb, int cur, const SahRange& r, int a,
+                                                int n_int, const SahView& S, BvhView& B) {
+  static_assert(kSahSmallBins == 16 && kSahSmall == 128, "half a warp per axis; four triangles per lane");
+  const int lane = threadIdx.x & 31;
+  const int depth = r.sd >> 1;
+  // the range's triangles, in position order, and their centroids' bounds
+  int id[4];
+  float lo[3], hi[3], sc[3];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) id[q] = q * 32 + lane < r.n ? sh.ids[r.a + q * 32 + lane] : -1;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    uint32_t l = 0xffffffffu, h = 0u;
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (id[q] >= 0) {
+        const uint32_t o = f2ord(sh.cen[k][id[q]]);
+        l = min(l, o);
+        h = max(h, o);
+      }
+    lo[k] = ord2f(__reduce_min_sync(kFull, l));
+    hi[k] = ord2f(__reduce_max_sync(kFull, h));
+    sc[k] = sah_scale<kSahSmallBins>(lo[k], hi[k]);
   }
-}
-
-// 4/4: stable scatter of every chunk to [left | right] of its task
-__global__ void __launch_bounds__(kSahThreads) k_sah_scatter(int level, SahView S, BvhView B) {
-  __shared__ uint32_t s_warp[kSahThreads / 32];
-  __shared__ int s_prefix;
-  const SahLevel L = sah_level(S, level);
-  const SahTask* tasks = S.tasks[level & 1];
-  const uint32_t* __restrict__ in = S.idx[level & 1];
-  uint32_t* out = S.idx[(level + 1) & 1];
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  for (int c = blockIdx.x; c < L.nchunk; c += gridDim.x) {
-    const SahTask T = tasks[sah_find_task(tasks, L.ntask, c)];
-    float sc[3];
-    sah_free(T, sc);
-    if (tid == 0) s_prefix = 0;
-    __syncthreads();
-    int pre = 0;
-    for (int j = T.chunk0 + tid; j < c; j += blockDim.x) pre += (int)S.chunk_left[j];
-    for (int o = 16; o > 0; o >>= 1) pre += __shfl_xor_sync(kFull, pre, o);
-    if (lane == 0 && pre) atomicAdd(&s_prefix, pre);
-    __syncthreads();
-    const int i0 = (c - T.chunk0) * kSahChunk, i1 = min(T.n, i0 + kSahChunk);
-    int lbase = s_prefix, rbase = i0 - s_prefix;
-    for (int base = i0; base < i1; base += blockDim.x) {
-      const int i = base + tid;
-      const bool valid = i < i1;
-      uint32_t p = 0u;
-      bool left = false;
-      if (valid) {
-        p = in[T.a + i];
-        left = sah_goes_left(S, T, sc, p, i);
-      }
-      const unsigned bal = __ballot_sync(kFull, left);
-      if (lane == 0) s_warp[wid] = __popc(bal);
-      __syncthreads();
-      int woff = 0, tot = 0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-        const int cw = (int)s_warp[w];
-        if (w < wid) woff += cw;
-        tot += cw;
-      }
-      const int lrank = woff + __popc(bal & ((1u << lane) - 1u));
-      if (valid) {  // positions stay inside the task even if bins and partition disagreed
-        const int q = left ? lbase + lrank : T.nl + rbase + (i - base - lrank);
-        if (q < T.n) out[T.a + q] = p;
-      }
-      lbase += tot;
-      rbase += min((int)blockDim.x, i1 - base) - tot;
-      __syncthreads();
+  int axis = -1, bin = -1, nl = r.n / 2;
+  if (depth < kSahSmallFreeDepth && (sc[0] > 0.f || sc[1] > 0.f || sc[2] > 0.f)) {
+    sah_zero_bins(&sb, lane, 32);
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (id[q] < 0) continue;
+      const float3 plo = mk(sh.lo[0][id[q]], sh.lo[1][id[q]], sh.lo[2][id[q]]);
+      const float3 phi = mk(sh.hi[0][id[q]], sh.hi[1][id[q]], sh.hi[2][id[q]]);
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        if (sc[k] > 0.f) sah_flush(sb, k, sah_bin<kSahSmallBins>(sh.cen[k][id[q]], lo[k], sc[k]), 1u, plo, phi);
     }
-    if (tid == 0 && i1 == T.n && lbase != T.nl) atomicExch(&B.hdr->corrupt, 1);  // never expected
+    __syncwarp();
+    // lanes 0..15 scan the bins upward (left of boundary i: lane i), lanes 16..31
+    // downward (right of boundary i: bins i + 1.., lane 16 + 14 - i)
+    float bc = INFINITY;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      if (!(sc[k] > 0.f)) continue;
+      const int b = lane < 16 ? lane : 31 - lane;
+      uint32_t c = sb.cnt[k][b];
+      float3 l = mk(INFINITY, INFINITY, INFINITY), h = mk(-INFINITY, -INFINITY, -INFINITY);
+      if (c) {
+        l = mk(ord2f(sb.lo[k][b][0]), ord2f(sb.lo[k][b][1]), ord2f(sb.lo[k][b][2]));
+        h = mk(ord2f(sb.hi[k][b][0]), ord2f(sb.hi[k][b][1]), ord2f(sb.hi[k][b][2]));
+      }
+#pragma unroll
+      for (int o = 1; o < 16; o <<= 1) {
+        const uint32_t oc = __shfl_up_sync(kFull, c, o, 16);
+        const float3 ol = mk(__shfl_up_sync(kFull, l.x, o, 16), __shfl_up_sync(kFull, l.y, o, 16), __shfl_up_sync(kFull, l.z, o, 16));
+        const float3 oh = mk(__shfl_up_sync(kFull, h.x, o, 16), __shfl_up_sync(kFull, h.y, o, 16), __shfl_up_sync(kFull, h.z, o, 16));
+        if ((lane & 15) >= o) {
+          c += oc;
+          l = mk(fminf(l.x, ol.x), fminf(l.y, ol.y), fminf(l.z, ol.z));
+          h = mk(fmaxf(h.x, oh.x), fmaxf(h.y, oh.y), fmaxf(h.z, oh.z));
+        }
+      }
+      const float area = c ? sah_area(l, h) : 0.f;
+      const int from = lane < 15 ? 30 - lane : lane;
+      const uint32_t rc = __shfl_sync(kFull, c, from);
+      const float rarea = __shfl_sync(kFull, area, from);
+      const bool cut = lane < 15 && c > 0 && rc > 0;
+      const float cost = cut ? area * (float)c + rarea * (float)rc : INFINITY;
+      const uint32_t key = cut && cost < INFINITY ? __float_as_uint(cost) : 0x7f800000u;
+      const uint32_t least = __reduce_min_sync(kFull, key);
+      if (least < 0x7f800000u && __uint_as_float(least) < bc) {
+        bc = __uint_as_float(least);
+        axis = k;
+        bin = __ffs(__ballot_sync(kFull, key == least)) - 1;
+        nl = (int)__shfl_sync(kFull, c, bin);
+      }
+    }
+    __syncwarp();
+  }
+  // stable partition in place (every lane holds its triangles)
+  int lbase = 0, rbase = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const bool valid = id[q] >= 0;
+    bool left = false;
+    if (valid) {
+      if (axis < 0) left = q * 32 + lane < nl;
+      else {
+        const float c = axis == 0 ? sh.cen[0][id[q]] : (axis == 1 ? sh.cen[1][id[q]] : sh.cen[2][id[q]]);
+        const float l = axis == 0 ? lo[0] : (axis == 1 ? lo[1] : lo[2]), s = axis == 0 ? sc[0] : (axis == 1 ? sc[1] : sc[2]);
+        left = sah_bin<kSahSmallBins>(c, l, s) <= bin;
+      }
+    }
+    const unsigned bl = __ballot_sync(kFull, left), bv = __ballot_sync(kFull, valid);
+    const unsigned below = (1u << lane) - 1u;
+    if (valid) {  // inside the range even if bins and partition disagreed
+      const int p = left ? lbase + __popc(bl & below) : nl + rbase + __popc(bv & ~bl & below);
+      if (p < r.n) sh.ids[r.a + p] = (uint8_t)id[q];
+    }
+    lbase += __popc(bl);
+    rbase += __popc(bv & ~bl);
+  }
+  if (lane == 0) {
+    if (lbase != nl) atomicExch(&B.hdr->corrupt, 1);
+    sah_small_node(sh, cur, r, nl, a, n_int, S, B);
   }
 }
 
-// Small tasks: one warp builds a whole subtree (at most kSahSmall triangles)
-// with the same binned SAH, the range held in shared memory.
+// The split of a range of 2..kSahTiny triangles, by four lanes (`live`: the
+// group has one; every lane of the warp calls): the median of the centroids
+// along their longest extent (ties by position); binning would cost far more
+// than it can gain on a handful of triangles.
+__device__ __forceinline__ void sah_tiny_split(SahSmallShared& sh, int cur, bool live, const SahRange& r, int a,
+                                               int n_int, const SahView& S, BvhView& B) {
+  const int lane = threadIdx.x & 31, l4 = lane & 3;
+  const bool mine = live && l4 < r.n;
+  const int id = mine ? sh.ids[r.a + l4] : 0;
+  float c[3], ext[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    c[k] = mine ? sh.cen[k][id] : 0.f;
+    float lo = mine ? c[k] : INFINITY, hi = mine ? c[k] : -INFINITY;
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+      lo = fminf(lo, __shfl_xor_sync(kFull, lo, o));
+      hi = fmaxf(hi, __shfl_xor_sync(kFull, hi, o));
+    }
+    ext[k] = hi - lo;
+  }
+  const int la = (ext[0] >= ext[1] && ext[0] >= ext[2]) ? 0 : (ext[1] >= ext[2] ? 1 : 2);
+  const float x = la == 0 ? c[0] : (la == 1 ? c[1] : c[2]);
+  int rank = 0;
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    const float xj = __shfl_sync(kFull, x, j, 4);
+    if (j < r.n) rank += (xj < x || (xj == x && j < l4)) ? 1 : 0;
+  }
+  const int nl = r.n / 2;
+  const bool left = mine && rank < nl;
+  const unsigned bl = (__ballot_sync(kFull, left) >> (lane & 28)) & 15u;
+  const unsigned bv = (__ballot_sync(kFull, mine) >> (lane & 28)) & 15u;
+  const unsigned below = (1u << l4) - 1u;
+  if (mine) {
+    const int p = left ? __popc(bl & below) : nl + __popc(bv & ~bl & below);
+    if (p < r.n) sh.ids[r.a + p] = (uint8_t)id;
+  }
+  if (live && l4 == 0) {
+    if (__popc(bl) != nl) atomicExch(&B.hdr->corrupt, 1);
+    sah_small_node(sh, cur, r, nl, a, n_int, S, B);
+  }
+}
+
 __global__ void __launch_bounds__(32 * kSahSmallWarps) k_sah_small(SahView S, BvhView B) {
-  __shared__ uint32_t s_ids[kSahSmallWarps][kSahSmall], s_tmp[kSahSmallWarps][kSahSmall];
-  __shared__ int4 s_stack[kSahSmallWarps][kSahSmall / 2 + 1];
-  __shared__ SahSmallBins s_bins[kSahSmallWarps];
+  static_assert(kSahTiny == 4, "a tiny range has four lanes");
+  __shared__ SahSmallShared sh;
   const int n_int = B.hdr->n_int;
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint32_t* ids = s_ids[w];
-  uint32_t* tmp = s_tmp[w];
-  int4* stack = s_stack[w];
-  SahSmallBins& sb = s_bins[w];
+  const int tid = threadIdx.x, w = tid >> 5;
   const int nsmall = min(S.st->n_small, S.max_small);
-  for (int t = blockIdx.x * kSahSmallWarps + w; t < nsmall; t += gridDim.x * kSahSmallWarps) {
+  for (int t = blockIdx.x; t < nsmall; t += gridDim.x) {
     const int4 T = S.small[t];
     const int a = T.x, n = T.y;
     const uint32_t* in = S.idx[(T.w >> 30) & 1];
     if (n == 1) {  // a one-triangle child of a large task
-      if (lane == 0) {
+      if (tid == 0) {
         sah_set_child(B, T.z, T.w & 1, ~a);
         B.parent[n_int + a] = T.z;
         B.leaf_tri[a] = (int32_t)in[a];
       }
-      continue;
+      continue;  // uniform over the CTA
     }
-    for (int i = lane; i < n; i += 32) ids[i] = in[a + i];
-    int sroot = T.z < 0 ? -1 : S.st->sroot;
-    int sp = 0;
-    if (lane == 0) stack[0] = make_int4(0, n, T.z, T.w & 0x3fffffff);
-    sp = 1;
-    __syncwarp();
-    while (sp > 0) {
-      --sp;
-      const int4 e = stack[sp];
-      __syncwarp();
-      const int ra = e.x, rn = e.y, par = e.z, side = e.w & 1, depth = e.w >> 1;
-      // centroid bounds of the range
-      float3 lo = mk(INFINITY, INFINITY, INFINITY), hi = mk(-INFINITY, -INFINITY, -INFINITY);
-      for (int i = lane; i < rn; i += 32) {
-        const float4 c = S.cen[ids[ra + i]];
-        lo = mk(fminf(lo.x, c.x), fminf(lo.y, c.y), fminf(lo.z, c.z));
-        hi = mk(fmaxf(hi.x, c.x), fmaxf(hi.y, c.y), fmaxf(hi.z, c.z));
-      }
-      for (int o = 16; o > 0; o >>= 1) {
-        lo.x = fminf(lo.x, __shfl_xor_sync(kFull, lo.x, o));
-        lo.y = fminf(lo.y, __shfl_xor_sync(kFull, lo.y, o));
-        lo.z = fminf(lo.z, __shfl_xor_sync(kFull, lo.z, o));
-        hi.x = fmaxf(hi.x, __shfl_xor_sync(kFull, hi.x, o));
-        hi.y = fmaxf(hi.y, __shfl_xor_sync(kFull, hi.y, o));
-        hi.z = fmaxf(hi.z, __shfl_xor_sync(kFull, hi.z, o));
-      }
-      const float sc[3] = {sah_scale<kSahSmallBins>(lo.x, hi.x), sah_scale<kSahSmallBins>(lo.y, hi.y),
-                           sah_scale<kSahSmallBins>(lo.z, hi.z)};
-      int axis = -1, bin = -1, nl = rn / 2;
-      // a range of at most kSahTiny triangles splits at the median of its
-      // centroids along their longest extent (ties by position): binning
-      // would cost far more than it can gain on a handful of triangles
-      const bool tiny = rn <= kSahTiny;
-      int tiny_rank = 0;
-      if (tiny) {
-        const float3 ext = hi - lo;
-        const int la = (ext.x >= ext.y && ext.x >= ext.z) ? 0 : (ext.y >= ext.z ? 1 : 2);
-        const float c = lane < rn ? comp(S.cen[ids[ra + lane]], la) : 0.f;
-        for (int j = 0; j < rn; ++j) {
-          const float cj = __shfl_sync(kFull, c, j);
-          tiny_rank += (cj < c || (cj == c && j < (int)lane)) ? 1 : 0;
-        }
-      } else if (depth < kSahSmallFreeDepth && (sc[0] > 0.f || sc[1] > 0.f || sc[2] > 0.f)) {
-        sah_zero_bins(&sb, lane, 32);
-        __syncwarp();
-        for (int i = lane; i < rn; i += 32) {
-          const uint32_t p = ids[ra + i];
-          const float4 c = S.cen[p], plo = S.pbox[2 * p], phi = S.pbox[2 * p + 1];
-          for (int k = 0; k < 3; ++k) {
-            if (sc[k] <= 0.f) continue;
-            sah_flush(sb, k, sah_bin<kSahSmallBins>(comp(c, k), comp3(lo, k), sc[k]), 1u, mk(plo.x, plo.y, plo.z),
-                      mk(phi.x, phi.y, phi.z));
-          }
-        }
-        __syncwarp();
-        SahSplit sp3;
-        sp3.cost = INFINITY; sp3.bin = -1; sp3.axis = lane; sp3.nl = 0;
-        if (lane < 3 && sc[lane] > 0.f) sp3 = sah_sweep(sb, lane);
-        float bc = INFINITY;
-        for (int k = 0; k < 3; ++k) {
-          const float ck = __shfl_sync(kFull, sp3.cost, k);
-          const int bk = __shfl_sync(kFull, sp3.bin, k);
-          if (bk >= 0 && ck < bc) { bc = ck; axis = k; }
-        }
-        if (axis >= 0) {
-          bin = __shfl_sync(kFull, sp3.bin, axis);
-          nl = __shfl_sync(kFull, sp3.nl, axis);
-        }
-        __syncwarp();
-      }
-      // stable partition of ids[ra, ra + rn) through tmp
-      int lbase = 0;
-      int rbase = 0;
-      for (int base = 0; base < rn; base += 32) {
-        const int i = base + lane;
-        const bool valid = i < rn;
-        uint32_t p = 0u;
-        bool left = false;
-        if (valid) {
-          p = ids[ra + i];
-          left = tiny ? tiny_rank < nl
-                      : (axis >= 0 ? sah_bin<kSahSmallBins>(comp(S.cen[p], axis), comp3(lo, axis), sc[axis]) <= bin
-                                   : i < nl);
-        }
-        const unsigned bal = __ballot_sync(kFull, left);
-        const int lr = __popc(bal & ((1u << lane) - 1u));
-        if (valid) {  // inside the range even if bins and partition disagreed
-          const int q = left ? lbase + lr : nl + rbase + (lane - lr);
-          if (q < rn) tmp[ra + q] = p;
-        }
-        const int tot = __popc(bal);
-        lbase += tot;
-        rbase += min(32, rn - base) - tot;
-      }
-      __syncwarp();
-      for (int i = lane; i < rn; i += 32) ids[ra + i] = tmp[ra + i];
-      __syncwarp();
-      if (lbase != nl && lane == 0) atomicExch(&B.hdr->corrupt, 1);
-      const int s = a + ra + nl - 1;
-      if (par < 0) sroot = s;  // the whole tree is this one task
-      const int id = sah_split_id(s, sroot);
-      if (lane == 0) {
-        B.parent[id] = par;
-        if (par >= 0) sah_set_child(B, par, side, id);
-        if (par < 0) S.st->sroot = s;
-      }
-      for (int c = 1; c >= 0; --c) {
-        const int ca = c ? ra + nl : ra, cn = c ? rn - nl : nl;
-        if (cn == 1) {
-          if (lane == 0) {
-            sah_set_child(B, id, c, ~(a + ca));
-            B.parent[n_int + a + ca] = id;
-          }
-        } else {
-          if (lane == 0) stack[sp] = make_int4(ca, cn, id, c | ((depth + 1) << 1));
-          ++sp;
-        }
-      }
-      __syncwarp();
+    for (int i = tid; i < n; i += blockDim.x) {
+      const uint32_t p = in[a + i];
+      const float4 c = S.cen[p], lo = S.pbox[2 * p], hi = S.pbox[2 * p + 1];
+      sh.prim[i] = p;
+      sh.ids[i] = (uint8_t)i;
+      sh.cen[0][i] = c.x; sh.cen[1][i] = c.y; sh.cen[2][i] = c.z;
+      sh.lo[0][i] = lo.x; sh.lo[1][i] = lo.y; sh.lo[2][i] = lo.z;
+      sh.hi[0][i] = hi.x; sh.hi[1][i] = hi.y; sh.hi[2][i] = hi.z;
     }
-    for (int i = lane; i < n; i += 32) B.leaf_tri[a + i] = (int32_t)ids[i];
-    __syncwarp();
+    if (tid == 0) {
+      const SahRange r{0, n, T.z, T.w & 0x3fffffff};
+      sh.n_big[0] = n > kSahTiny;
+      sh.n_tiny[0] = n <= kSahTiny;
+      if (n > kSahTiny) sh.big[0][0] = r; else sh.tiny[0][0] = r;
+      sh.n_big[1] = sh.n_tiny[1] = 0;
+      sh.sroot = T.z < 0 ? -1 : S.st->sroot;
+    }
+    __syncthreads();
+    for (int cur = 0;; cur ^= 1) {
+      const int nb = sh.n_big[cur], nt = sh.n_tiny[cur];
+      if (nb == 0 && nt == 0) break;  // uniform: read between two barriers
+      for (int i = w; i < nb; i += kSahSmallWarps) sah_small_split(sh, sh.bins[w], cur, sh.big[cur][i], a, n_int, S, B);
+      // (the warps take the tiny ranges from the other end, so that the big ones' do not wait)
+      for (int i0 = (kSahSmallWarps - 1 - w) * 8; i0 < nt; i0 += kSahSmallWarps * 8) {
+        const int i = i0 + ((tid & 31) >> 2);
+        sah_tiny_split(sh, cur, i < nt, sh.tiny[cur][i < nt ? i : i0], a, n_int, S, B);
+      }
+      __syncthreads();
+      if (tid == 0) sh.n_big[cur] = sh.n_tiny[cur] = 0;
+      __syncthreads();
+    }
+    for (int i = tid; i < n; i += blockDim.x) B.leaf_tri[a + i] = (int32_t)sh.prim[sh.ids[i]];
+    __syncthreads();
   }
 }
 
@@ -1118,7 +1364,11 @@ __global__ void k_validate(BvhView B) {
   if (bad) atomicExch(&B.hdr->corrupt, 1);
 }
 
-__global__ void k_bvh_header(BvhHeader* h, int32_t nf) {
+// the header, the (empty) centroid bounds and the SAH build's state
+__global__ void k_bvh_header(BvhHeader* h, int32_t nf, uint32_t* bounds, SahState* st) {
+  if (threadIdx.x < 6) bounds[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
+  for (uint32_t i = threadIdx.x; i < sizeof(SahState) / 4; i += blockDim.x) reinterpret_cast<uint32_t*>(st)[i] = 0u;
+  if (threadIdx.x) return;
   h->nf = nf;
   h->n_int = nf > 1 ? nf - 1 : 1;
   h->n4 = 0;
@@ -1128,7 +1378,7 @@ __global__ void k_bvh_header(BvhHeader* h, int32_t nf) {
 
 // scratch layout for build/refit
 struct BuildScratch {
-  uint32_t *keys_a, *keys_b, *vals_a, *vals_b, *hist, *arrive, *bounds;
+  uint32_t *keys_a, *keys_b, *vals_a, *vals_b, *hist, *arrive, *bounds, *totals;
   SahView sah;
   size_t total;
   BuildScratch(void* base, int32_t nf) {
@@ -1141,6 +1391,7 @@ struct BuildScratch {
     const size_t hi = take(sizeof(uint32_t) * 256 * (size_t)nblocks);
     const size_t ar = take(sizeof(uint32_t) * n_int);
     const size_t bo = take(sizeof(uint32_t) * 8);
+    const size_t to = take(sizeof(uint32_t) * kScanBlocks);
     // binned SAH build: centroids, boxes, task lists and bins of two levels,
     // left counts per chunk, small tasks
     sah.max_large = nf / (kSahSmall + 1) + 1;
@@ -1149,13 +1400,15 @@ struct BuildScratch {
     const size_t ce = take(sizeof(float4) * nf), pb = take(sizeof(float4) * 2 * (size_t)nf);
     const size_t t0 = take(sizeof(SahTask) * sah.max_large), t1 = take(sizeof(SahTask) * sah.max_large);
     const size_t b0 = take(sizeof(SahBins) * sah.max_large), b1 = take(sizeof(SahBins) * sah.max_large);
-    const size_t cl = take(sizeof(uint32_t) * sah.max_chunks);
+    const size_t c0 = take(sizeof(int) * sah.max_chunks), c1 = take(sizeof(int) * sah.max_chunks);
+    const size_t cl = take(sizeof(uint32_t) * 3 * kSahBins * (size_t)sah.max_chunks);
     const size_t sm = take(sizeof(int4) * sah.max_small), st = take(sizeof(SahState));
     total = o;
     char* b = (char*)base;
     keys_a = (uint32_t*)(b + ka); keys_b = (uint32_t*)(b + kb);
     vals_a = (uint32_t*)(b + va); vals_b = (uint32_t*)(b + vb);
     hist = (uint32_t*)(b + hi); arrive = (uint32_t*)(b + ar); bounds = (uint32_t*)(b + bo);
+    totals = (uint32_t*)(b + to);
     sah.cen = (float4*)(b + ce);
     sah.pbox = (float4*)(b + pb);
     sah.idx[0] = vals_a;
@@ -1164,7 +1417,9 @@ struct BuildScratch {
     sah.tasks[1] = (SahTask*)(b + t1);
     sah.bins[0] = (SahBins*)(b + b0);
     sah.bins[1] = (SahBins*)(b + b1);
-    sah.chunk_left = (uint32_t*)(b + cl);
+    sah.chunk_task[0] = (int*)(b + c0);
+    sah.chunk_task[1] = (int*)(b + c1);
+    sah.chunk_cnt = (uint32_t*)(b + cl);
     sah.small = (int4*)(b + sm);
     sah.st = (SahState*)(b + st);
   }
@@ -1195,12 +1450,10 @@ void launch_refit(const float* V, const int32_t* F, int32_t nf, void* bvh, void*
 // ceil(log2(nf / kSahSmall)) + 1 more levels every task is small; small
 // tasks take free splits to depth kSahSmallFreeDepth, then at most
 // log2(kSahSmall) median levels: the tree is at most 63 deep, within the
-// traversal's 64-entry stack.  Levels beyond the last large one launch and
-// return at once (the host does not wait to learn how many there were).
+// traversal's 64-entry stack.
 static void launch_sah_topology(const float* V, const int32_t* F, int32_t nf, BvhView& B, BuildScratch& S,
                                 cudaStream_t s) {
-  k_sah_prims<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, S.sah, B);
-  k_sah_root<<<1, 64, 0, s>>>(nf, S.bounds, S.sah);
+  k_sah_prims<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, S.bounds, S.sah, B);
   int levels = 0;
   if (nf > kSahSmall) {
     int lg = 0;
@@ -1208,22 +1461,30 @@ static void launch_sah_topology(const float* V, const int32_t* F, int32_t nf, Bv
     levels = kSahFreeDepth + lg + 2;
     if (levels > kSahMaxLevels) levels = kSahMaxLevels;
   }
-  const int grid = 4 * num_sms();
   {
     ProfScope ps("sah_large_levels", s);
-    for (int L = 0; L < levels; ++L) {
-      k_sah_bin<<<grid, kSahThreads, 0, s>>>(L, S.sah);
-      k_sah_split<<<grid_for(S.sah.max_large * 32, 128), 128, 0, s>>>(L, S.sah, B);
-      k_sah_count<<<grid, kSahThreads, 0, s>>>(L, S.sah);
-      k_sah_scatter<<<grid, kSahThreads, 0, s>>>(L, S.sah, B);
-    }
+    // one CTA per 512 triangles: enough for the tasks of the last levels, and
+    // a small mesh's barriers stay cheap
+    int blocks = (nf + 511) / 512;
+    int most = kSahBlocksPerSm * num_sms();
+    if (most > kBarrierBlocks) most = kBarrierBlocks;
+    if (blocks > most) blocks = most;
+    const uint32_t* bounds = S.bounds;
+    void* args[] = {&nf, &levels, &bounds, &S.sah, &B};
+    cudaLaunchCooperativeKernel((const void*)k_sah_levels, dim3(blocks), dim3(kSahThreads), args, 0, s);
   }
   ProfScope ps("sah_small", s);
-  k_sah_small<<<grid_for(nf / 2 + 1, 32 * kSahSmallWarps), 32 * kSahSmallWarps, 0, s>>>(S.sah, B);
+  // at most one task per two triangles, a CTA each; about kSahSmall / 2 in practice
+  k_sah_small<<<grid_for(nf / 32 + 1, 1), 32 * kSahSmallWarps, 0, s>>>(S.sah, B);
 }
 
-// Exclusive scan of m entries in place (one CTA; used by the mesh topology).
-void launch_scan_exclusive(uint32_t* a, int32_t m, cudaStream_t s) { k_scan_exclusive<<<1, 1024, 0, s>>>(a, m); }
+void launch_scan_exclusive(const uint32_t* src, uint32_t* dst, int32_t m, uint32_t* totals, cudaStream_t s) {
+  const int64_t tiles = ((int64_t)m + kScanTile - 1) / kScanTile;
+  const int64_t per = (tiles + kScanBlocks - 1) / kScanBlocks;  // tiles per span
+  const int blocks = (int)((tiles + per - 1) / per);
+  if (blocks > 1) k_scan_totals<<<blocks, kScanThreads, 0, s>>>(src, m, per * kScanTile, totals);
+  k_scan_apply<<<blocks, kScanThreads, 0, s>>>(src, dst, m, per * kScanTile, totals);
+}
 
 void launch_build(const float* V, const int32_t* F, int32_t nf, void* bvh, void* scratch, cudaStream_t s) {
   BvhView B = bvh_view(bvh, nf);
@@ -1232,18 +1493,17 @@ void launch_build(const float* V, const int32_t* F, int32_t nf, void* bvh, void*
   const bool sah = g_tuning.bvh_builder == 1 && nf > 1;
   {
     ProfScope ps(sah ? "sah_build" : "lbvh_build", s);
-    k_bvh_header<<<1, 1, 0, s>>>(B.hdr, nf);
-    k_init_bounds<<<1, 32, 0, s>>>(S.bounds);
-    k_centroid_bounds<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, S.bounds);
+    k_bvh_header<<<1, 256, 0, s>>>(B.hdr, nf, S.bounds, S.sah.st);
     if (sah) {
       launch_sah_topology(V, F, nf, B, S, s);
     } else {
+      k_centroid_bounds<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, S.bounds);
       k_morton<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, S.bounds, S.keys_a, S.vals_a);
       const int nblocks = (nf + kSortTile - 1) / kSortTile;
       uint32_t *kin = S.keys_a, *vin = S.vals_a, *kout = S.keys_b, *vout = S.vals_b;
       for (int shift = 0; shift < 32; shift += 8) {
         k_radix_hist<<<nblocks, kSortThreads, 0, s>>>(kin, nf, shift, S.hist);
-        k_scan_exclusive<<<1, 1024, 0, s>>>(S.hist, 256 * nblocks);
+        launch_scan_exclusive(S.hist, S.hist, 256 * nblocks, S.totals, s);
         k_radix_scatter<<<nblocks, kSortThreads, 0, s>>>(kin, vin, nf, shift, S.hist, kout, vout);
         uint32_t* t = kin; kin = kout; kout = t;
         t = vin; vin = vout; vout = t;
@@ -1259,7 +1519,7 @@ void launch_build(const float* V, const int32_t* F, int32_t nf, void* bvh, void*
     // 4-wide topology: even-depth nodes, numbered by a scan
     uint32_t* flag = S.keys_b;  // free after the sort (unused by the SAH build)
     k_even_depth<<<grid_for(n_int, 256), 256, 0, s>>>(B, flag);
-    k_scan_exclusive<<<1, 1024, 0, s>>>(flag, n_int);
+    launch_scan_exclusive(flag, flag, n_int, S.totals, s);
     k_bin_to4<<<grid_for(n_int, 256), 256, 0, s>>>(B, flag);
     k_node4_topology<<<grid_for(n_int, 256), 256, 0, s>>>(B);
     k_validate<<<grid_for(n_int, 256), 256, 0, s>>>(B);

@@ -421,6 +421,56 @@ __device__ __forceinline__ float warp_sum(float v) {
   return v;
 }
 
+// ---------------------------------------------------------------------------
+// Barrier of a cooperative grid: every CTA publishes its arrival, CTA 0 polls
+// the arrivals and publishes the release, which the others poll (in one of
+// eight copies, a 128-byte line each).  What any thread wrote before it, every
+// thread can read after it.  Every wait is bounded: a launch that is not
+// co-resident gives up after a second or so (failed), and the caller leaves.
+// ---------------------------------------------------------------------------
+constexpr int kBarrierBlocks = 1024;  // most CTAs
+constexpr int kBarrierCopies = 8;
+constexpr size_t kBarrierWords = kBarrierBlocks + 32 * kBarrierCopies;  // cleared before the launch
+constexpr int kBarrierSpins = 1 << 21;
+
+struct GridBarrier {
+  uint32_t* word;
+  uint32_t n;
+  bool failed;
+};
+__device__ __forceinline__ bool barrier_wait(const uint32_t* p, uint32_t n) {
+  uint32_t v;
+  int spins = 0;
+  do {
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    if (v == n) return true;
+  } while (++spins < kBarrierSpins);
+  return false;
+}
+__device__ __forceinline__ void barrier_post(uint32_t* p, uint32_t n) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(n) : "memory");
+}
+__device__ __forceinline__ void grid_barrier(GridBarrier& g) {
+  ++g.n;
+  if (gridDim.x == 1) {  // atomics' results as well (they do not pass through L1)
+    __threadfence();
+    __syncthreads();
+    __threadfence();
+    return;
+  }
+  __syncthreads();
+  bool ok = true;
+  if (blockIdx.x == 0) {
+    for (uint32_t i = threadIdx.x + 1; i < gridDim.x && ok; i += blockDim.x) ok = barrier_wait(g.word + i, g.n);
+  } else if (threadIdx.x == 0) {
+    barrier_post(g.word + blockIdx.x, g.n);
+    ok = barrier_wait(g.word + kBarrierBlocks + 32 * (blockIdx.x % kBarrierCopies), g.n);
+  }
+  if (__syncthreads_or(!ok)) g.failed = true;
+  if (blockIdx.x == 0 && threadIdx.x < kBarrierCopies && !g.failed)
+    barrier_post(g.word + kBarrierBlocks + 32 * threadIdx.x, g.n);
+}
+
 // PCG hash (Jarzynski & Olano, "Hash Functions for GPU Rendering", JCGT 2020)
 __host__ __device__ __forceinline__ uint32_t pcg_hash(uint32_t v) {
   uint32_t state = v * 747796405u + 2891336453u;
@@ -434,7 +484,10 @@ __host__ __device__ __forceinline__ uint32_t pcg_hash(uint32_t v) {
 dt_status set_error(dt_status code, const char* fmt, ...);
 dt_status check_launch(const char* what);
 int num_sms();
-void launch_scan_exclusive(uint32_t* a, int32_t m, cudaStream_t s);  // dt_bvh.cu
+// Exclusive scan of m entries (dt_bvh.cu), 16-byte aligned arrays, src == dst
+// allowed; totals: kScanBlocks words.
+constexpr int kScanBlocks = 1024;
+void launch_scan_exclusive(const uint32_t* src, uint32_t* dst, int32_t m, uint32_t* totals, cudaStream_t s);
 
 // Per-kernel event timing (dt_profile_enable).  Scoped: records a start event
 // on construction and a stop event on destruction when profiling is on.

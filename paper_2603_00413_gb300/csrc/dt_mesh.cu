@@ -32,7 +32,7 @@ struct TopoHeader {
 };
 
 struct TopoLayout {
-  size_t off_row, off_col, off_raw_cnt, off_raw_off, off_cursor, off_raw, total;
+  size_t off_row, off_col, off_raw_cnt, off_raw_off, off_cursor, off_totals, off_raw, total;
   TopoLayout(int32_t nv, int32_t nf) {
     size_t o = 256;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
@@ -41,6 +41,7 @@ struct TopoLayout {
     off_raw_cnt = take(((size_t)nv + 1) * sizeof(uint32_t));
     off_raw_off = take(((size_t)nv + 1) * sizeof(uint32_t));
     off_cursor = take((size_t)nv * sizeof(uint32_t));
+    off_totals = take((size_t)kScanBlocks * sizeof(uint32_t));
     off_raw = take((size_t)6 * nf * sizeof(int32_t));
     total = o;
   }
@@ -53,6 +54,7 @@ struct TopoView {
   uint32_t* raw_cnt;
   uint32_t* raw_off;
   uint32_t* cursor;
+  uint32_t* totals;
   int32_t* raw;
 };
 
@@ -61,7 +63,7 @@ static TopoView topo_view(void* base, int32_t nv, int32_t nf) {
   char* b = (char*)base;
   return TopoView{(TopoHeader*)b, (int32_t*)(b + L.off_row), (int32_t*)(b + L.off_col),
                   (uint32_t*)(b + L.off_raw_cnt), (uint32_t*)(b + L.off_raw_off), (uint32_t*)(b + L.off_cursor),
-                  (int32_t*)(b + L.off_raw)};
+                  (uint32_t*)(b + L.off_totals), (int32_t*)(b + L.off_raw)};
 }
 
 size_t topology_bytes(int32_t nv, int32_t nf) { return TopoLayout(nv, nf).total; }
@@ -155,12 +157,12 @@ void launch_build_topology(const int32_t* F, int32_t nf, int32_t nv, void* topo,
   cudaMemsetAsync(T.cursor, 0, (size_t)nv * sizeof(uint32_t), s);
   k_topo_count<<<blocks_for(nf, 256), 256, 0, s>>>(F, nf, nv, T.raw_cnt);
   cudaMemcpyAsync(T.raw_off, T.raw_cnt, ((size_t)nv + 1) * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-  launch_scan_exclusive(T.raw_off, nv + 1, s);
+  launch_scan_exclusive(T.raw_off, T.raw_off, nv + 1, T.totals, s);
   k_topo_fill<<<blocks_for(nf, 256), 256, 0, s>>>(F, nf, nv, T.raw_off, T.cursor, T.raw);
   k_topo_dedupe<<<blocks_for(nv, 128), 128, 0, s>>>(nv, T.raw_off, T.raw_cnt, T.raw, T.hdr);
   // distinct counts -> row starts (the cursor array, free now, holds the scan)
   cudaMemcpyAsync(T.cursor, T.raw_cnt, (size_t)nv * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s);
-  launch_scan_exclusive(T.cursor, nv, s);
+  launch_scan_exclusive(T.cursor, T.cursor, nv, T.totals, s);
   k_topo_compact<<<blocks_for(nv, 256), 256, 0, s>>>(nv, T.raw_off, T.raw_cnt, T.cursor, T.raw, T.row, T.col,
                                                       T.hdr);
 }
