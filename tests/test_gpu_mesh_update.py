@@ -134,3 +134,21 @@ def test_large_steps_update_in_a_graph():
     torch.cuda.synchronize()
     assert torch.equal(Va, Vb)
     assert (Va - torch.from_numpy(V).cuda()).abs().max() > 1e-4
+
+
+@pytest.mark.parametrize("nv,nf", [(3, 1), (17, 40), (700, 900), (700, 1900), (700, 6000), (5000, 30000)])
+def test_topology_of_random_triangles(nv, nf):
+    """Lists below, at and above a group's 16 entries, with repeats, repeated
+    vertices and vertices of no triangle."""
+    F = np.random.default_rng(nf).integers(0, nv, (nf, 3)).astype(np.int32)
+    topo = dt.Topology(torch.from_numpy(F).cuda(), nv)
+    ne, md, row, col = topo.info()
+    row, col = row.cpu().numpy(), col.cpu().numpy()
+    E = {(int(a), int(b)) for t in F for a in t for b in t if a != b}
+    assert 2 * ne == len(E) == row[-1]
+    assert md == np.diff(row).max()
+    for v in range(nv):
+        got = col[row[v]:row[v + 1]]
+        assert (np.diff(got) > 0).all()  # sorted, distinct
+    src = np.repeat(np.arange(nv), np.diff(row))
+    assert {(int(a), int(b)) for a, b in zip(src, col)} == E
