@@ -60,3 +60,20 @@ def test_paper_loss_seeds_the_backward():
     gref[bad] = 0.0
     J = np.einsum("khwc,hwc->k", dI, gref)
     np.testing.assert_allclose(dsig, J, rtol=GRAD_RTOL, atol=1e-6 * max(1e-3, np.abs(J).max()))
+
+
+@pytest.mark.parametrize("off", [0, 1, 3])
+@pytest.mark.parametrize("n", [1, 3, 4, 5, 1023, 4096, 1300003])
+def test_paper_loss_sizes_and_alignment(n, off):
+    """Every remainder of the four-pixel words, and arrays that start off a
+    16-byte boundary, against the oracle."""
+    rng = np.random.default_rng(n)
+    a, b = rng.uniform(0.05, 1.5, size=(2, n, 3)).astype(np.float32)
+    ta, tb, tg = (torch.empty(3 * n + off, device="cuda")[off:].view(n, 3) for _ in range(3))
+    ta.copy_(torch.from_numpy(a))
+    tb.copy_(torch.from_numpy(b))
+    g, loss = dt.paper_loss_grad(ta, tb, 0.6, 1.4, grad=tg)
+    assert g.data_ptr() == tg.data_ptr()
+    total, lc, lt, gref = O.paper_losses(a.astype(np.float64)[None], b.astype(np.float64)[None], 0.6, 1.4)
+    np.testing.assert_allclose(loss.cpu().numpy(), [total, lc, lt], rtol=2e-5, atol=2e-6)
+    np.testing.assert_allclose(g.cpu().numpy(), gref[0], rtol=2e-5, atol=1e-6 * np.abs(gref).max())
