@@ -47,80 +47,6 @@ __device__ __forceinline__ MediumView medium_view(const SceneEntry& E, const Sce
                     mk(E.gscale_x, E.gscale_y, E.gscale_z), E.gstep, E.glevels, Eg->glev};
 }
 
-// Cell of x: per axis u = (x - lo) scale clamped to [0, n - 1], cell index
-// min(floor(u), n - 2) and fraction u - index; `free` = the axis was not
-// clamped (a clamped coordinate is constant, so it has no derivative).
-struct GridCell {
-  size_t base;             // node index of the cell's (0, 0, 0) corner
-  int sx, sy;              // node index strides along y and z (nx, nx ny)
-  float fx, fy, fz;
-  bool free_x, free_y, free_z;
-};
-
-__device__ __forceinline__ float grid_axis(float x, float lo, float scale, int n, int& i, bool& free) {
-  float u = (x - lo) * scale;
-  const float top = (float)(n - 1);
-  free = u >= 0.0f && u <= top;
-  u = fminf(fmaxf(u, 0.0f), top);
-  i = min((int)u, n - 2);
-  return u - (float)i;
-}
-
-__device__ __forceinline__ GridCell grid_cell(const MediumView& g, float3 x) {
-  GridCell c;
-  int i, j, k;
-  c.fx = grid_axis(x.x, g.lo.x, g.scale.x, g.nx, i, c.free_x);
-  c.fy = grid_axis(x.y, g.lo.y, g.scale.y, g.ny, j, c.free_y);
-  c.fz = grid_axis(x.z, g.lo.z, g.scale.z, g.nz, k, c.free_z);
-  c.sx = g.nx;
-  c.sy = g.nx * g.ny;
-  c.base = ((uint32_t)k * (uint32_t)g.ny + (uint32_t)j) * (uint32_t)g.nx + (uint32_t)i;  // < 2^31 nodes (checked)
-  return c;
-}
-
-// The eight corner values of a cell (xyz of the float4 nodes).
-struct CellNodes {
-  float3 c000, c100, c010, c110, c001, c101, c011, c111;
-};
-
-__device__ __forceinline__ CellNodes cell_nodes(const MediumView& g, const GridCell& c) {
-  const float4* p = g.mu + c.base;
-  CellNodes q;
-  q.c000 = xyz(__ldg(p));
-  q.c100 = xyz(__ldg(p + 1));
-  q.c010 = xyz(__ldg(p + c.sx));
-  q.c110 = xyz(__ldg(p + c.sx + 1));
-  q.c001 = xyz(__ldg(p + c.sy));
-  q.c101 = xyz(__ldg(p + c.sy + 1));
-  q.c011 = xyz(__ldg(p + c.sy + c.sx));
-  q.c111 = xyz(__ldg(p + c.sy + c.sx + 1));
-  return q;
-}
-
-__device__ __forceinline__ float3 lerp3(float3 a, float3 b, float f) { return a + (b - a) * f; }
-
-// G at the cell position.
-template <class Cell>
-__device__ __forceinline__ float3 trilinear(const CellNodes& q, const Cell& c) {
-  const float3 x00 = lerp3(q.c000, q.c100, c.fx), x10 = lerp3(q.c010, q.c110, c.fx);
-  const float3 x01 = lerp3(q.c001, q.c101, c.fx), x11 = lerp3(q.c011, q.c111, c.fx);
-  return lerp3(lerp3(x00, x10, c.fy), lerp3(x01, x11, c.fy), c.fz);
-}
-
-// dG_c/dx_a for the three channels c: columns gx, gy, gz (each a float3 over
-// the channels), zero along clamped axes.
-template <class Cell>
-__device__ __forceinline__ void trilinear_grad(const CellNodes& q, const Cell& c, float3 scale, float3& gx,
-                                               float3& gy, float3& gz) {
-  const float ux = 1.0f - c.fx, uy = 1.0f - c.fy, uz = 1.0f - c.fz;
-  gx = ((q.c100 - q.c000) * (uy * uz) + (q.c110 - q.c010) * (c.fy * uz) + (q.c101 - q.c001) * (uy * c.fz) +
-        (q.c111 - q.c011) * (c.fy * c.fz)) * (c.free_x ? scale.x : 0.0f);
-  gy = ((q.c010 - q.c000) * (ux * uz) + (q.c110 - q.c100) * (c.fx * uz) + (q.c011 - q.c001) * (ux * c.fz) +
-        (q.c111 - q.c101) * (c.fx * c.fz)) * (c.free_y ? scale.y : 0.0f);
-  gz = ((q.c001 - q.c000) * (ux * uy) + (q.c101 - q.c100) * (c.fx * uy) + (q.c011 - q.c010) * (ux * c.fy) +
-        (q.c111 - q.c110) * (c.fx * c.fy)) * (c.free_z ? scale.z : 0.0f);
-}
-
 // Number of full steps of a segment of length t.
 __device__ __forceinline__ int medium_full_steps(float t, float h) {
   const float m = floorf(t / h);
@@ -128,75 +54,25 @@ __device__ __forceinline__ int medium_full_steps(float t, float h) {
   return m >= (float)kMaxMediumSteps ? kMaxMediumSteps : (int)m;
 }
 
+// A segment's steps: sample i < m at the middle of full step i, sample m at the
+// middle of the last one, of length r.
+struct MediumSteps {
+  float h, r;
+  int m;
+  __device__ __forceinline__ MediumSteps(float t, float step) : h(step), m(medium_full_steps(t, step)) { r = t - (float)m * h; }
+  __device__ __forceinline__ float weight(int i) const { return i < m ? h : r; }
+  __device__ __forceinline__ float place(int i) const {
+    return i < m ? ((float)i + 0.5f) * h : (float)m * h + 0.5f * r;
+  }
+};
+
 // ---------------------------------------------------------------------------
-// hash texture
+// lattices
 // ---------------------------------------------------------------------------
 // Instant-NGP's spatial hash of a lattice point (Mueller et al. 2022, Eq. 4
 // with d = 3): XOR of the coordinates times 1, 2654435761 and 805459861 in
 // 32-bit arithmetic; the level keeps its low bits (tables are powers of two).
 constexpr uint32_t kHashPrimeY = 2654435761u, kHashPrimeZ = 805459861u;
-
-// A level's cell containing x: fractions and clamping as grid_cell, and the
-// lattice coordinates of its (0, 0, 0) corner.
-struct LevelCell {
-  uint32_t i, j, k;
-  float fx, fy, fz;
-  bool free_x, free_y, free_z;
-};
-
-__device__ __forceinline__ LevelCell level_cell(const GridLevel& L, float3 lo, float3 x) {
-  LevelCell c;
-  int i, j, k;
-  c.fx = grid_axis(x.x, lo.x, L.sx, L.n, i, c.free_x);
-  c.fy = grid_axis(x.y, lo.y, L.sy, L.n, j, c.free_y);
-  c.fz = grid_axis(x.z, lo.z, L.sz, L.n, k, c.free_z);
-  c.i = (uint32_t)i;
-  c.j = (uint32_t)j;
-  c.k = (uint32_t)k;
-  return c;
-}
-
-// The table entries of the eight corners of a level's cell at lattice point
-// (i, j, k), corner q = (i + (q & 1), j + ((q >> 1) & 1), k + (q >> 2)):
-// the level's first entry plus, when the lattice fits the table, the dense
-// index (k n + j) n + i (so the corners add 0, 1, n, n + 1, n^2, ...), else
-// the spatial hash masked to the table, with the per-axis terms formed once
-// ((j + 1) kHashPrimeY = j kHashPrimeY + kHashPrimeY in 32-bit arithmetic,
-// likewise for k), so each corner is one three-way XOR, a mask and an add.
-__device__ __forceinline__ void level_corner_entries(const GridLevel& L, const LevelCell& c, size_t (&e)[8]) {
-  if (L.mask) {
-    const uint32_t x0 = c.i, x1 = c.i + 1u;
-    const uint32_t y0 = c.j * kHashPrimeY, y1 = y0 + kHashPrimeY;
-    const uint32_t z0 = c.k * kHashPrimeZ, z1 = z0 + kHashPrimeZ;
-    e[0] = L.off + ((x0 ^ y0 ^ z0) & L.mask);
-    e[1] = L.off + ((x1 ^ y0 ^ z0) & L.mask);
-    e[2] = L.off + ((x0 ^ y1 ^ z0) & L.mask);
-    e[3] = L.off + ((x1 ^ y1 ^ z0) & L.mask);
-    e[4] = L.off + ((x0 ^ y0 ^ z1) & L.mask);
-    e[5] = L.off + ((x1 ^ y0 ^ z1) & L.mask);
-    e[6] = L.off + ((x0 ^ y1 ^ z1) & L.mask);
-    e[7] = L.off + ((x1 ^ y1 ^ z1) & L.mask);
-  } else {
-    const uint32_t n = (uint32_t)L.n, b = L.off + (c.k * n + c.j) * n + c.i, nn = n * n;
-    e[0] = b; e[1] = b + 1u; e[2] = b + n; e[3] = b + n + 1u;
-    e[4] = b + nn; e[5] = b + nn + 1u; e[6] = b + nn + n; e[7] = b + nn + n + 1u;
-  }
-}
-
-__device__ __forceinline__ CellNodes level_nodes(const float4* mu, const GridLevel& L, const LevelCell& c) {
-  size_t e[8];
-  level_corner_entries(L, c, e);
-  CellNodes q;
-  q.c000 = xyz(__ldg(mu + e[0]));
-  q.c100 = xyz(__ldg(mu + e[1]));
-  q.c010 = xyz(__ldg(mu + e[2]));
-  q.c110 = xyz(__ldg(mu + e[3]));
-  q.c001 = xyz(__ldg(mu + e[4]));
-  q.c101 = xyz(__ldg(mu + e[5]));
-  q.c011 = xyz(__ldg(mu + e[6]));
-  q.c111 = xyz(__ldg(mu + e[7]));
-  return q;
-}
 
 __device__ __forceinline__ GridLevel load_level(const GridLevel* p) {
   GridLevel L;
@@ -212,152 +88,350 @@ __device__ __forceinline__ GridLevel load_level(const GridLevel* p) {
   return L;
 }
 
-// Optical depth of the hash texture over o + s d, s in [0, t]: the steps of
-// medium_depth, level by level.
-__device__ __forceinline__ float3 hash_depth(const MediumView& g, float3 o, float3 d, float t) {
-  const float h = g.step;
-  const int m = medium_full_steps(t, h);
-  const float r = t - (float)m * h;
-  float3 sum = mk(0.f, 0.f, 0.f);
-  for (int l = 0; l < g.levels; ++l) {
+// One lattice (the dense grid, or a level of the hash texture) along one
+// segment: the sample at s is at the lattice position u0 + s du, one fused
+// multiply-add per axis.
+struct Lattice {
+  float3 scale, u0, du;
+  int nx, ny, nz;
+  uint32_t off, mask;  // first entry; hashed level: entries - 1 (0: dense index (k ny + j) nx + i)
+};
+
+template <bool kHash>
+__device__ __forceinline__ Lattice lattice_of(const MediumView& g, int l, float3 o, float3 d) {
+  Lattice T;
+  if (kHash && g.levels) {
     const GridLevel L = load_level(g.lev + l);
-    for (int i = 0; i <= m; ++i) {
-      const float w = i < m ? h : r;
-      const float s = i < m ? ((float)i + 0.5f) * h : (float)m * h + 0.5f * r;
-      const LevelCell c = level_cell(L, g.lo, o + d * s);
-      sum = sum + trilinear(level_nodes(g.mu, L, c), c) * w;
-    }
+    T.scale = mk(L.sx, L.sy, L.sz);
+    T.nx = T.ny = T.nz = L.n;
+    T.off = L.off;
+    T.mask = L.mask;
+  } else {
+    T.scale = g.scale;
+    T.nx = g.nx;
+    T.ny = g.ny;
+    T.nz = g.nz;
+    T.off = T.mask = 0u;
+  }
+  T.u0 = mul(o - g.lo, T.scale);
+  T.du = mul(d, T.scale);
+  return T;
+}
+
+// Whether the segment stays inside the lattice's box (an object's box usually
+// holds it whole): its samples then need no clamping.  The margin, 1/64 of a
+// cell or a millionth of the lattice where that is more, is above the rounding
+// of a position.
+__device__ __forceinline__ bool lattice_inside(const Lattice& T, float t) {
+  auto in = [&](float u0, float du, int n) {
+    const float u1 = fmaf(t, du, u0), e = fmaxf(0.015625f, (float)n * 1e-6f);
+    return fminf(u0, u1) >= e && fmaxf(u0, u1) <= (float)(n - 1) - e;
+  };
+  return in(T.u0.x, T.du.x, T.nx) && in(T.u0.y, T.du.y, T.ny) && in(T.u0.z, T.du.z, T.nz);
+}
+
+// The cell of a sample: per axis u clamped to [0, n - 1], cell index
+// min(floor(u), n - 2) and fraction u - index; `free` = the axis was not
+// clamped (a clamped coordinate is constant, so it has no derivative).
+// kInside: known to need no clamping.
+struct LatticeCell {
+  int i, j, k;
+  float fx, fy, fz;
+  bool free_x, free_y, free_z;
+};
+
+template <bool kInside>
+__device__ __forceinline__ float lattice_axis(float u, int n, int& i, bool& free) {
+  if (kInside) {
+    const float f = floorf(u);
+    i = (int)f;
+    free = true;
+    return u - f;
+  }
+  const float top = (float)(n - 1);
+  free = u >= 0.0f && u <= top;
+  u = fminf(fmaxf(u, 0.0f), top);
+  i = min((int)u, n - 2);
+  return u - (float)i;
+}
+
+template <bool kInside>
+__device__ __forceinline__ LatticeCell lattice_cell(const Lattice& T, float s) {
+  LatticeCell c;
+  c.fx = lattice_axis<kInside>(fmaf(s, T.du.x, T.u0.x), T.nx, c.i, c.free_x);
+  c.fy = lattice_axis<kInside>(fmaf(s, T.du.y, T.u0.y), T.ny, c.j, c.free_y);
+  c.fz = lattice_axis<kInside>(fmaf(s, T.du.z, T.u0.z), T.nz, c.k, c.free_z);
+  return c;
+}
+
+// The entries of the lattice points (x0 or x1, y0 or y1, z0 or z1), entry q
+// taking x1 for bit 0 of q, y1 for bit 1, z1 for bit 2; the per-axis terms are
+// formed once, so an entry is a three-way XOR, a mask and an add, or two adds.
+__device__ __forceinline__ void lattice_entries(const Lattice& T, uint32_t x0, uint32_t x1, uint32_t y0, uint32_t y1,
+                                                uint32_t z0, uint32_t z1, uint32_t (&e)[8]) {
+  if (T.mask) {
+    y0 *= kHashPrimeY; y1 *= kHashPrimeY;
+    z0 *= kHashPrimeZ; z1 *= kHashPrimeZ;
+    const uint32_t a = y0 ^ z0, b = y1 ^ z0, c = y0 ^ z1, d = y1 ^ z1;
+    e[0] = T.off + ((x0 ^ a) & T.mask); e[1] = T.off + ((x1 ^ a) & T.mask);
+    e[2] = T.off + ((x0 ^ b) & T.mask); e[3] = T.off + ((x1 ^ b) & T.mask);
+    e[4] = T.off + ((x0 ^ c) & T.mask); e[5] = T.off + ((x1 ^ c) & T.mask);
+    e[6] = T.off + ((x0 ^ d) & T.mask); e[7] = T.off + ((x1 ^ d) & T.mask);
+  } else {
+    const uint32_t nx = (uint32_t)T.nx, ny = (uint32_t)T.ny;
+    const uint32_t a = T.off + (z0 * ny + y0) * nx, b = T.off + (z0 * ny + y1) * nx;
+    const uint32_t c = T.off + (z1 * ny + y0) * nx, d = T.off + (z1 * ny + y1) * nx;
+    e[0] = a + x0; e[1] = a + x1; e[2] = b + x0; e[3] = b + x1;
+    e[4] = c + x0; e[5] = c + x1; e[6] = d + x0; e[7] = d + x1;
+  }
+}
+
+// The eight corner values of a cell (xyz of the float4 entries).
+struct CellNodes {
+  float3 c000, c100, c010, c110, c001, c101, c011, c111;
+};
+
+__device__ __forceinline__ CellNodes cell_nodes(const float4* __restrict__ mu, const Lattice& T, const LatticeCell& c) {
+  const uint32_t i = (uint32_t)c.i, j = (uint32_t)c.j, k = (uint32_t)c.k;
+  uint32_t e[8];
+  lattice_entries(T, i, i + 1u, j, j + 1u, k, k + 1u, e);
+  CellNodes q;
+  q.c000 = xyz(__ldg(mu + e[0]));
+  q.c100 = xyz(__ldg(mu + e[1]));
+  q.c010 = xyz(__ldg(mu + e[2]));
+  q.c110 = xyz(__ldg(mu + e[3]));
+  q.c001 = xyz(__ldg(mu + e[4]));
+  q.c101 = xyz(__ldg(mu + e[5]));
+  q.c011 = xyz(__ldg(mu + e[6]));
+  q.c111 = xyz(__ldg(mu + e[7]));
+  return q;
+}
+
+// G and its gradient (dG_c/dx_a for the three channels c: columns gx, gy, gz,
+// zero along clamped axes), sharing the interpolation's intermediate values:
+// the differences along x feed both the x interpolations and dG/dx, the
+// differences of the x-interpolated values along y feed the y interpolations
+// and dG/dy, and the difference of the two y-interpolated values along z gives
+// G and dG/dz.
+__device__ __forceinline__ float3 trilinear_value_grad(const CellNodes& q, const LatticeCell& c, float3 scale,
+                                                       float3& gx, float3& gy, float3& gz) {
+  const float3 a00 = q.c100 - q.c000, a10 = q.c110 - q.c010, a01 = q.c101 - q.c001, a11 = q.c111 - q.c011;
+  const float3 x00 = q.c000 + a00 * c.fx, x10 = q.c010 + a10 * c.fx;
+  const float3 x01 = q.c001 + a01 * c.fx, x11 = q.c011 + a11 * c.fx;
+  const float3 b0 = x10 - x00, b1 = x11 - x01;
+  const float3 y0 = x00 + b0 * c.fy, y1 = x01 + b1 * c.fy;
+  const float3 e = y1 - y0;
+  const float3 ax0 = a00 + (a10 - a00) * c.fy, ax1 = a01 + (a11 - a01) * c.fy;
+  gx = (ax0 + (ax1 - ax0) * c.fz) * (c.free_x ? scale.x : 0.0f);
+  gy = (b0 + (b1 - b0) * c.fz) * (c.free_y ? scale.y : 0.0f);
+  gz = e * (c.free_z ? scale.z : 0.0f);
+  return y0 + e * c.fz;
+}
+
+// ---------------------------------------------------------------------------
+// optical depth
+// ---------------------------------------------------------------------------
+// Samples p, p + lanes, ... of one lattice: each adds its weight times G, as
+// eight products of the corner values.
+template <bool kInside>
+__device__ __forceinline__ void depth_walk(const float4* __restrict__ mu, const Lattice& T, const MediumSteps& st, int p,
+                                           int lanes, float3& sum) {
+  for (int i = p; i <= st.m; i += lanes) {
+    const LatticeCell c = lattice_cell<kInside>(T, st.place(i));
+    const CellNodes q = cell_nodes(mu, T, c);
+    const float w = st.weight(i), ux = 1.0f - c.fx, uy = 1.0f - c.fy, wz = w * c.fz, uz = w - wz;
+    const float a = ux * uy, b = c.fx * uy, d = ux * c.fy, e = c.fx * c.fy;
+    sum = sum + q.c000 * (a * uz) + q.c100 * (b * uz) + q.c010 * (d * uz) + q.c110 * (e * uz) + q.c001 * (a * wz) +
+          q.c101 * (b * wz) + q.c011 * (d * wz) + q.c111 * (e * wz);
+  }
+}
+
+// The part of the optical depth over o + s d, s in [0, t], that lane p of
+// `lanes` sums: the samples p, p + lanes, ..., of every level of the hash
+// texture, or of the dense grid (kHash: the scene may hold a hash texture;
+// without it that code is not compiled).
+template <bool kHash>
+__device__ __forceinline__ float3 medium_depth_part(const MediumView& g, float3 o, float3 d, float t, int p, int lanes) {
+  const MediumSteps st(t, g.step);
+  float3 sum = mk(0.f, 0.f, 0.f);
+  const int levels = kHash && g.levels ? g.levels : 1;
+  for (int l = 0; l < levels; ++l) {
+    const Lattice T = lattice_of<kHash>(g, l, o, d);
+    // one copy of the loop for a warp, whichever its lanes need
+    if (__all_sync(__activemask(), lattice_inside(T, t))) depth_walk<true>(g.mu, T, st, p, lanes, sum);
+    else depth_walk<false>(g.mu, T, st, p, lanes, sum);
   }
   return sum;
 }
 
-__device__ __forceinline__ float3 hash_depth_dt(const MediumView& g, float3 o, float3 d, float t) {
-  const float h = g.step;
-  const int m = medium_full_steps(t, h);
-  const float r = t - (float)m * h;
-  const float3 x = o + d * ((float)m * h + 0.5f * r);
-  float3 sum = mk(0.f, 0.f, 0.f);
-  for (int l = 0; l < g.levels; ++l) {
-    const GridLevel L = load_level(g.lev + l);
-    const LevelCell c = level_cell(L, g.lo, x);
-    const CellNodes q = level_nodes(g.mu, L, c);
-    float3 gx, gy, gz;
-    trilinear_grad(q, c, mk(L.sx, L.sy, L.sz), gx, gy, gz);
-    sum = sum + trilinear(q, c) + (gx * d.x + gy * d.y + gz * d.z) * (0.5f * r);
-  }
-  return sum;
-}
-
-// Optical depth of the grid over o + s d, s in [0, t] (kHash: the scene may
-// hold a hash texture instead; without it that code is not compiled).
+// Optical depth over o + s d, s in [0, t].
 template <bool kHash>
 __device__ __forceinline__ float3 medium_depth(const MediumView& g, float3 o, float3 d, float t) {
-  if (kHash && g.levels) return hash_depth(g, o, d, t);
-  const float h = g.step;
-  const int m = medium_full_steps(t, h);
-  float3 sum = mk(0.f, 0.f, 0.f);
-  for (int i = 0; i < m; ++i) {
-    const GridCell c = grid_cell(g, o + d * (((float)i + 0.5f) * h));
-    sum = sum + trilinear(cell_nodes(g, c), c) * h;
-  }
-  const float r = t - (float)m * h;
-  const GridCell c = grid_cell(g, o + d * ((float)m * h + 0.5f * r));
-  return sum + trilinear(cell_nodes(g, c), c) * r;
+  return medium_depth_part<kHash>(g, o, d, t, 0, 1);
 }
 
 // dS/dt per channel (only the partial last step depends on t).
 template <bool kHash>
 __device__ __forceinline__ float3 medium_depth_dt(const MediumView& g, float3 o, float3 d, float t) {
-  if (kHash && g.levels) return hash_depth_dt(g, o, d, t);
-  const float h = g.step;
-  const int m = medium_full_steps(t, h);
-  const float r = t - (float)m * h;
-  const GridCell c = grid_cell(g, o + d * ((float)m * h + 0.5f * r));
-  const CellNodes q = cell_nodes(g, c);
-  float3 gx, gy, gz;
-  trilinear_grad(q, c, g.scale, gx, gy, gz);
-  return trilinear(q, c) + (gx * d.x + gy * d.y + gz * d.z) * (0.5f * r);
+  const MediumSteps st(t, g.step);
+  float3 sum = mk(0.f, 0.f, 0.f);
+  const int levels = kHash && g.levels ? g.levels : 1;
+  for (int l = 0; l < levels; ++l) {
+    const Lattice T = lattice_of<kHash>(g, l, o, d);
+    const LatticeCell c = lattice_cell<false>(T, st.place(st.m));
+    float3 gx, gy, gz;
+    const float3 G = trilinear_value_grad(cell_nodes(g.mu, T, c), c, T.scale, gx, gy, gz);
+    sum = sum + G + (gx * d.x + gy * d.y + gz * d.z) * (0.5f * st.r);
+  }
+  return sum;
 }
 
-// One 128-bit vector atomic per node (w unused).
-__device__ __forceinline__ void medium_atomic4(float4* p, float3 v) {
-  atomicAdd(p, make_float4(v.x, v.y, v.z, 0.f));
+// ---------------------------------------------------------------------------
+// march tiles
+// ---------------------------------------------------------------------------
+// The segments of a level that march the medium are some of its segments, of
+// lengths from nothing to the object's diameter: 32 neighbours marched by a
+// warp as they come leave two thirds of its lanes idle.  A CTA therefore takes a
+// tile of the level's positions, lists those that march in shared memory by
+// falling number of steps (a counting sort), and its warps take units of
+// listed segments of nearly equal length, the longest first: 32 segments on one
+// level of the texture for the adjoint, whose walks run along a segment, or
+// eight segments with four lanes each for the forward passes, whose samples are
+// independent (neighbouring samples read the same cells, so the four lanes
+// share their reads as well).
+constexpr int kTileThreads = 256;
+constexpr int kTileMax = 512;  // positions
+constexpr int kTileKeys = 128;
+constexpr int kPartSteps = 16;
+
+struct MarchTile {
+  uint32_t pos[kTileMax];
+  int hist[kTileKeys];
+  int n, levels, next;
+  int parts;  // of the longest listed segment
+};
+
+// Key of a segment of m full steps: m itself below 64, then eight per octave.
+__device__ __forceinline__ int march_key(int m) {
+  if (m < 64) return m;
+  const int e = 31 - __clz(m);  // >= 6; m <= 8192
+  return min(kTileKeys - 1, 64 + 8 * (e - 6) + ((m >> (e - 3)) & 7));
 }
 
-template <bool kHash>
-__device__ __forceinline__ void medium_scatter(const MediumView& g, float4* dmu, float3 o, float3 d, float t,
-                                               float3 sbar);
+// Positions per tile for a level of n: 512, or 256 where the level would not
+// fill the CTAs four times over.
+__device__ __forceinline__ uint32_t march_tile(uint32_t n, uint32_t ctas) {
+  return n >= 4u * kTileMax * ctas ? (uint32_t)kTileMax : kTileMax / 2u;
+}
 
-// The samples' share of the adjoint of hash_depth, level by level: per
-// sample the gradient of sbar . G_l from sbar . (corner values).
-__device__ __forceinline__ void hash_backward(const MediumView& g, float3 o, float3 d, float t, float3 sbar,
-                                              float3& obar, float3& dbar) {
-  const float h = g.step;
-  const int m = medium_full_steps(t, h);
-  const float r = t - (float)m * h;
-  for (int l = 0; l < g.levels; ++l) {
-    const GridLevel L = load_level(g.lev + l);
-    for (int i = 0; i <= m; ++i) {
-      const float w = i < m ? h : r;
-      const float s = i < m ? ((float)i + 0.5f) * h : (float)m * h + 0.5f * r;
-      const LevelCell c = level_cell(L, g.lo, o + d * s);
-      float sv[8];  // sbar . G at the eight corners
-      size_t e[8];
-      level_corner_entries(L, c, e);
+// Lists the positions [first, first + size) with steps(i, levels) >= 0 (levels:
+// the lattices the position marches) by falling key.  By the whole CTA; the
+// list may be read on return.
+template <class Steps>
+__device__ __forceinline__ void march_list(MarchTile& T, uint32_t first, uint32_t size, const Steps& steps) {
+  constexpr int kPer = kTileMax / kTileThreads;
+  for (int i = threadIdx.x; i < kTileKeys; i += kTileThreads) T.hist[i] = 0;
+  if (threadIdx.x == 0) T.levels = T.next = T.parts = 0;
+  __syncthreads();
+  int key[kPer], rank[kPer], most = 0, parts = 0;
 #pragma unroll
-      for (int q = 0; q < 8; ++q) sv[q] = dot(sbar, xyz(__ldg(g.mu + e[q])));
-      const float ux = 1.0f - c.fx, uy = 1.0f - c.fy, uz = 1.0f - c.fz;
-      const float3 gp =
-          mk(((sv[1] - sv[0]) * (uy * uz) + (sv[3] - sv[2]) * (c.fy * uz) + (sv[5] - sv[4]) * (uy * c.fz) +
-              (sv[7] - sv[6]) * (c.fy * c.fz)) * (c.free_x ? L.sx : 0.0f),
-             ((sv[2] - sv[0]) * (ux * uz) + (sv[3] - sv[1]) * (c.fx * uz) + (sv[6] - sv[4]) * (ux * c.fz) +
-              (sv[7] - sv[5]) * (c.fx * c.fz)) * (c.free_y ? L.sy : 0.0f),
-             ((sv[4] - sv[0]) * (ux * uy) + (sv[5] - sv[1]) * (c.fx * uy) + (sv[6] - sv[2]) * (ux * c.fy) +
-              (sv[7] - sv[3]) * (c.fx * c.fy)) * (c.free_z ? L.sz : 0.0f)) * w;
-      obar = obar + gp;
-      dbar = dbar + gp * s;
+  for (int j = 0; j < kPer; ++j) {
+    key[j] = -1;
+    const uint32_t p = j * kTileThreads + threadIdx.x;
+    if (p >= size) continue;
+    int levels = 0;
+    const int m = steps(first + p, levels);
+    if (m < 0) continue;
+    key[j] = march_key(m);
+    rank[j] = atomicAdd(&T.hist[key[j]], 1);
+    most = max(most, levels);
+    parts = max(parts, m / kPartSteps + 1);
+  }
+  most = __reduce_max_sync(kFull, most);
+  parts = __reduce_max_sync(kFull, parts);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMax(&T.levels, most);
+    atomicMax(&T.parts, parts);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {  // counts -> starts, from the longest down
+    const int k0 = kTileKeys - 1 - 4 * (int)threadIdx.x;
+    int c[4], sum = 0;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      c[q] = T.hist[k0 - q];
+      sum += c[q];
+    }
+    int x = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(kFull, x, o);
+      if ((int)threadIdx.x >= o) x += y;
+    }
+    if (threadIdx.x == 31) T.n = x;
+    x -= sum;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      T.hist[k0 - q] = x;
+      x += c[q];
     }
   }
+  __syncthreads();
+#pragma unroll
+  for (int j = 0; j < kPer; ++j)
+    if (key[j] >= 0) T.pos[T.hist[key[j]] + rank[j]] = first + j * kTileThreads + threadIdx.x;
+  __syncthreads();
 }
 
-// Adjoint of the optical depth at fixed t: sbar = dJ/dS (per channel, one
-// value for the whole segment).  Adds dJ/do and dJ/dd to obar and dbar
-// (the samples move with o and d; the gradient of sbar . G needs only sbar .
-// G at each sample's corners) and, when dmu is given, dJ/dG at the nodes or
-// entries (medium_scatter).
+// The warp's next unit of the forward passes: a listed segment's index for each
+// group of kLanes lanes (T.n and above: none); false when the list is done.
+// Lanes per segment: of the depth march (hash texture, 8 views of 360x360: 7.7,
+// 6.0 and 5.9 ms of shading with 2, 4 and 8; with 8 the dense grid's takes 7 %
+// more), and of the moments', whose 24 sums are added up across the lanes (dense
+// grid, 16 views of 384x384: 1.87, 1.51 and 1.66 ms with 1, 2 and 4; hash texture
+// 16.0, 9.75 and 7.05 ms).
+constexpr int kDepthLanes = 4;
 template <bool kHash>
-__device__ __forceinline__ void medium_backward(const MediumView& g, float4* dmu, float3 o, float3 d, float t,
-                                                float3 sbar, float3& obar, float3& dbar) {
-  if (kHash && g.levels) {
-    hash_backward(g, o, d, t, sbar, obar, dbar);
-  } else {
-    const float h = g.step;
-    const int m = medium_full_steps(t, h);
-    const float r = t - (float)m * h;
-    const int sx = g.nx, sy = g.nx * g.ny;
-    for (int i = 0; i <= m; ++i) {
-      const float w = i < m ? h : r;
-      const float s = i < m ? ((float)i + 0.5f) * h : (float)m * h + 0.5f * r;
-      const GridCell c = grid_cell(g, o + d * s);
-      const float4* p = g.mu + c.base;
-      // sbar . G at the eight corners
-      const float s000 = dot(sbar, xyz(__ldg(p))), s100 = dot(sbar, xyz(__ldg(p + 1)));
-      const float s010 = dot(sbar, xyz(__ldg(p + sx))), s110 = dot(sbar, xyz(__ldg(p + sx + 1)));
-      const float s001 = dot(sbar, xyz(__ldg(p + sy))), s101 = dot(sbar, xyz(__ldg(p + sy + 1)));
-      const float s011 = dot(sbar, xyz(__ldg(p + sy + sx))), s111 = dot(sbar, xyz(__ldg(p + sy + sx + 1)));
-      const float ux = 1.0f - c.fx, uy = 1.0f - c.fy, uz = 1.0f - c.fz;
-      const float3 gp =
-          mk(((s100 - s000) * (uy * uz) + (s110 - s010) * (c.fy * uz) + (s101 - s001) * (uy * c.fz) +
-              (s111 - s011) * (c.fy * c.fz)) * (c.free_x ? g.scale.x : 0.0f),
-             ((s010 - s000) * (ux * uz) + (s110 - s100) * (c.fx * uz) + (s011 - s001) * (ux * c.fz) +
-              (s111 - s101) * (c.fx * c.fz)) * (c.free_y ? g.scale.y : 0.0f),
-             ((s001 - s000) * (ux * uy) + (s101 - s100) * (c.fx * uy) + (s011 - s010) * (ux * c.fy) +
-              (s111 - s110) * (c.fx * c.fy)) * (c.free_z ? g.scale.z : 0.0f)) * w;  // w dJ/dx at this sample
-      obar = obar + gp;
-      dbar = dbar + gp * s;
-    }
+constexpr int kMomentLanes = kHash ? 4 : 2;
+template <int kLanes>
+__device__ __forceinline__ bool march_group(MarchTile& T, int& index) {
+  int u = 0;
+  if ((threadIdx.x & 31) == 0) u = atomicAdd(&T.next, 32 / kLanes);
+  u = __shfl_sync(kFull, u, 0);
+  index = u + (int)(threadIdx.x & 31) / kLanes;
+  return u < T.n;
+}
+// The sum of v over the lanes of a group (in every lane of it).
+template <int kLanes>
+__device__ __forceinline__ float group_sum(float v) {
+#pragma unroll
+  for (int o = 1; o < kLanes; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+
+// The warp's next unit of the adjoint: a listed segment's index for each lane
+// (T.n and above: none), a level and a part of the samples; false when the list
+// is done.  With few levels a tile has about as many chunks of 32 segments as
+// the CTA has warps, the longest many times the shortest, and the warps would
+// wait for the longest: its walks are cut into parts of kPartSteps samples
+// (each ends with its eight corners' atomics).
+constexpr int kPartLevels = 2;  // levels up to which walks are cut
+__device__ __forceinline__ bool march_unit(MarchTile& T, int& index, int& level, int& part) {
+  int u = 0;
+  if ((threadIdx.x & 31) == 0) u = atomicAdd(&T.next, 1);
+  u = __shfl_sync(kFull, u, 0);
+  const int levels = max(T.levels, 1), chunks = (T.n + 31) / 32;
+  level = levels - 1 - u % levels;
+  const int v = u / levels;
+  part = 0;
+  int chunk = v;
+  if (levels <= kPartLevels && chunks > 0) {
+    part = v / chunks;
+    chunk = v % chunks;
+    if (part >= T.parts) return false;
   }
-  if (dmu) medium_scatter<kHash>(g, dmu, o, d, t, sbar);
+  index = chunk * 32 + (int)(threadIdx.x & 31);
+  return chunk < chunks;
 }
 
 // ---------------------------------------------------------------------------
@@ -372,14 +446,6 @@ __device__ __forceinline__ void medium_backward(const MediumView& g, float4* dmu
 // so the forward, which reads the corner values of every sample anyway,
 // keeps the two 3x3 sums and the backward needs no corner value at all.
 // gx, gy, gz of trilinear_grad are the columns dG/dx_a over the channels.
-//
-// The scatter of dJ/dG into the medium walks each level's cells along the
-// segment.  Consecutive samples share their cell, or step to a neighbouring
-// cell (at most one cell along each axis) with which it shares a face, an
-// edge or a vertex: the corners the two cells share keep their pending
-// weight sums, and only the corners the step leaves behind are flushed with
-// an atomic -- on the bench's hash texture about 40 % fewer atomics than
-// flushing the whole cell at every change.
 struct MediumMoments {
   float3 S, dt;
   float3 ox, oy, oz;  // columns of Do: dS/do_x, dS/do_y, dS/do_z (each over the channels)
@@ -398,221 +464,163 @@ __device__ __forceinline__ void moments_sample(MediumMoments& M, float3 G, float
   M.dz = M.dz + gz * ws;
 }
 
-// Corner q of a cell is (q & 1, (q >> 1) & 1, q >> 2).  For a step by
-// (dx, dy, dz), each in {-1, 0, 1}: the old corners the new cell does not
-// hold, and the new corners the old cell did not hold.
-__device__ __forceinline__ unsigned corners_left(int dx, int dy, int dz) {
-  return (dx > 0 ? 0x55u : 0u) | (dx < 0 ? 0xAAu : 0u) | (dy > 0 ? 0x33u : 0u) | (dy < 0 ? 0xCCu : 0u) |
-         (dz > 0 ? 0x0Fu : 0u) | (dz < 0 ? 0xF0u : 0u);
-}
-__device__ __forceinline__ unsigned corners_added(int dx, int dy, int dz) {
-  return (dx > 0 ? 0xAAu : 0u) | (dx < 0 ? 0x55u : 0u) | (dy > 0 ? 0xCCu : 0u) | (dy < 0 ? 0x33u : 0u) |
-         (dz > 0 ? 0xF0u : 0u) | (dz < 0 ? 0x0Fu : 0u);
-}
-
-// Moves the per-corner values of the old cell to the corners they are in
-// the new one (the added corners keep stale values: the caller refills or
-// clears them).  Axis by axis over the pairs of corners that differ in it.
-template <class T>
-__device__ __forceinline__ void shift_pairs(T (&v)[8], int dl, int bit) {
-#pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    if (q & bit) continue;
-    const T a = v[q], b = v[q | bit];
-    v[q] = dl > 0 ? b : a;
-    v[q | bit] = dl < 0 ? a : b;
-  }
-}
-template <class T>
-__device__ __forceinline__ void shift_corners(T (&v)[8], int dx, int dy, int dz) {
-  shift_pairs(v, dx, 1);
-  shift_pairs(v, dy, 2);
-  shift_pairs(v, dz, 4);
-}
-
-__device__ __forceinline__ bool one_step(int dx, int dy, int dz) {
-  return dx >= -1 && dx <= 1 && dy >= -1 && dy <= 1 && dz >= -1 && dz <= 1;
-}
-
-// Lattice coordinates of the dense grid's cell (clamping as grid_cell).
-struct GridIJK {
-  int i, j, k;
-  float fx, fy, fz;
-  bool free_x, free_y, free_z;
-};
-__device__ __forceinline__ GridIJK grid_ijk(const MediumView& g, float3 x) {
-  GridIJK c;
-  c.fx = grid_axis(x.x, g.lo.x, g.scale.x, g.nx, c.i, c.free_x);
-  c.fy = grid_axis(x.y, g.lo.y, g.scale.y, g.ny, c.j, c.free_y);
-  c.fz = grid_axis(x.z, g.lo.z, g.scale.z, g.nz, c.k, c.free_z);
-  return c;
-}
-__device__ __forceinline__ uint32_t grid_corner(const MediumView& g, int i, int j, int k, int q) {
-  return ((uint32_t)(k + (q >> 2)) * (uint32_t)g.ny + (uint32_t)(j + ((q >> 1) & 1))) * (uint32_t)g.nx +
-         (uint32_t)(i + (q & 1));
-}
-
-// G and its gradient together, sharing the interpolation's intermediate
-// values: the differences along x feed both the x interpolations and
-// dG/dx, the differences of the x-interpolated values along y feed the y
-// interpolations and dG/dy, and the difference of the two y-interpolated
-// values along z gives G and dG/dz (the derivatives of trilinear; about
-// half of the arithmetic of trilinear and trilinear_grad apart).
-template <class Cell>
-__device__ __forceinline__ float3 trilinear_value_grad(const CellNodes& q, const Cell& c, float3 scale, float3& gx,
-                                                       float3& gy, float3& gz) {
-  const float3 a00 = q.c100 - q.c000, a10 = q.c110 - q.c010, a01 = q.c101 - q.c001, a11 = q.c111 - q.c011;
-  const float3 x00 = q.c000 + a00 * c.fx, x10 = q.c010 + a10 * c.fx;
-  const float3 x01 = q.c001 + a01 * c.fx, x11 = q.c011 + a11 * c.fx;
-  const float3 b0 = x10 - x00, b1 = x11 - x01;
-  const float3 y0 = x00 + b0 * c.fy, y1 = x01 + b1 * c.fy;
-  const float3 e = y1 - y0;
-  const float3 ax0 = a00 + (a10 - a00) * c.fy, ax1 = a01 + (a11 - a01) * c.fy;
-  gx = (ax0 + (ax1 - ax0) * c.fz) * (c.free_x ? scale.x : 0.0f);
-  gy = (b0 + (b1 - b0) * c.fz) * (c.free_y ? scale.y : 0.0f);
-  gz = e * (c.free_z ? scale.z : 0.0f);
-  return y0 + e * c.fz;
-}
-
-// One level's (or the dense grid's) samples for the forward: each sample's
-// eight corner values, its G and gradient into the moments.  (Carrying the
-// shared corners' values from cell to cell, as the scatter below carries its
-// sums, read 60 % fewer entries but made this pass twice as slow: the
-// per-sample reads are independent of one another, the carried ones are
-// not.)
-template <class Cell, class Entry>
-__device__ __forceinline__ void moments_walk(MediumMoments& M, const float4* mu, float3 o, float3 d, float h, int m,
-                                             float r, float3 scale, const Cell& cell_of, const Entry& entry_of) {
-  for (int i = 0; i <= m; ++i) {
-    const float w = i < m ? h : r;
-    const float s = i < m ? ((float)i + 0.5f) * h : (float)m * h + 0.5f * r;
-    const auto c = cell_of(o + d * s);
-    size_t e[8];
-    entry_of(c, e);
-    CellNodes qn;
-    qn.c000 = xyz(__ldg(mu + e[0]));
-    qn.c100 = xyz(__ldg(mu + e[1]));
-    qn.c010 = xyz(__ldg(mu + e[2]));
-    qn.c110 = xyz(__ldg(mu + e[3]));
-    qn.c001 = xyz(__ldg(mu + e[4]));
-    qn.c101 = xyz(__ldg(mu + e[5]));
-    qn.c011 = xyz(__ldg(mu + e[6]));
-    qn.c111 = xyz(__ldg(mu + e[7]));
+// Samples p, p + lanes, ... of one lattice for the forward: G and its gradient
+// into the moments.
+template <bool kInside>
+__device__ __forceinline__ void moments_walk(MediumMoments& M, const float4* __restrict__ mu, const Lattice& T,
+                                             const MediumSteps& st, float3 d, int p, int lanes) {
+  for (int i = p; i <= st.m; i += lanes) {
+    const float w = st.weight(i), s = st.place(i);
+    const LatticeCell c = lattice_cell<kInside>(T, s);
     float3 gx, gy, gz;
-    const float3 G = trilinear_value_grad(qn, c, scale, gx, gy, gz);
+    const float3 G = trilinear_value_grad(cell_nodes(mu, T, c), c, T.scale, gx, gy, gz);
     moments_sample(M, G, gx, gy, gz, w, s);
-    if (i == m) M.dt = M.dt + G + (gx * d.x + gy * d.y + gz * d.z) * (0.5f * r);
+    if (i == st.m) M.dt = M.dt + G + (gx * d.x + gy * d.y + gz * d.z) * (0.5f * st.r);
   }
 }
 
+// Lane p's part (the samples p, p + lanes, ...) of a segment's moments.
 template <bool kHash>
-__device__ __forceinline__ MediumMoments medium_moments(const MediumView& g, float3 o, float3 d, float t) {
-  const float h = g.step;
-  const int m = medium_full_steps(t, h);
-  const float r = t - (float)m * h;
+__device__ __forceinline__ MediumMoments medium_moments(const MediumView& g, float3 o, float3 d, float t, int p,
+                                                        int lanes) {
+  const MediumSteps st(t, g.step);
   MediumMoments M;
   M.S = M.dt = M.ox = M.oy = M.oz = M.dx = M.dy = M.dz = mk(0.f, 0.f, 0.f);
-  if (kHash && g.levels) {
-    for (int l = 0; l < g.levels; ++l) {
-      const GridLevel L = load_level(g.lev + l);
-      moments_walk(M, g.mu, o, d, h, m, r, mk(L.sx, L.sy, L.sz),
-                   [&](float3 x) { return level_cell(L, g.lo, x); },
-                   [&](const LevelCell& c, size_t (&e)[8]) { level_corner_entries(L, c, e); });
-    }
-    return M;
+  const int levels = kHash && g.levels ? g.levels : 1;
+  for (int l = 0; l < levels; ++l) {
+    const Lattice T = lattice_of<kHash>(g, l, o, d);
+    if (__all_sync(__activemask(), lattice_inside(T, t))) moments_walk<true>(M, g.mu, T, st, d, p, lanes);
+    else moments_walk<false>(M, g.mu, T, st, d, p, lanes);
   }
-  moments_walk(M, g.mu, o, d, h, m, r, g.scale, [&](float3 x) { return grid_ijk(g, x); },
-               [&](const GridIJK& c, size_t (&e)[8]) {
-                 const uint32_t b = grid_corner(g, c.i, c.j, c.k, 0), sx = (uint32_t)g.nx, sy = sx * (uint32_t)g.ny;
-                 e[0] = b; e[1] = b + 1; e[2] = b + sx; e[3] = b + sx + 1;
-                 e[4] = b + sy; e[5] = b + sy + 1; e[6] = b + sy + sx; e[7] = b + sy + sx + 1;
-               });
   return M;
 }
 
-// dJ/dG at the table entries (or grid nodes) for one segment: sbar times
-// the sum over samples of w_i times each corner's trilinear weight.  The
-// sums are kept per corner of the current cell and carried along shared
-// corners; a corner is added to its entry with one 128-bit atomic when the
-// walk leaves it (hashed corners that share an entry add).
-template <class Cell, class Entry>
-__device__ __forceinline__ void scatter_walk(float4* dmu, float3 o, float3 d, float h, int m, float r, float3 sbar,
-                                             const Cell& cell_of, const Entry& entry_of) {
+// ---------------------------------------------------------------------------
+// adjoint
+// ---------------------------------------------------------------------------
+// One 128-bit vector reduction per entry (w unused) where `on`: predicated, not
+// branched around.
+__device__ __forceinline__ void red4_if(bool on, float4* p, float3 v) {
+  asm volatile("{ .reg .pred q; setp.ne.u32 q, %0, 0; @q red.relaxed.gpu.global.add.v4.f32 [%1], {%2, %3, %4, %5}; }" ::"r"(
+                   (uint32_t)on), "l"(p), "f"(v.x), "f"(v.y), "f"(v.z), "f"(0.f)
+               : "memory");
+}
+
+// Adjoint of one lattice's share of the optical depth over the samples
+// [i0, i1) of one segment at fixed t (sbar = dJ/dS per channel): dJ/dG into dmu
+// (unless null) and, when `gather` is set (the forward kept no moments of this
+// segment), dJ/du0 and the sum of s dJ/du (lattice units) added to ob and db,
+// from sbar . G at the samples' corners.
+//
+// Consecutive samples share their cell, or step to a neighbouring one (at
+// most one cell along each axis), which shares corners with it: the weight
+// sums of shared corners are carried along, and only the corners left behind
+// are added to their entries with an atomic (about 40 % fewer atomics than for
+// whole cells; hashed corners that share an entry add).  The eight slots are
+// the parities of the corners' lattice coordinates (bit a of a slot: the
+// coordinate along axis a is odd), so a corner has the same slot in every cell
+// that holds it and nothing moves on a step: a step's new corners take the
+// slots of those it leaves.  Within a cell sbar . G is a polynomial in the odd
+// coordinates' weights X, Y, Z, whose coefficients are formed once per cell: its
+// gradient is then nine fused multiply-adds a sample.
+template <bool kInside>
+__device__ __forceinline__ void adjoint_walk(const float4* __restrict__ mu, float4* __restrict__ dmu, const Lattice& T,
+                                             const MediumSteps& st, int i0, int i1, float3 sbar, bool gather, float3& ob,
+                                             float3& db) {
   float acc[8];
-  int pi = 0, pj = 0, pk = 0;
-  bool have = false;
-  for (int i = 0; i <= m; ++i) {
-    const float w = i < m ? h : r;
-    const float s = i < m ? ((float)i + 0.5f) * h : (float)m * h + 0.5f * r;
-    const auto c = cell_of(o + d * s);
-    const int dx = (int)c.i - pi, dy = (int)c.j - pj, dz = (int)c.k - pk;
-    if (!have || dx || dy || dz) {
-      unsigned fresh = 0xFFu;
-      if (have) {
-        const bool near = one_step(dx, dy, dz);
-        const unsigned left = near ? corners_left(dx, dy, dz) : 0xFFu;
-        size_t e[8];
-        entry_of(pi, pj, pk, e);
+  uint32_t e[8];
+  float px = 0.f, py = 0.f, pz = 0.f, pxy = 0.f, pxz = 0.f, pyz = 0.f, pxyz = 0.f;
 #pragma unroll
-        for (int q = 0; q < 8; ++q)
-          if (left & (1u << q)) medium_atomic4(dmu + e[q], sbar * acc[q]);
-        if (near) {
-          shift_corners(acc, dx, dy, dz);
-          fresh = corners_added(dx, dy, dz);
+  for (int q = 0; q < 8; ++q) {
+    acc[q] = 0.f;
+    e[q] = 0u;
+  }
+  int pi = 0, pj = 0, pk = 0;
+  for (int i = i0; i < i1; ++i) {
+    const float w = st.weight(i), s = st.place(i);
+    const LatticeCell c = lattice_cell<kInside>(T, s);
+    const int dx = c.i - pi, dy = c.j - pj, dz = c.k - pk;
+    if ((dx | dy | dz) != 0 || i == i0) {
+      // slots whose corner the cell before does not share
+      unsigned fresh = 0xFFu;
+      if (i > i0) {
+        if (((dx + 1) | (dy + 1) | (dz + 1) | (1 - dx) | (1 - dy) | (1 - dz)) >= 0) {
+          // the coordinate left behind along an axis: p for a step up, p + 1 for one down
+          fresh = (dx ? (((pi + (dx < 0)) & 1) ? 0xAAu : 0x55u) : 0u) | (dy ? (((pj + (dy < 0)) & 1) ? 0xCCu : 0x33u) : 0u) |
+                  (dz ? (((pk + (dz < 0)) & 1) ? 0xF0u : 0x0Fu) : 0u);
+        }
+        if (dmu) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) red4_if((fresh >> q) & 1u, dmu + e[q], sbar * acc[q]);
         }
       }
+      lattice_entries(T, (uint32_t)((c.i + 1) & ~1), (uint32_t)(c.i | 1), (uint32_t)((c.j + 1) & ~1), (uint32_t)(c.j | 1),
+                      (uint32_t)((c.k + 1) & ~1), (uint32_t)(c.k | 1), e);
 #pragma unroll
-      for (int q = 0; q < 8; ++q)
-        if (fresh & (1u << q)) acc[q] = 0.f;
-      have = true;
-      pi = (int)c.i;
-      pj = (int)c.j;
-      pk = (int)c.k;
+      for (int q = 0; q < 8; ++q) acc[q] = fresh & (1u << q) ? 0.f : acc[q];
+      if (gather) {
+        float v[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) v[q] = dot(sbar, xyz(__ldg(mu + e[q])));
+        const float a0 = v[1] - v[0], a1 = v[3] - v[2], a2 = v[5] - v[4], a3 = v[7] - v[6];
+        const float b0 = v[2] - v[0], b2 = v[6] - v[4];
+        px = a0;
+        py = b0;
+        pz = v[4] - v[0];
+        pxy = a1 - a0;
+        pxz = a2 - a0;
+        pyz = b2 - b0;
+        pxyz = (a3 - a2) - (a1 - a0);
+      }
+      pi = c.i;
+      pj = c.j;
+      pk = c.k;
     }
-    const float ux = 1.0f - c.fx, uy = 1.0f - c.fy, uz = 1.0f - c.fz;
-    acc[0] += w * (ux * uy * uz);
-    acc[1] += w * (c.fx * uy * uz);
-    acc[2] += w * (ux * c.fy * uz);
-    acc[3] += w * (c.fx * c.fy * uz);
-    acc[4] += w * (ux * uy * c.fz);
-    acc[5] += w * (c.fx * uy * c.fz);
-    acc[6] += w * (ux * c.fy * c.fz);
-    acc[7] += w * (c.fx * c.fy * c.fz);
+    // weights of the odd and the even coordinate along each axis
+    const float X = c.i & 1 ? 1.0f - c.fx : c.fx, Y = c.j & 1 ? 1.0f - c.fy : c.fy, Z = c.k & 1 ? 1.0f - c.fz : c.fz;
+    const float xe = 1.0f - X, ye = 1.0f - Y, wzo = w * Z, wze = w - wzo;
+    const float w00 = xe * ye, w10 = X * ye, w01 = xe * Y, w11 = X * Y;
+    acc[0] += w00 * wze;
+    acc[1] += w10 * wze;
+    acc[2] += w01 * wze;
+    acc[3] += w11 * wze;
+    acc[4] += w00 * wzo;
+    acc[5] += w10 * wzo;
+    acc[6] += w01 * wzo;
+    acc[7] += w11 * wzo;
+    if (gather) {
+      const float gx = fmaf(Z, fmaf(pxyz, Y, pxz), fmaf(pxy, Y, px)) * w;
+      const float gy = fmaf(Z, fmaf(pxyz, X, pyz), fmaf(pxy, X, py)) * w;
+      const float gz = fmaf(Y, fmaf(pxyz, X, pyz), fmaf(pxz, X, pz)) * w;
+      // (X grows with u where the lower coordinate is even)
+      const float3 gp = mk(kInside || c.free_x ? (c.i & 1 ? -gx : gx) : 0.0f, kInside || c.free_y ? (c.j & 1 ? -gy : gy) : 0.0f,
+                           kInside || c.free_z ? (c.k & 1 ? -gz : gz) : 0.0f);
+      ob = ob + gp;
+      db = db + gp * s;
+    }
   }
-  if (have) {
-    size_t e[8];
-    entry_of(pi, pj, pk, e);
+  if (dmu && i1 > i0) {
 #pragma unroll
-    for (int q = 0; q < 8; ++q) medium_atomic4(dmu + e[q], sbar * acc[q]);
+    for (int q = 0; q < 8; ++q) red4_if(true, dmu + e[q], sbar * acc[q]);
   }
 }
 
+// adjoint_walk over part `part` of a segment's samples (kPartSteps of them, or
+// all with `whole`) on level l of the hash texture, or on the dense grid (l =
+// 0): adds dJ/do and dJ/dd.
 template <bool kHash>
-__device__ __forceinline__ void medium_scatter(const MediumView& g, float4* dmu, float3 o, float3 d, float t,
-                                               float3 sbar) {
-  const float h = g.step;
-  const int m = medium_full_steps(t, h);
-  const float r = t - (float)m * h;
-  if (kHash && g.levels) {
-    for (int l = 0; l < g.levels; ++l) {
-      const GridLevel L = load_level(g.lev + l);
-      scatter_walk(dmu, o, d, h, m, r, sbar, [&](float3 x) { return level_cell(L, g.lo, x); },
-                   [&](int i, int j, int k, size_t (&e)[8]) {
-                     LevelCell c;
-                     c.i = (uint32_t)i;
-                     c.j = (uint32_t)j;
-                     c.k = (uint32_t)k;
-                     level_corner_entries(L, c, e);
-                   });
-    }
-    return;
-  }
-  scatter_walk(dmu, o, d, h, m, r, sbar, [&](float3 x) { return grid_ijk(g, x); },
-               [&](int i, int j, int k, size_t (&e)[8]) {
-                 const uint32_t b = grid_corner(g, i, j, k, 0), sx = (uint32_t)g.nx, sy = sx * (uint32_t)g.ny;
-                 e[0] = b; e[1] = b + 1; e[2] = b + sx; e[3] = b + sx + 1;
-                 e[4] = b + sy; e[5] = b + sy + 1; e[6] = b + sy + sx; e[7] = b + sy + sx + 1;
-               });
+__device__ __forceinline__ void medium_level_adjoint(const MediumView& g, float4* dmu, int l, int part, bool whole,
+                                                     float3 o, float3 d, float t, float3 sbar, bool gather, float3& ob,
+                                                     float3& db) {
+  const MediumSteps st(t, g.step);
+  const int i0 = whole ? 0 : part * kPartSteps, i1 = whole ? st.m + 1 : min(i0 + kPartSteps, st.m + 1);
+  if (i0 >= i1) return;
+  const Lattice T = lattice_of<kHash>(g, l, o, d);
+  float3 uo = mk(0.f, 0.f, 0.f), ud = uo;
+  if (__all_sync(__activemask(), lattice_inside(T, t))) adjoint_walk<true>(g.mu, dmu, T, st, i0, i1, sbar, gather, uo, ud);
+  else adjoint_walk<false>(g.mu, dmu, T, st, i0, i1, sbar, gather, uo, ud);
+  ob = ob + mul(uo, T.scale);
+  db = db + mul(ud, T.scale);
 }
 
 }  // namespace dt

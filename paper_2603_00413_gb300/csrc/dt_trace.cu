@@ -646,6 +646,75 @@ __global__ void __launch_bounds__(128) k_closest_hit_rays(const uint4* __restric
 constexpr int kShadeThreads = 256;
 constexpr int kShadeMinBlocks = 4;  // CTAs per SM the register budget is sized for
 
+// Whether segment a of level k (hit record hh) marches the medium of its scene:
+// a hit above the depth limit from inside (the shading's test of the geometric
+// normal).
+template <bool kBatch>
+__device__ __forceinline__ bool marches(const WsView& W, int k, const SceneEntry& E0, int n_scenes, uint32_t a,
+                                        float4 hh, int& scene) {
+  const int tri = __float_as_int(hh.w);
+  if (tri < 0) return false;
+  scene = kBatch ? find_scene(W.th->starts, n_scenes, __float_as_uint(W.ray_o[a].w)) : 0;
+  const SceneEntry& E = kBatch ? W.ent[scene] : E0;
+  if (!E.mu || k >= E.max_depth) return false;
+  const int i0 = __ldg(E.F + 3 * tri), i1 = __ldg(E.F + 3 * tri + 1), i2 = __ldg(E.F + 3 * tri + 2);
+  const float3 v0 = load3(E.V + 3 * i0), v1 = load3(E.V + 3 * i1), v2 = load3(E.V + 3 * i2);
+  return !(dot(xyz(W.ray_d[a]), cross(v1 - v0, v2 - v0)) < 0.0f);
+}
+
+// The optical depths of the medium over the segments of a shading tile, by the
+// whole CTA (march tiles, dt_medium.cuh): returns the calling thread's segment's
+// (NaN: it needs none, or the moments pass has it).  Marched by each
+// segment's own thread, with 11 to 13 of 32 lanes busy and the CTA waiting for
+// its longest segment, the shading of 8 views of 360x360 with an 8-level hash
+// texture took 11.7 ms; it takes 6.0, at 90 % of L1's data pipe (eight 16-byte
+// reads per sample and level; reading a corner once for all the samples around
+// it, with the adjoint's walk, was slower: 8.4 ms).
+template <bool kBatch, int kGrid>
+__device__ __forceinline__ float3 shade_march(const WsView& W, int k, const SceneEntry& E0, int n_scenes, uint32_t n,
+                                              uint32_t start, uint32_t tile, uint32_t& c_med) {
+  static_assert(kShadeThreads == kTileThreads, "a thread per position");
+  if (W.mom) return mk(NAN, 0.f, 0.f);  // the moments pass has marched them
+  __shared__ MarchTile T;
+  __shared__ float s_S[3][kShadeThreads];
+  const uint32_t size = min((uint32_t)kShadeThreads, n - tile);
+  // (-1: none; every thread asks about its own position)
+  int steps = -1, scene = 0;
+  if (threadIdx.x < size) {
+    const uint32_t i = tile + threadIdx.x, a = start + i;
+    const float4 hh = W.hit[hit_slot(W, k, a, i)];
+    if (marches<kBatch>(W, k, E0, n_scenes, a, hh, scene)) {
+      const SceneEntry& E = kBatch ? W.ent[scene] : E0;
+      steps = medium_full_steps(hh.x, E.gstep);
+      c_med += (uint32_t)steps + 1u;
+    }
+  }
+  if (!__syncthreads_or(steps >= 0)) return mk(NAN, 0.f, 0.f);
+  s_S[0][threadIdx.x] = NAN;
+  march_list(T, tile, size, [&](uint32_t, int&) { return steps; });
+  for (int at; march_group<kDepthLanes>(T, at);) {
+    float3 S = mk(0.f, 0.f, 0.f);
+    uint32_t i = 0;
+    if (at < T.n) {
+      i = T.pos[at];
+      const uint32_t a = start + i;
+      const float4 ro = W.ray_o[a], rd = W.ray_d[a];
+      const int sc = kBatch ? find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w)) : 0;
+      const SceneEntry& E = kBatch ? W.ent[sc] : E0;
+      S = medium_depth_part<kGrid == 2>(medium_view(E, W.ent + sc), xyz(ro), xyz(rd), W.hit[hit_slot(W, k, a, i)].x,
+                                        threadIdx.x & (kDepthLanes - 1), kDepthLanes);
+    }
+    S = mk(group_sum<kDepthLanes>(S.x), group_sum<kDepthLanes>(S.y), group_sum<kDepthLanes>(S.z));
+    if (at < T.n && (threadIdx.x & (kDepthLanes - 1)) == 0) {
+      s_S[0][i - tile] = S.x;
+      s_S[1][i - tile] = S.y;
+      s_S[2][i - tile] = S.z;
+    }
+  }
+  __syncthreads();
+  return mk(s_S[0][threadIdx.x], s_S[1][threadIdx.x], s_S[2][threadIdx.x]);
+}
+
 // order_bits != 0: each child is also counted in its traversal-order
 // bucket (order_bucket of ray_order_key with that many bits; dt_order.cu)
 // and its bucket is stored with the next level.  kGrid: 1 = some scene has
@@ -678,6 +747,8 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeMinBlocks) k_shade(WsView
   for (uint32_t tile = blockIdx.x * kShadeThreads; tile < n; tile += gridDim.x * kShadeThreads) {
     const uint32_t i = tile + threadIdx.x;
     const uint32_t a = start + i;
+    [[maybe_unused]] float3 S_med = mk(NAN, 0.f, 0.f);  // optical depth of the medium (NaN: not marched)
+    if constexpr (kGrid != 0) S_med = shade_march<kBatch, kGrid>(W, k, E0, n_scenes, n, start, tile, c_med);
     int nchild = 0;
     uint32_t fl = 0, scene_id = 0;
     uint32_t b_r = ~0u, p_r = 0, b_t = ~0u, p_t = 0;  // order buckets and next-level positions of the children
@@ -716,10 +787,11 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeMinBlocks) k_shade(WsView
           shade_hit(xyz(ro), d, hh.x, hh.y, hh.z, v0, v1, v2, load3(E.N + 3 * i0), load3(E.N + 3 * i1),
                     load3(E.N + 3 * i2), ior, sigma, h);
           if (kGrid && E.mu && !h.entering) {  // Sec. 3.4 step 5 with the grid's optical depth
-            // tape_mode 2: the medium pass has marched it (S_0 = NaN: not marched there)
-            float3 S = mk(NAN, 0.f, 0.f);
-            if (W.mom) S = mk(W.mom[(kMomS + 0) * W.cap + a], W.mom[(kMomS + 1) * W.cap + a], W.mom[(kMomS + 2) * W.cap + a]);
-            if (isnan(S.x)) {
+            float3 S = S_med;
+            // tape_mode 2: the medium pass has marched it
+            if (W.mom && isnan(S.x))
+              S = mk(W.mom[(kMomS + 0) * W.cap + a], W.mom[(kMomS + 1) * W.cap + a], W.mom[(kMomS + 2) * W.cap + a]);
+            if (isnan(S.x)) {  // marched by neither (the inside test rounded the other way there)
               S = medium_depth<kGrid == 2>(medium_view(E, W.ent + scene), xyz(ro), d, hh.x);
               c_med += (uint32_t)medium_full_steps(hh.x, E.gstep) + 1u;
             }
@@ -833,76 +905,59 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeMinBlocks) k_shade(WsView
 // (medium_moments) into the moments arrays; a segment found entering gets
 // S_0 = NaN, so a shading pass that rounds the test the other way marches
 // it itself.  A pass of its own: the march's accumulators need more
-// registers than the shading pass runs with.  A warp classifies 32
-// positions at a time (hit, a medium, not at the depth limit, from inside),
-// queues the interior ones in shared memory and marches them 32 at a time,
-// so its lanes march together rather than beside lanes whose segment needs
-// no march.
-constexpr int kMedFwdWarps = 8;
+// registers than the shading pass runs with.  March tiles, as in shade_march.
+// (Queued 32 at a time by each warp, a lane per segment, 16 views of 384x384
+// with a 64^3 grid took 2.07 ms; 1.51 now.)
 template <bool kBatch, bool kHash>
-__global__ void __launch_bounds__(32 * kMedFwdWarps, 2) k_medium_forward(WsView W, int k, const SceneEntry E0) {
-  __shared__ uint32_t s_queue[kMedFwdWarps][64];
+__global__ void __launch_bounds__(kTileThreads, 2) k_medium_forward(WsView W, int k, const SceneEntry E0) {
+  __shared__ MarchTile T;
   WsHeader* H = W.hdr;
   const int n_scenes = kBatch ? W.th->n : 1;
   const uint32_t n = level_size(H, k);
   const uint32_t start = H->level_start[k];
   const unsigned long long cap = W.cap;
   float* __restrict__ M = W.mom;
-  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  uint32_t* q = s_queue[wid];
-  const uint32_t warps = gridDim.x * kMedFwdWarps;
-  uint32_t c_med = 0, cnt = 0;
-  for (uint32_t base = (blockIdx.x * kMedFwdWarps + wid) * 32u;; base += warps * 32u) {
-    const bool more = base < n;
-    if (more) {
-      const uint32_t i = base + lane;
-      bool v = false;
-      if (i < n) {
-        const uint32_t a = start + i;
-        const float4 hh = W.hit[hit_slot(W, k, a, i)];
-        const int tri = __float_as_int(hh.w);
-        if (tri >= 0) {
-          const float4 rd = W.ray_d[a];
-          const int scene = kBatch ? find_scene(W.th->starts, n_scenes, __float_as_uint(W.ray_o[a].w)) : 0;
-          const SceneEntry& E = kBatch ? W.ent[scene] : E0;
-          if (E.mu && k < E.max_depth) {
-            const int i0 = __ldg(E.F + 3 * tri), i1 = __ldg(E.F + 3 * tri + 1), i2 = __ldg(E.F + 3 * tri + 2);
-            const float3 v0 = load3(E.V + 3 * i0), v1 = load3(E.V + 3 * i1), v2 = load3(E.V + 3 * i2);
-            if (dot(xyz(rd), cross(v1 - v0, v2 - v0)) < 0.0f) M[kMomS * cap + a] = NAN;  // entering: no medium
-            else v = true;
-          }
-        }
+  const uint32_t size = march_tile(n, gridDim.x);
+  uint32_t c_med = 0;
+  for (uint32_t first = blockIdx.x * size; first < n; first += gridDim.x * size) {
+    march_list(T, first, min(size, n - first), [&](uint32_t i, int&) {
+      const uint32_t a = start + i;
+      const float4 hh = W.hit[hit_slot(W, k, a, i)];
+      int scene = 0;
+      if (!marches<kBatch>(W, k, E0, n_scenes, a, hh, scene)) {
+        M[kMomS * cap + a] = NAN;  // no medium, or entering: not marched here
+        return -1;
       }
-      const unsigned b = __ballot_sync(kFull, v);
-      if (v) q[cnt + __popc(b & ((1u << lane) - 1u))] = i;
-      cnt += (uint32_t)__popc(b);
-      __syncwarp();
-    }
-    while (cnt >= 32u || (!more && cnt > 0u)) {
-      const uint32_t take = cnt < 32u ? cnt : 32u;
-      if (lane < take) {
-        const uint32_t i = q[lane], a = start + i;
-        const float4 hh = W.hit[hit_slot(W, k, a, i)];
+      const int steps = medium_full_steps(hh.x, (kBatch ? W.ent[scene] : E0).gstep);
+      c_med += (uint32_t)steps + 1u;
+      return steps;
+    });
+    for (int at; march_group<kMomentLanes<kHash>>(T, at);) {
+      const int p = threadIdx.x & (kMomentLanes<kHash> - 1);
+      MediumMoments m;
+      m.S = m.dt = m.ox = m.oy = m.oz = m.dx = m.dy = m.dz = mk(0.f, 0.f, 0.f);
+      uint32_t a = 0;
+      if (at < T.n) {
+        const uint32_t i = T.pos[at];
+        a = start + i;
         const float4 ro = W.ray_o[a], rd = W.ray_d[a];
         const int scene = kBatch ? find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w)) : 0;
         const SceneEntry& E = kBatch ? W.ent[scene] : E0;
-        const MediumMoments m = medium_moments<kHash>(medium_view(E, W.ent + scene), xyz(ro), xyz(rd), hh.x);
-        c_med += (uint32_t)medium_full_steps(hh.x, E.gstep) + 1u;
-        const float v[kMomFloats] = {m.S.x,  m.S.y,  m.S.z,  m.dt.x, m.dt.y, m.dt.z, m.ox.x, m.oy.x,
-                                     m.oz.x, m.ox.y, m.oy.y, m.oz.y, m.ox.z, m.oy.z, m.oz.z, m.dx.x,
-                                     m.dy.x, m.dz.x, m.dx.y, m.dy.y, m.dz.y, m.dx.z, m.dy.z, m.dz.z};
-#pragma unroll
-        for (int j = 0; j < kMomFloats; ++j) M[j * cap + a] = v[j];
+        m = medium_moments<kHash>(medium_view(E, W.ent + scene), xyz(ro), xyz(rd), W.hit[hit_slot(W, k, a, i)].x, p,
+                                  kMomentLanes<kHash>);
       }
-      __syncwarp();
-      const uint32_t rest = cnt - take;
-      const uint32_t x = lane < rest ? q[take + lane] : 0u;
-      __syncwarp();
-      if (lane < rest) q[lane] = x;
-      __syncwarp();
-      cnt = rest;
+      float v[kMomFloats] = {m.S.x,  m.S.y,  m.S.z,  m.dt.x, m.dt.y, m.dt.z, m.ox.x, m.oy.x,
+                             m.oz.x, m.ox.y, m.oy.y, m.oz.y, m.ox.z, m.oy.z, m.oz.z, m.dx.x,
+                             m.dy.x, m.dz.x, m.dx.y, m.dy.y, m.dz.y, m.dx.z, m.dy.z, m.dz.z};
+#pragma unroll
+      for (int j = 0; j < kMomFloats; ++j) v[j] = group_sum<kMomentLanes<kHash>>(v[j]);
+      if (at < T.n) {
+#pragma unroll
+        for (int j = 0; j < kMomFloats; ++j)
+          if (j % kMomentLanes<kHash> == p) M[j * cap + a] = v[j];
+      }
     }
-    if (!more) break;
+    __syncthreads();  // the list is made anew
   }
   warp_add_u64(&H->counters[CNT_MEDIUM], c_med);
 }
@@ -1031,7 +1086,7 @@ void launch_forward_table(const TableHeader& th, const SceneEntry* entries, void
     }
     if (W.mom && th.any_medium) {
       ProfScope ps("k_medium_forward", s);
-      const int mb = 8 * num_sms();
+      const int mb = 2 * num_sms();
       if (th.any_medium == 2) {
         if (batch) k_medium_forward<true, true><<<mb, 256, 0, s>>>(W, k, E0);
         else k_medium_forward<false, true><<<mb, 256, 0, s>>>(W, k, E0);

@@ -188,3 +188,66 @@ def test_medium_arguments_are_checked():
             gs.render(medium=dt.Medium(mu, bad["lo"], bad["hi"], bad["step"]))
     with pytest.raises(ValueError):
         dt.Medium(torch.zeros(1, 3, 3, 4, device="cuda"), LO, HI, 0.1)
+
+
+@pytest.mark.parametrize("kind", ["grid", "hash"])
+@pytest.mark.parametrize("step", [5.0, 0.31, 0.02, 0.004, 1e-4])
+@pytest.mark.parametrize("half", [1.3, 0.6])
+def test_march_tapes_agree_over_steps_and_boxes(kind, step, half):
+    """Segments of no full step, of a few, of more than a tile's plain keys and
+    beyond the cap of 8192 steps; boxes that hold the object and boxes that cut
+    it (clamped samples).  The full tape (depths marched by the shading pass,
+    motion by the adjoint) and the moments tape (all marched by the forward) sum
+    the same samples in another order: n terms of FP32 in two orders differ by
+    at most n 2^-24 of their absolute sum (n <= 8193 here), by its square root
+    in practice; gradients of sums that cancel lose another factor of ten."""
+    V, F = S.icosphere(3, 1.0)
+    lo, hi = (-half,) * 3, (half,) * 3
+    if kind == "grid":
+        g = S.random_absorption_grid((9, 12, 10), lo, hi, 3, scale=0.3)
+        med = dt.Medium(torch.from_numpy(g["mu"]).cuda(), lo, hi, step)
+    else:
+        h = S.random_hash_texture(3, 9, 4, 20, lo, hi, 3, scale=0.3)
+        med = dt.HashTexture(torch.from_numpy(h["table"]).cuda(), h["res"], lo, hi, step)
+    cams = S.fibonacci_views(2, 3.0, 33, 27)
+    got = []
+    for moments in (False, True):
+        gs = GpuScene(V, F, 1.4, np.array([0.3, 0.1, 0.6], np.float32), S.sh_env_map(64, 32, 4), cams, 33, 27, 4)
+        gs.params = dt.Params(4, moments=moments)
+        img, tape = gs.render(medium=med)
+        g = torch.from_numpy(np.random.default_rng(1).uniform(0.5, 1.0, img.shape).astype(np.float32)).cuda()
+        got.append((img,) + dt.render_backward(tape, g))
+        samples = tape.stats["medium_samples"]
+    assert samples > 0
+    tol = np.sqrt(min(8193.0, 2.0 / step + 1.0)) * 2.0 ** -24
+    for k, (a, b) in enumerate(zip(*got)):
+        a, b = a.double(), b.double()
+        err = float((a - b).norm() / b.norm())
+        assert err <= (10 * tol + 1e-6 if k == 0 else 100 * tol + 1e-5), (k, err)
+
+
+def test_batch_of_media_and_none_matches_single_renders():
+    """One batch of a dense grid, hash textures of different levels and no
+    medium: images and gradients as rendered one by one."""
+    V, F = S.icosphere(3, 1.0)
+    lo, hi = (-1.3,) * 3, (1.3,) * 3
+    g = S.random_absorption_grid((9, 12, 10), lo, hi, 3)
+    meds = [dt.Medium(torch.from_numpy(g["mu"]).cuda(), lo, hi, 0.05), None]
+    for levels in (1, 4):
+        h = S.random_hash_texture(levels, 8, 4, 20, lo, hi, levels)
+        meds.append(dt.HashTexture(torch.from_numpy(h["table"]).cuda(), h["res"], lo, hi, 0.03 * levels))
+    items, single = [], []
+    for i, med in enumerate(meds):
+        gs = GpuScene(V, F, 1.3 + 0.1 * i, np.array([0.3, 0.1, 0.6], np.float32), S.sh_env_map(64, 32, i),
+                      S.fibonacci_views(1, 3.0, 30 + i, 25), 30 + i, 25, 3 + i)
+        items.append(dt.BatchItem(gs.V, gs.F, gs.bvh, gs.N, gs.ior, gs.sigma, gs.env, gs.cams, 30 + i, 25, gs.params,
+                                  medium=med))
+        img, tape = gs.render(medium=med)
+        single.append((img,) + dt.render_backward(tape, torch.ones_like(img)))
+    imgs, tape = dt.render_batch(items)
+    grads = dt.render_batch_backward(tape, [torch.ones_like(i) for i in imgs])
+    for s, img, gr in zip(single, imgs, grads):
+        for a, b in zip(s, (img,) + tuple(gr)):
+            assert a.shape == b.shape
+            # the same FP32 terms, added in another order by atomics
+            assert float((a.double() - b.double()).norm()) <= 2e-5 * float(a.double().norm())
