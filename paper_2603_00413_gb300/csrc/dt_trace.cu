@@ -128,15 +128,19 @@ __global__ void k_camera(WsView W, unsigned long long capacity) {
 // by +-1e-20 so no 0*inf NaN appears; the far distance is widened by
 // 1 + 2*gamma(3) (Ize, "Robust BVH Ray Traversal", JCGT 2013) so rounding
 // never culls a box the ray touches.
-__device__ __forceinline__ bool slab(float3 o, float3 idir, float lox, float hix, float loy, float hiy, float loz,
-                                     float hiz, float tmin, float tmax, float& tnear) {
+__device__ __forceinline__ void slab_span(float3 o, float3 idir, float lox, float hix, float loy, float hiy, float loz,
+                                          float hiz, float tmin, float& tnear, float& tfar) {
   const float tx0 = (lox - o.x) * idir.x, tx1 = (hix - o.x) * idir.x;
   const float ty0 = (loy - o.y) * idir.y, ty1 = (hiy - o.y) * idir.y;
   const float tz0 = (loz - o.z) * idir.z, tz1 = (hiz - o.z) * idir.z;
-  const float tn = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), tmin));
-  const float tf = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1)) * 1.0000004f;
-  tnear = tn;
-  return tn <= fminf(tf, tmax);
+  tnear = fmaxf(fmaxf(fminf(tx0, tx1), fminf(ty0, ty1)), fmaxf(fminf(tz0, tz1), tmin));
+  tfar = fminf(fminf(fmaxf(tx0, tx1), fmaxf(ty0, ty1)), fmaxf(tz0, tz1)) * 1.0000004f;
+}
+__device__ __forceinline__ bool slab(float3 o, float3 idir, float lox, float hix, float loy, float hiy, float loz,
+                                     float hiz, float tmin, float tmax, float& tnear) {
+  float tfar;
+  slab_span(o, idir, lox, hix, loy, hiy, loz, hiz, tmin, tnear, tfar);
+  return tnear <= fminf(tfar, tmax);
 }
 
 __device__ __forceinline__ float safe_inv(float v) {
@@ -597,6 +601,133 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
   __syncthreads();
   if (threadIdx.x == 0 && s_count[0]) atomicAdd(&H->counters[CNT_NODES], s_count[0]);
   if (threadIdx.x == 1 && s_count[1]) atomicAdd(&H->counters[CNT_TRIS], s_count[1]);
+}
+
+// The traversal of a small render: a level of a few thousand rays leaves most
+// of the lanes without one, and its time is the longest ray's chain of
+// dependent instructions (21 us per level of a 64x64 frame of a 1280-triangle
+// mesh).  Four lanes share a ray: each tests one child of a 4-wide node and, if
+// that is a leaf, its triangle, so a ray makes half as many steps of a third of
+// the instructions; the rays' stacks are in shared memory, where the lanes push
+// their own children.  (The same on nodes coded in 16 bits is slower, 142 us: the
+// decoding is a sixth of the chain.)
+constexpr uint32_t kSmallRender = 40960;  // camera rays: see launch_forward_table
+// A box counts as reached a little (84 roundings) before it is: where a ray
+// meets an edge, both triangles are tested and the smaller one is kept, as with
+// the coded boxes, which are wider than the triangles.
+constexpr float kBoxSlack = 0.99999f;
+constexpr int kSmallThreads = 128;
+constexpr int kSmallRays = kSmallThreads / 4;
+constexpr int kSmallStack = 3 * kTraceStack / 2;  // three siblings per two levels of the binary tree
+template <bool kBatch>
+__global__ void __launch_bounds__(kSmallThreads) k_trace_small(WsView W, int k, const SceneEntry E0,
+                                                               int sorted) {
+  __shared__ int s_stack[kSmallRays][kSmallStack + 4];
+  WsHeader* H = W.hdr;
+  const uint32_t n = level_size(H, k), start = H->level_start[k];
+  const int n_scenes = kBatch ? W.th->n : 1;
+  const int lane = threadIdx.x & 31, c = lane & 3, group = lane & ~3;
+  int* stack = s_stack[threadIdx.x >> 2];
+  uint32_t nvis = 0, ntest = 0;
+  bool overflow = false;
+  // as few rays per warp as the warps allow (a warp takes as many steps as its longest ray, and tests
+  // triangles in most of them when it has eight)
+  const uint32_t warps = gridDim.x * (kSmallThreads / 32);
+  const uint32_t per = min(8u, max(1u, (n + warps - 1u) / warps));
+  for (uint32_t w0 = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * per; w0 < n; w0 += warps * per) {
+    const uint32_t slot = (uint32_t)(lane >> 2);
+    uint32_t pos = slot < per ? w0 + slot : n;
+    if (sorted && pos < n) pos = W.sflag[start + pos];
+    const uint32_t a = start + pos;
+    int node = -1, sp = 0, visits = 0, max_iter = 0, src = -1;
+    float tmin = 0.f;
+    float3 o = mk(0.f, 0.f, 0.f), d = o, idir = o;
+    const float4 *node4 = nullptr, *tris = nullptr;
+    float t = INFINITY, b1 = 0.f, b2 = 0.f;  // this lane's nearest hit
+    int tri = -1;
+    if (pos < n) {
+      const float4 ro = W.ray_o[a], rd = W.ray_d[a], rw = W.ray_w[a];
+      const SceneEntry& E = kBatch ? W.ent[find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w))] : E0;
+      o = xyz(ro);
+      d = xyz(rd);
+      idir = mk(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
+      src = __float_as_int(rw.w);
+      tmin = E.t_min;
+      node4 = E.node4;
+      tris = E.tris;
+      if (E.bh->corrupt) overflow = true;  // a tree that failed validation is not traced
+      else {
+        node = 0;
+        max_iter = E.max_iter;
+      }
+    }
+    float tmax = INFINITY;
+    while (__any_sync(kFull, node >= 0)) {
+      int key = 0x7fffffff, ref = -1;
+      bool inner = false;
+      if (node >= 0) {
+        const float* b = reinterpret_cast<const float*>(node4 + 8 * (size_t)node) + c;
+        ref = __ldg(reinterpret_cast<const int*>(b) + 24);
+        float tn, tf;
+        slab_span(o, idir, __ldg(b), __ldg(b + 4), __ldg(b + 8), __ldg(b + 12), __ldg(b + 16), __ldg(b + 20), tmin, tn, tf);
+        const bool hit = tn * kBoxSlack <= fminf(tf, tmax) && ref != kNoChild;
+        inner = hit && ref >= 0;
+        if (inner) key = (__float_as_int(tn) & ~3) | c;  // (tn >= t_min >= 0: its bits order like the number)
+        if (hit && ref < 0) {
+          float4 rec = make_float4(t, b1, b2, 0.f);
+          HitSoFar h{t, tri, &rec};
+          test_leaf(tris, ~ref, o, d, src, tmin, h, ntest);
+          t = h.t;
+          tri = h.tri;
+          b1 = rec.y;
+          b2 = rec.z;
+        }
+        ++visits;
+      }
+      // the nearest hit of the four lanes, and each inner child's place among them
+      tmax = fminf(t, __shfl_xor_sync(kFull, t, 1));
+      tmax = fminf(tmax, __shfl_xor_sync(kFull, tmax, 2));
+      const int k1 = __shfl_xor_sync(kFull, key, 1), k2 = __shfl_xor_sync(kFull, key, 2), k3 = __shfl_xor_sync(kFull, key, 3);
+      const int rank = (k1 < key) + (k2 < key) + (k3 < key), first = min(min(key, k1), min(k2, k3));
+      const int count = __popc((__ballot_sync(kFull, inner) >> group) & 15u);
+      const int next = __shfl_sync(kFull, ref, group | (first & 3));
+      if (node >= 0) {
+        if (count > 0) {
+          if (inner && rank > 0) stack[sp + count - 1 - rank] = ref;
+          sp += count - 1;
+          node = next;
+        } else {
+          node = -2;  // pop, once the pushes are visible
+        }
+      }
+      __syncwarp();
+      if (node == -2) node = sp > 0 ? stack[--sp] : -1;
+      if (node >= 0 && (sp > kSmallStack || visits >= max_iter)) {  // deeper than a valid tree, or a runaway ray
+        overflow = true;
+        node = -1;
+      }
+      __syncwarp();  // a popped entry may be written over
+    }
+    // the nearest of the lanes' hits, ties to the smaller triangle
+#pragma unroll
+    for (int x = 1; x < 4; x <<= 1) {
+      const float ot = __shfl_xor_sync(kFull, t, x), o1 = __shfl_xor_sync(kFull, b1, x), o2 = __shfl_xor_sync(kFull, b2, x);
+      const int oi = __shfl_xor_sync(kFull, tri, x);
+      if (oi >= 0 && (tri < 0 || ot < t || (ot == t && oi < tri))) {
+        t = ot;
+        b1 = o1;
+        b2 = o2;
+        tri = oi;
+      }
+    }
+    if (c == 0) nvis += (uint32_t)visits;
+    if (pos < n && c == 0)
+      W.hit[hit_slot(W, k, a, pos)] = tri >= 0 ? make_float4(t, b1, b2, __int_as_float(tri))
+                                               : make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+  }
+  warp_add_u64(&H->counters[CNT_NODES], nvis);
+  warp_add_u64(&H->counters[CNT_TRIS], ntest);
+  if (__any_sync(kFull, overflow) && lane == 0) atomicOr(&H->status, ST_STACK_OVERFLOW);
 }
 
 // Closest hit of arbitrary rays (tooling and tests).
@@ -1071,12 +1202,26 @@ void launch_forward_table(const TableHeader& th, const SceneEntry* entries, void
   // the camera rays keep pixel order, which is coherent
   // (small renders are launch-bound: their levels keep append order)
   const int order_bits = th.n_samples >= (uint32_t)g_tuning.order_min_rays ? g_tuning.trace_order : 0;
+  // Four lanes per ray while the rays do not fill the lanes.  Whole passes, one
+  // lane per ray against four, of a convex object of 1280 triangles, two tori
+  // of 20k and a genus-2 body of 67k: 64x64 140 -> 131, 499 -> 357, 589 -> 456
+  // us; 128x128 173 -> 145, 535 -> 409, 671 -> 529; 200x200 195 -> 183, 619 ->
+  // 467, 795 -> 618; 250x250 205 -> 214, 656 -> 485, 856 -> 754: the line is
+  // drawn below the first that loses.  (Whether a level is ordered does not
+  // enter: the order changes neither the nodes visited nor the tests.)
+  const bool small = g_tuning.bvh_width == 2 && th.n_samples <= kSmallRender;
   for (int k = 0; k <= th.max_depth; ++k) {
     const int sorted = order_bits && k > 0;
     if (sorted) launch_order(W, k, order_bits, s);
     {
       ProfScope ps("k_trace", s);
-      if (g_tuning.bvh_width == 4) {
+      if (small) {
+        // a warp per ray as far as the SMs hold them (a level of a convex object has about 1.1 times the camera rays)
+        int g = (int)((3 * (uint64_t)th.n_samples / 2 + kSmallThreads / 32 - 1) / (kSmallThreads / 32));
+        if (g > 8 * num_sms()) g = 8 * num_sms();
+        if (batch) k_trace_small<true><<<g, kSmallThreads, 0, s>>>(W, k, E0, sorted);
+        else k_trace_small<false><<<g, kSmallThreads, 0, s>>>(W, k, E0, sorted);
+      } else if (g_tuning.bvh_width == 4) {
         if (batch) launch_trace_w<4, true>(bps, s, W, k, st, rf, E0, sorted);
         else launch_trace_w<4, false>(bps, s, W, k, st, rf, E0, sorted);
       } else {
