@@ -127,7 +127,8 @@ __device__ __forceinline__ float3 recovered_absorption(const WsView& W, const Sc
 template <bool kBatch, int kGrid>
 __global__ void __launch_bounds__(256, kAdjointMinBlocks) k_adjoint(WsView W, int k, const AdjRecords out_next,
                                                                    const AdjRecords out_cur, const SceneEntry E0,
-                                                                   float4* __restrict__ med_side) {
+                                                                   float4* med_side) {
+  chain_begin();
   extern __shared__ float sums_smem[];
   const WsHeader* H = W.hdr;
   const int n_scenes = kBatch ? W.th->n : 1;
@@ -327,8 +328,9 @@ __global__ void __launch_bounds__(256, kAdjointMinBlocks) k_adjoint(WsView W, in
 // atomics.)
 template <bool kBatch, bool kHash>
 __global__ void __launch_bounds__(kTileThreads, 3) k_medium_adjoint(WsView W, int k, const AdjRecords out_cur,
-                                                                    const float4* __restrict__ med_side,
+                                                                    const float4* med_side,
                                                                     const SceneEntry E0) {
+  chain_begin();
   __shared__ MarchTile T;
   __shared__ float s_motion[6][kTileMax];  // dJ/do, dJ/dd of the listed segments
   const WsHeader* H = W.hdr;
@@ -410,6 +412,7 @@ constexpr int kEnvSharedTexels = 4096;  // 48 KB of float sums
 
 template <bool kBatch, bool kShared>
 __global__ void __launch_bounds__(256) k_env_adjoint(WsView W, const SceneEntry E0) {
+  chain_begin();
   extern __shared__ float env_acc[];
   const WsHeader* H = W.hdr;
   const int n_scenes = kBatch ? W.th->n : 1;
@@ -472,7 +475,8 @@ __global__ void __launch_bounds__(256) k_env_adjoint(WsView W, const SceneEntry 
 
 // zero every scene's accumulators, dIoR, dsigma and absorption-grid
 // gradient (blockIdx.y = scene)
-__global__ void k_zero_grads(const SceneEntry* __restrict__ ent) {
+__global__ void k_zero_grads(const SceneEntry* ent) {
+  chain_begin();
   const SceneEntry& E = ent[blockIdx.y];
   const size_t n = 2 * (size_t)E.nv;
   float4* acc = acc_dN4(E);
@@ -496,7 +500,8 @@ __global__ void k_zero_grads(const SceneEntry* __restrict__ ent) {
 
 // Eq. 13 backward for every scene (blockIdx.y = scene): dN -> dV, on the
 // float4 accumulators (the same arithmetic as face_normal_backward_one)
-__global__ void k_face_normals_backward_table(const SceneEntry* __restrict__ ent) {
+__global__ void k_face_normals_backward_table(const SceneEntry* ent) {
+  chain_begin();
   const SceneEntry& E = ent[blockIdx.y];
   const float4* dN4 = acc_dN4(E);
   float4* dV4 = acc_dV4(E);
@@ -518,7 +523,8 @@ __global__ void k_face_normals_backward_table(const SceneEntry* __restrict__ ent
 }
 
 // the caller's dV [nv][3] from the accumulator (blockIdx.y = scene)
-__global__ void k_finish_grads_table(const SceneEntry* __restrict__ ent) {
+__global__ void k_finish_grads_table(const SceneEntry* ent) {
+  chain_begin();
   const SceneEntry& E = ent[blockIdx.y];
   const float4* dV4 = acc_dV4(E);
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < E.nv; v += gridDim.x * blockDim.x) {
@@ -644,7 +650,8 @@ void launch_l2_loss_grad(const float* img, const float* target, int64_t n, float
   k_l2_loss_grad<<<(int)b, 256, 0, s>>>(img, target, n, scale, grad, loss);
 }
 
-void launch_write_table(const WsView& W, const TableHeader& th, const SceneEntry* entries, int n, cudaStream_t s);
+void launch_write_table(const WsView& W, const TableHeader& th, const SceneEntry* entries, int n, bool clear,
+                        cudaStream_t s);
 
 // Backward of a table of scenes over the tape in ws: rewrites the table with
 // the gradient pointers, zeroes the gradients, sweeps k = D..0, then the
@@ -655,7 +662,7 @@ void launch_backward_table(const TableHeader& th, const SceneEntry* entries, con
   BwsLayout L(max_level, 0);
   const AdjRecords buf[2] = {L.records(bws, 0), L.records(bws, 1)};
   const int n = th.n;
-  launch_write_table(W, th, entries, n, s);
+  launch_write_table(W, th, entries, n, false, s);
   int max_nv = 1, max_nf = 1;
   for (int i = 0; i < n; ++i) {
     if (entries[i].nv > max_nv) max_nv = entries[i].nv;
@@ -666,7 +673,7 @@ void launch_backward_table(const TableHeader& th, const SceneEntry* entries, con
   if (zb > cap_blocks) zb = cap_blocks;
   {
     ProfScope ps("k_zero_grads", s);
-    k_zero_grads<<<dim3(zb, n), 256, 0, s>>>(W.ent);
+    launch_chained(k_zero_grads, dim3(zb, n), 256, 0, s, W.ent);
   }
   const int blocks = kAdjointMinBlocks * num_sms();  // one wave of the resident CTAs
   const size_t smem = sizeof(float) * 4 * (size_t)n;
@@ -676,25 +683,25 @@ void launch_backward_table(const TableHeader& th, const SceneEntry* entries, con
     {
       ProfScope ps("k_adjoint", s);
       if (th.any_medium == 2) {
-        if (n > 1) k_adjoint<true, 2><<<blocks, 256, smem, s>>>(W, k, nx, cu, entries[0], side);
-        else k_adjoint<false, 2><<<blocks, 256, smem, s>>>(W, k, nx, cu, entries[0], side);
+        if (n > 1) launch_chained(k_adjoint<true, 2>, blocks, 256, smem, s, W, k, nx, cu, entries[0], side);
+        else launch_chained(k_adjoint<false, 2>, blocks, 256, smem, s, W, k, nx, cu, entries[0], side);
       } else if (th.any_medium) {
-        if (n > 1) k_adjoint<true, 1><<<blocks, 256, smem, s>>>(W, k, nx, cu, entries[0], side);
-        else k_adjoint<false, 1><<<blocks, 256, smem, s>>>(W, k, nx, cu, entries[0], side);
+        if (n > 1) launch_chained(k_adjoint<true, 1>, blocks, 256, smem, s, W, k, nx, cu, entries[0], side);
+        else launch_chained(k_adjoint<false, 1>, blocks, 256, smem, s, W, k, nx, cu, entries[0], side);
       } else {
-        if (n > 1) k_adjoint<true, 0><<<blocks, 256, smem, s>>>(W, k, nx, cu, entries[0], side);
-        else k_adjoint<false, 0><<<blocks, 256, smem, s>>>(W, k, nx, cu, entries[0], side);
+        if (n > 1) launch_chained(k_adjoint<true, 0>, blocks, 256, smem, s, W, k, nx, cu, entries[0], side);
+        else launch_chained(k_adjoint<false, 0>, blocks, 256, smem, s, W, k, nx, cu, entries[0], side);
       }
     }
     if (th.any_medium) {
       ProfScope ps("k_medium_adjoint", s);
       const int mb = 3 * num_sms();
       if (th.any_medium == 2) {
-        if (n > 1) k_medium_adjoint<true, true><<<mb, 256, 0, s>>>(W, k, cu, side, entries[0]);
-        else k_medium_adjoint<false, true><<<mb, 256, 0, s>>>(W, k, cu, side, entries[0]);
+        if (n > 1) launch_chained(k_medium_adjoint<true, true>, mb, 256, 0, s, W, k, cu, side, entries[0]);
+        else launch_chained(k_medium_adjoint<false, true>, mb, 256, 0, s, W, k, cu, side, entries[0]);
       } else {
-        if (n > 1) k_medium_adjoint<true, false><<<mb, 256, 0, s>>>(W, k, cu, side, entries[0]);
-        else k_medium_adjoint<false, false><<<mb, 256, 0, s>>>(W, k, cu, side, entries[0]);
+        if (n > 1) launch_chained(k_medium_adjoint<true, false>, mb, 256, 0, s, W, k, cu, side, entries[0]);
+        else launch_chained(k_medium_adjoint<false, false>, mb, 256, 0, s, W, k, cu, side, entries[0]);
       }
     }
   }
@@ -702,18 +709,18 @@ void launch_backward_table(const TableHeader& th, const SceneEntry* entries, con
     ProfScope ps("k_env_adjoint", s);
     const SceneEntry& E0 = entries[0];
     const int tex = E0.env_w * E0.env_h;
-    if (n > 1) k_env_adjoint<true, false><<<4 * num_sms(), 256, 0, s>>>(W, E0);
+    if (n > 1) launch_chained(k_env_adjoint<true, false>, 4 * num_sms(), 256, 0, s, W, E0);
     else if (tex <= kEnvSharedTexels)
-      k_env_adjoint<false, true><<<4 * num_sms(), 256, 3 * sizeof(float) * (size_t)tex, s>>>(W, E0);
-    else k_env_adjoint<false, false><<<4 * num_sms(), 256, 0, s>>>(W, E0);
+      launch_chained(k_env_adjoint<false, true>, 4 * num_sms(), 256, 3 * sizeof(float) * (size_t)tex, s, W, E0);
+    else launch_chained(k_env_adjoint<false, false>, 4 * num_sms(), 256, 0, s, W, E0);
   }
   int fb = (max_nf + 255) / 256;
   if (fb > cap_blocks) fb = cap_blocks;
   ProfScope ps("k_face_normals_backward", s);
-  k_face_normals_backward_table<<<dim3(fb, n), 256, 0, s>>>(W.ent);
+  launch_chained(k_face_normals_backward_table, dim3(fb, n), 256, 0, s, W.ent);
   int vb = (max_nv + 255) / 256;
   if (vb > cap_blocks) vb = cap_blocks;
-  k_finish_grads_table<<<dim3(vb, n), 256, 0, s>>>(W.ent);
+  launch_chained(k_finish_grads_table, dim3(vb, n), 256, 0, s, W.ent);
 }
 
 // The backward scratch of a table: the two level buffers, then every

@@ -489,6 +489,38 @@ int num_sms();
 constexpr int kScanBlocks = 1024;
 void launch_scan_exclusive(const uint32_t* src, uint32_t* dst, int32_t m, uint32_t* totals, cudaStream_t s);
 
+// Chained launches.  The kernels of a pass follow each other with a few
+// microseconds of work each, of which a plain launch costs one or two between
+// the end of a kernel and the first instruction of the next.  A kernel that is
+// launched by launch_chained begins while the one before it runs and starts
+// with chain_begin(): it lets the kernel after it be set up as well, then waits
+// until all before it has ended and is visible.  The kernel that opens a chain
+// is launched plainly, so that what the pass only reads (scene, tree, cameras)
+// was complete before any kernel of the chain began; data of the chain itself
+// are read by ordinary loads after the wait (no __restrict__, no __ldg).  A
+// kernel can only be set up early once every CTA of those before it is on an SM
+// or done, so waiting CTAs keep no other from starting.  64x64 frame of a
+// 1280-triangle mesh, 12 launches: 131 -> 112 us; a step of 48 views: 17.36 ->
+// 17.30 ms.
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename... P, typename... A>
+inline void launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t s, const A&... args) {
+  cudaLaunchAttribute attr = {};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // Per-kernel event timing (dt_profile_enable).  Scoped: records a start event
 // on construction and a stop event on destruction when profiling is on.
 struct ProfScope {

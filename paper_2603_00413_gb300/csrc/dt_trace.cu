@@ -55,9 +55,14 @@ static_assert(sizeof(TableChunk) <= 32764, "a table chunk must fit the kernel-pa
 static_assert(sizeof(TableChunk) + sizeof(TableHeader) + 64 <= 32764,
               "the table header and a chunk must fit the kernel-parameter space together");
 
-// One chunk of the table's entries, and with the first chunk the header.
+// One chunk of the table's entries, and with the first chunk the header; a
+// forward pass also clears the workspace header here.
+constexpr int kWsHeaderBytes = 1024;
 __global__ void k_write_table(TableHeader* hdst, const TableHeader hsrc, SceneEntry* dst, const TableChunk src,
-                              int with_header) {
+                              int with_header, uint32_t* clear) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");  // opens the pass's chain
+  if (clear)
+    for (int i = threadIdx.x; i < kWsHeaderBytes / 4; i += blockDim.x) clear[i] = 0;
   if (with_header) {
     const uint32_t* a = reinterpret_cast<const uint32_t*>(&hsrc);
     uint32_t* b = reinterpret_cast<uint32_t*>(hdst);
@@ -89,6 +94,7 @@ __device__ __forceinline__ uint32_t tiled_pixel(uint32_t q, uint32_t w, uint32_t
 // sample also clears the pixel in the image the shading passes add to (one
 // launch less per render than a clearing kernel of its own).
 __global__ void k_camera(WsView W, unsigned long long capacity) {
+  chain_begin();
   const SceneEntry& E = W.ent[blockIdx.y];
   if (blockIdx.x == 0 && threadIdx.x == 0 && E.bh->coarse > kQCoarse) atomicOr(&W.hdr->exact, 1u);
   if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) {
@@ -449,6 +455,7 @@ constexpr int kTraceThreads = 128;
 template <int kMinBlocks, int kWidth, bool kBatch>
 __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, int k, int steps, int refill,
                                                            const SceneEntry E0, int sorted) {
+  chain_begin();
   WsHeader* H = W.hdr;
   if (kWidth == 2 && H->exact) {
     trace_level_exact(W, k, sorted);
@@ -520,7 +527,7 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
       if (qb > qe) qb = qe;
       if (cursor_done && qb >= qe) exhausted = true;
       if (!active && i < n) {
-        const uint32_t pos = order ? __ldg(order + i) : i;
+        const uint32_t pos = order ? order[i] : i;
         if (pos >= n) overflow = true;  // not a permutation of the level: reported, not traced
         else {
           const uint32_t a = start + pos;
@@ -622,6 +629,7 @@ constexpr int kSmallStack = 3 * kTraceStack / 2;  // three siblings per two leve
 template <bool kBatch>
 __global__ void __launch_bounds__(kSmallThreads) k_trace_small(WsView W, int k, const SceneEntry E0,
                                                                int sorted) {
+  chain_begin();
   __shared__ int s_stack[kSmallRays][kSmallStack + 4];
   WsHeader* H = W.hdr;
   const uint32_t n = level_size(H, k), start = H->level_start[k];
@@ -854,6 +862,7 @@ __device__ __forceinline__ float3 shade_march(const WsView& W, int k, const Scen
 template <bool kBatch, int kGrid>
 __global__ void __launch_bounds__(kShadeThreads, kShadeMinBlocks) k_shade(WsView W, int k, const SceneEntry E0,
                                                                          int order_bits) {
+  chain_begin();
   WsHeader* H = W.hdr;
   const int n_scenes = kBatch ? W.th->n : 1;
   const uint32_t n = level_size(H, k);
@@ -1041,6 +1050,7 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeMinBlocks) k_shade(WsView
 // with a 64^3 grid took 2.07 ms; 1.51 now.)
 template <bool kBatch, bool kHash>
 __global__ void __launch_bounds__(kTileThreads, 2) k_medium_forward(WsView W, int k, const SceneEntry E0) {
+  chain_begin();
   __shared__ MarchTile T;
   WsHeader* H = W.hdr;
   const int n_scenes = kBatch ? W.th->n : 1;
@@ -1155,23 +1165,25 @@ template <int kWidth, bool kBatch, typename... A>
 static void launch_trace_w(int bps, cudaStream_t s, A... a) {
   const int sms = num_sms();
   switch (bps) {
-    case 1: case 2: case 3: k_trace<6, kWidth, kBatch><<<2 * bps * sms, kTraceThreads, 0, s>>>(a...); break;
-    case 4: k_trace<8, kWidth, kBatch><<<8 * sms, kTraceThreads, 0, s>>>(a...); break;
-    case 5: k_trace<9, kWidth, kBatch><<<9 * sms, kTraceThreads, 0, s>>>(a...); break;
-    default: k_trace<12, kWidth, kBatch><<<2 * bps * sms, kTraceThreads, 0, s>>>(a...); break;
+    case 1: case 2: case 3: launch_chained(k_trace<6, kWidth, kBatch>, 2 * bps * sms, kTraceThreads, 0, s, a...); break;
+    case 4: launch_chained(k_trace<8, kWidth, kBatch>, 8 * sms, kTraceThreads, 0, s, a...); break;
+    case 5: launch_chained(k_trace<9, kWidth, kBatch>, 9 * sms, kTraceThreads, 0, s, a...); break;
+    default: launch_chained(k_trace<12, kWidth, kBatch>, 2 * bps * sms, kTraceThreads, 0, s, a...); break;
   }
 }
 static int traversal_limit(int32_t nf) { return 2 * n_int_of(nf) + 8; }
 
 // Writes the scene table (header + entries) into the workspace.
-void launch_write_table(const WsView& W, const TableHeader& th, const SceneEntry* entries, int n, cudaStream_t s) {
+void launch_write_table(const WsView& W, const TableHeader& th, const SceneEntry* entries, int n, bool clear,
+                        cudaStream_t s) {
   ProfScope ps("k_write_table", s);
   for (int first = 0; first < n; first += kEntriesPerChunk) {
     TableChunk c;
     c.first = first;
     c.count = n - first < kEntriesPerChunk ? n - first : kEntriesPerChunk;
     for (int k = 0; k < c.count; ++k) c.e[k] = entries[first + k];
-    k_write_table<<<1, 256, 0, s>>>(W.th, th, W.ent, c, first == 0 ? 1 : 0);
+    k_write_table<<<1, 256, 0, s>>>(W.th, th, W.ent, c, first == 0 ? 1 : 0,
+                                 clear && first == 0 ? reinterpret_cast<uint32_t*>(W.hdr) : nullptr);
   }
 }
 
@@ -1182,8 +1194,7 @@ void launch_forward_table(const TableHeader& th, const SceneEntry* entries, void
                           unsigned long long ring, bool mom, cudaStream_t s) {
   WsView W = ws_view(ws, cap, ring, mom);
   const int n = th.n;
-  cudaMemsetAsync(ws, 0, 1024, s);
-  launch_write_table(W, th, entries, n, s);
+  launch_write_table(W, th, entries, n, true, s);
   uint32_t max_s = 0;
   for (int i = 0; i < n; ++i) {
     const uint32_t ns = entries[i].pix_count * (uint32_t)entries[i].spp;
@@ -1193,7 +1204,7 @@ void launch_forward_table(const TableHeader& th, const SceneEntry* entries, void
   if (cb > 4 * num_sms()) cb = 4 * num_sms();
   {
     ProfScope ps("k_camera", s);
-    k_camera<<<dim3(cb > 0 ? cb : 1, n), 256, 0, s>>>(W, cap);
+    launch_chained(k_camera, dim3(cb > 0 ? cb : 1, n), 256, 0, s, W, cap);
   }
   const bool batch = n > 1;
   const SceneEntry& E0 = entries[0];
@@ -1213,14 +1224,16 @@ void launch_forward_table(const TableHeader& th, const SceneEntry* entries, void
   for (int k = 0; k <= th.max_depth; ++k) {
     const int sorted = order_bits && k > 0;
     if (sorted) launch_order(W, k, order_bits, s);
+    const int bits = k < th.max_depth ? order_bits : 0;
+    if (bits) launch_order_clear(W, bits, s);  // (before the traversal: between kernels it would break the chain)
     {
       ProfScope ps("k_trace", s);
       if (small) {
         // a warp per ray as far as the SMs hold them (a level of a convex object has about 1.1 times the camera rays)
         int g = (int)((3 * (uint64_t)th.n_samples / 2 + kSmallThreads / 32 - 1) / (kSmallThreads / 32));
         if (g > 8 * num_sms()) g = 8 * num_sms();
-        if (batch) k_trace_small<true><<<g, kSmallThreads, 0, s>>>(W, k, E0, sorted);
-        else k_trace_small<false><<<g, kSmallThreads, 0, s>>>(W, k, E0, sorted);
+        if (batch) launch_chained(k_trace_small<true>, g, kSmallThreads, 0, s, W, k, E0, sorted);
+        else launch_chained(k_trace_small<false>, g, kSmallThreads, 0, s, W, k, E0, sorted);
       } else if (g_tuning.bvh_width == 4) {
         if (batch) launch_trace_w<4, true>(bps, s, W, k, st, rf, E0, sorted);
         else launch_trace_w<4, false>(bps, s, W, k, st, rf, E0, sorted);
@@ -1233,26 +1246,24 @@ void launch_forward_table(const TableHeader& th, const SceneEntry* entries, void
       ProfScope ps("k_medium_forward", s);
       const int mb = 2 * num_sms();
       if (th.any_medium == 2) {
-        if (batch) k_medium_forward<true, true><<<mb, 256, 0, s>>>(W, k, E0);
-        else k_medium_forward<false, true><<<mb, 256, 0, s>>>(W, k, E0);
+        if (batch) launch_chained(k_medium_forward<true, true>, mb, 256, 0, s, W, k, E0);
+        else launch_chained(k_medium_forward<false, true>, mb, 256, 0, s, W, k, E0);
       } else {
-        if (batch) k_medium_forward<true, false><<<mb, 256, 0, s>>>(W, k, E0);
-        else k_medium_forward<false, false><<<mb, 256, 0, s>>>(W, k, E0);
+        if (batch) launch_chained(k_medium_forward<true, false>, mb, 256, 0, s, W, k, E0);
+        else launch_chained(k_medium_forward<false, false>, mb, 256, 0, s, W, k, E0);
       }
     }
     {
-      const int bits = k < th.max_depth ? order_bits : 0;
-      if (bits) launch_order_clear(W, bits, s);
       ProfScope ps("k_shade", s);
       if (th.any_medium == 2) {
-        if (batch) k_shade<true, 2><<<shade_blocks(), kShadeThreads, 0, s>>>(W, k, E0, bits);
-        else k_shade<false, 2><<<shade_blocks(), kShadeThreads, 0, s>>>(W, k, E0, bits);
+        if (batch) launch_chained(k_shade<true, 2>, shade_blocks(), kShadeThreads, 0, s, W, k, E0, bits);
+        else launch_chained(k_shade<false, 2>, shade_blocks(), kShadeThreads, 0, s, W, k, E0, bits);
       } else if (th.any_medium) {
-        if (batch) k_shade<true, 1><<<shade_blocks(), kShadeThreads, 0, s>>>(W, k, E0, bits);
-        else k_shade<false, 1><<<shade_blocks(), kShadeThreads, 0, s>>>(W, k, E0, bits);
+        if (batch) launch_chained(k_shade<true, 1>, shade_blocks(), kShadeThreads, 0, s, W, k, E0, bits);
+        else launch_chained(k_shade<false, 1>, shade_blocks(), kShadeThreads, 0, s, W, k, E0, bits);
       } else {
-        if (batch) k_shade<true, 0><<<shade_blocks(), kShadeThreads, 0, s>>>(W, k, E0, bits);
-        else k_shade<false, 0><<<shade_blocks(), kShadeThreads, 0, s>>>(W, k, E0, bits);
+        if (batch) launch_chained(k_shade<true, 0>, shade_blocks(), kShadeThreads, 0, s, W, k, E0, bits);
+        else launch_chained(k_shade<false, 0>, shade_blocks(), kShadeThreads, 0, s, W, k, E0, bits);
       }
     }
   }
