@@ -208,9 +208,9 @@ __device__ __forceinline__ void ld_node2(const uint4* p, uint4& a, uint4& b) {
       : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w)
       : "l"(p));
 }
-__device__ __forceinline__ float4 ld_nc_l1na(const float4* p) {
+__device__ __forceinline__ float4 ld_l1na(const float4* p) {
   float4 r;
-  asm("ld.global.nc.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p));
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p) : "memory");
   return r;
 }
 
@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
           const uint32_t a = start + pos;
           // read once here: not allocated in L1, so they do not evict BVH
           // nodes (L2 keeps them for the shading pass that follows)
-          const float4 ro = ld_nc_l1na(W.ray_o + a), rd = ld_nc_l1na(W.ray_d + a), rw = ld_nc_l1na(W.ray_w + a);
+          const float4 ro = ld_l1na(W.ray_o + a), rd = ld_l1na(W.ray_d + a), rw = ld_l1na(W.ray_w + a);
           if (kBatch) {
             const SceneEntry& E = W.ent[find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w))];
             bh = E.bh;
