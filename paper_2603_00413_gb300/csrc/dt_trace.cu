@@ -168,7 +168,7 @@ struct HitSoFar {
 // the lanes of a warp test different triangles, and a branch per condition
 // runs the block's pieces one after another with a few lanes each (with the
 // branches in visit_node2 below gone as well: 13.2 -> 11.1 ms of traversal per
-// 48-view genus-2 step).
+// 48-view genus-2 step, then).
 __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, int leaf, float3 o, float3 d, int src,
                                           float tmin, HitSoFar& h, uint32_t& ntest) {
   const float4 a = __ldg(tris + 3 * leaf), b = __ldg(tris + 3 * leaf + 1), c = __ldg(tris + 3 * leaf + 2);
@@ -210,7 +210,10 @@ __device__ __forceinline__ void ld_node2(const uint4* p, uint4& a, uint4& b) {
 }
 __device__ __forceinline__ float4 ld_l1na(const float4* p) {
   float4 r;
-  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w) : "l"(p) : "memory");
+  asm volatile("ld.global.L1::no_allocate.v4.f32 {%0,%1,%2,%3}, [%4];"
+               : "=f"(r.x), "=f"(r.y), "=f"(r.z), "=f"(r.w)
+               : "l"(p)
+               : "memory");
   return r;
 }
 
@@ -258,59 +261,56 @@ __device__ __forceinline__ bool slab_q(const RayQ& r, uint32_t x, uint32_t y, ui
   return tnear <= fminf(fminf(far_plane(r.x, x), far_plane(r.y, y)), fminf(far_plane(r.z, z), tmax));
 }
 
-// One visit of binary node `node`: both children's boxes; hit leaves join the
-// queue p0..p2 (newest first), of the internal children that were hit the
+// One visit of binary node `node`: of the children whose boxes are hit the
 // nearer is returned and the other pushed, and with none the stack is popped
-// (its bottom entry is -1, the end of the search).  Selects and predicated
-// accesses instead of branches, as in test_leaf.  The caller intersects every
-// lane's queued triangles together after a few visits, so that the triangle
-// test runs as one block per few visits for the warp, and visits only while
-// fewer than two are queued, so three slots suffice.
+// (its bottom entry is kNoChild, the end of the search).  Leaves (~index, < 0)
+// go through the stack like nodes.  Selects and predicated accesses instead of
+// branches, as in test_leaf.
 __device__ __forceinline__ int visit_node2(const uint4* __restrict__ node2, int node, const RayQ& r, float tmin,
-                                           float tmax, int* stack, int& sp, int& p0, int& p1, int& p2) {
+                                           float tmax, int* stack, int& sp) {
   uint4 a, b;
   ld_node2(node2 + 2 * node, a, b);
   const int c0 = (int)b.z, c1 = (int)b.w;
   float t0, t1;
   const bool h0 = slab_q(r, a.x, a.y, a.z, tmin, tmax, t0), h1 = slab_q(r, a.w, b.x, b.y, tmin, tmax, t1);
-  const bool l0 = h0 && c0 < 0, l1 = h1 && c1 < 0, i0 = h0 && !l0, i1 = h1 && !l1;
-  p2 = l0 ? p1 : p2;
-  p1 = l0 ? p0 : p1;
-  p0 = l0 ? ~c0 : p0;
-  p2 = l1 ? p1 : p2;
-  p1 = l1 ? p0 : p1;
-  p0 = l1 ? ~c1 : p0;
-  const bool swap = !i0 || (i1 && t1 < t0);
+  const bool swap = !h0 || (h1 && t1 < t0);
   int next = swap ? c1 : c0;
-  if (i0 && i1) stack[sp] = swap ? c0 : c1;
-  sp += i0 && i1 ? 1 : 0;
-  if (!i0 && !i1) next = stack[--sp];
+  if (h0 && h1) stack[sp] = swap ? c0 : c1;
+  sp += h0 && h1 ? 1 : 0;
+  if (!h0 && !h1) next = stack[--sp];
   return next;
 }
 
-// Up to kLeafEvery visits, then the triangles they queued; true once the
-// search is over.  stack: kTraceStack entries above the bottom one, and room
-// for one group's pushes, which are checked here.
-constexpr int kLeafEvery = 6;  // (8 visits: 1 % slower on the 52k-triangle mesh, 1 % faster on the 1M one)
+// Up to kLeafEvery visits, until the next reference is a leaf, then up to
+// kLeafTests leaves in a row; true once the search is over.  A lane that comes
+// to a leaf waits for the others' visits, and the triangle test runs as one
+// block for the warp.  The traversal is bound by the instructions a visit
+// issues (two thirds of the issue slots, most of them on the ALU pipe), so a
+// visit that keeps no leaves aside is the faster one although lanes wait: with
+// leaves queued in registers over six visits, six selects and their predicates
+// more, 48 views of a genus-2 body took 11.06 against 10.41 ms, a million-triangle
+// step 22.7 against 21.8, a batch of meshes 5.89 against 5.51 (one leaf kept
+// aside: 10.9, 22.8, 5.7; all leaves in a row instead of two: 10.56, 22.0, 5.47;
+// one: 11.06, 22.5, 5.83; 4 visits: 10.42, 22.1, 5.56; 8: 10.8, 22.1, 5.65).
+// stack: kTraceStack entries above the bottom one, and room for one group's
+// pushes, which are checked here.
+constexpr int kLeafEvery = 6, kLeafTests = 2;
 constexpr int kStackWords = 1 + kTraceStack + kLeafEvery;
 __device__ __forceinline__ bool visit_group(const uint4* __restrict__ node2, const float4* __restrict__ tris,
                                             const RayQ& r, float3 o, float3 d, int src, float tmin, int* stack,
                                             int& sp, int& node, HitSoFar& h, int& visits, uint32_t& ntest,
                                             bool& overflow) {
-  int p0 = -1, p1 = -1, p2 = -1;
-  for (int j = 0; j < kLeafEvery && node >= 0 && p1 < 0; ++j, ++visits)
-    node = visit_node2(node2, node, r, tmin, h.t, stack, sp, p0, p1, p2);
-  while (p0 >= 0) {
-    test_leaf(tris, p0, o, d, src, tmin, h, ntest);
-    p0 = p1;
-    p1 = p2;
-    p2 = -1;
+  for (const int end = visits + kLeafEvery; node >= 0 && visits < end; ++visits)
+    node = visit_node2(node2, node, r, tmin, h.t, stack, sp);
+  for (int q = 0; q < kLeafTests && node < 0 && node != kNoChild; ++q) {
+    test_leaf(tris, ~node, o, d, src, tmin, h, ntest);
+    node = stack[--sp];
   }
   if (sp > kTraceStack + 1) {
     overflow = true;
-    node = -1;
+    node = kNoChild;
   }
-  return node < 0;
+  return node == kNoChild;
 }
 
 // Closest hit through the exact boxes of the refit, for scenes that the coded
@@ -442,9 +442,8 @@ __device__ __forceinline__ int visit_node4_deferred(const float4* __restrict__ n
 // A claim is one warp's width, so that the warps run out of work together:
 // with 64 the end of a level of 0.7M rays waited a quarter of its time for
 // the warps that had claimed last (12 views of 509x383: 2.88 -> 2.50 ms of
-// traversal).  Within a round, leaves hit by a visit are queued per lane and
-// intersected for the whole warp every kLeafEvery visits.  A warp stops when the level
-// is exhausted and its last ray is done.  sorted != 0: position i of the
+// traversal).  Within a round the lanes visit nodes and test triangles in
+// turns (visit_group).  A warp stops when the level is exhausted and its last ray is done.  sorted != 0: position i of the
 // level is the segment the traversal order put there (its flag word holds
 // it until the shading pass rewrites it).
 // kBatch = false: one scene, whose entry E0 arrives as a kernel parameter
@@ -483,7 +482,7 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
   const float4* tris = E0.tris;
   HitSoFar h{INFINITY, -1, nullptr};
   int stack[kStackWords];
-  stack[0] = -1;
+  stack[0] = kNoChild;
   // the warp's claimed batch [qb, qe) of the level's segments: one atomic on
   // the level cursor per kTraceClaim segments, not one per refill.  Warp w
   // starts with batch w of the level without an atomic, of B =
@@ -588,7 +587,7 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
       if (!done && iters >= max_iter) done = true;
     }
     if (done) {
-      if (node >= 0) overflow = true;  // stopped by the guard
+      if (kWidth == 2 ? node != kNoChild : node >= 0) overflow = true;  // stopped by the guard
       if (h.tri < 0) *h.rec = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
       active = false;
     }
@@ -761,7 +760,7 @@ __global__ void __launch_bounds__(128) k_closest_hit_rays(const uint4* __restric
     } else {
       const RayQ rq = ray_q(ro, rd, bh);
       int stack[kStackWords];
-      stack[0] = -1;
+      stack[0] = kNoChild;
       int sp = 1, node = 0, visits = 0;
       while (!visit_group(nodes, tris, rq, ro, rd, s, tmin, stack, sp, node, h, visits, nt, ovf))
         if (visits >= max_iter) {
@@ -1158,9 +1157,9 @@ static int n_int_of(int32_t nf) { return nf > 1 ? nf - 1 : 1; }
 // register budgets; trace_blocks_per_sm picks one in units of 256 resident
 // threads per SM.  The default 5 is the 56-register variant, nine CTAs (36
 // warps) per SM: at 48 registers and ten CTAs the ray's plane constants spill
-// (11.3 against 11.1 ms per 48-view genus-2 step, 23.0 against 22.4 ms on the
-// million-triangle step), at 64 and eight too few warps hide the node reads
-// (11.3 and 23.4 ms).
+// (10.5 against 10.4 ms per 48-view genus-2 step, 22.1 against 21.8 ms on the
+// million-triangle step, 5.85 against 5.5 ms per batch), at 64 and eight too few
+// warps hide the node reads (2 to 4 % slower).
 template <int kWidth, bool kBatch, typename... A>
 static void launch_trace_w(int bps, cudaStream_t s, A... a) {
   const int sms = num_sms();
