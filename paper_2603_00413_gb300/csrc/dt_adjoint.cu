@@ -353,9 +353,9 @@ __global__ void __launch_bounds__(256, kAdjointMinBlocks) k_adjoint(WsView W, in
 // the levels' parts of dJ/do and dJ/dd meet in shared memory.
 // (A lane per segment over all levels, 32 at a time as they came, 8 views of
 // 360x360 with an 8-level hash texture took 24.5 ms at 9 lanes per instruction;
-// 9.9 now, of which the atomics are 3 and the reads 2.  The same, moments tape:
-// 7.1.  16 views of 384x384 with a 64^3 grid: 2.56 -> 2.19 ms, half of it the
-// atomics.)
+// 8.1 now, of which the atomics are about 3 and the reads 2.  The same, moments
+// tape: 6.7.  16 views of 384x384 with a 64^3 grid: 2.56 -> 2.08 ms, half of it
+// the atomics.)
 template <bool kBatch, bool kHash>
 __global__ void __launch_bounds__(kTileThreads, 3) k_medium_adjoint(WsView W, int k, const AdjRecords out_cur,
                                                                     const float4* med_side,
