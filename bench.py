@@ -284,7 +284,7 @@ def run_reference(args):
 # GPU leg
 # ---------------------------------------------------------------------------
 # kernels launched per profiled scope (a scope may hold more than one kernel)
-KERNELS_PER_SCOPE = {"k_vertex_normals": 2, "k_refit": 3, "k_camera": 1, "k_trace": 1,
+KERNELS_PER_SCOPE = {"k_vertex_normals": 2, "k_refit": 2, "k_camera": 1, "k_trace": 1,
                      "k_shade": 1, "k_order": 2, "order_clear": 0,
                      "k_l2_loss_grad": 1, "k_adjoint": 1, "k_face_normals_backward": 1, "lbvh_build": 27,
                      "k_write_table": 1, "k_zero_grads": 1}

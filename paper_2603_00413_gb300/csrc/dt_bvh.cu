@@ -45,7 +45,8 @@ __global__ void k_face_normals_scatter(const float* __restrict__ V, const int32_
   }
 }
 
-__global__ void k_normals_finish(const unsigned long long* __restrict__ acc, int64_t n3, float* __restrict__ N) {
+__global__ void k_normals_finish(const unsigned long long* acc, int64_t n3, float* __restrict__ N) {
+  chain_begin();
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n3; i += (int64_t)gridDim.x * blockDim.x)
     N[i] = __fdiv_rn(__ll2float_rn((long long)acc[i]) * kNormalUnfix, 3.0f);
 }
@@ -67,7 +68,7 @@ void launch_vertex_normals(const float* V, int32_t nv, const int32_t* F, int32_t
   k_face_normals_scatter<<<blocks > 0 ? blocks : 1, 256, 0, s>>>(V, F, nf, acc);
   const int64_t n3 = 3 * (int64_t)nv;
   const int b2 = (int)((n3 + 255) / 256) < 4 * num_sms() ? (int)((n3 + 255) / 256) : 4 * num_sms();
-  k_normals_finish<<<b2 > 0 ? b2 : 1, 256, 0, s>>>(acc, n3, N);
+  launch_chained(k_normals_finish, b2 > 0 ? b2 : 1, 256, 0, s, acc, n3, N);
 }
 
 void launch_vertex_normals_backward(const float* V, int32_t nv, const int32_t* F, int32_t nf, const float* dN,
@@ -207,8 +208,9 @@ __device__ __forceinline__ void scan_load(const uint32_t* a, int64_t i, int64_t 
   }
 }
 
-__global__ void __launch_bounds__(kScanThreads) k_scan_totals(const uint32_t* __restrict__ a, int64_t m, int64_t span,
-                                                              uint32_t* __restrict__ totals) {
+__global__ void __launch_bounds__(kScanThreads) k_scan_totals(const uint32_t* a, int64_t m, int64_t span,
+                                                              uint32_t* totals) {
+  chain_begin();
   __shared__ uint32_t s_warp[kScanThreads / 32];
   const int64_t lo = blockIdx.x * span, hi = min(lo + span, m);
   uint32_t sum = 0, total;
@@ -223,7 +225,8 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_totals(const uint32_t* __
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_apply(const uint32_t* src, uint32_t* dst, int64_t m, int64_t span,
-                                                             const uint32_t* __restrict__ totals) {
+                                                             const uint32_t* totals) {
+  chain_begin();
   __shared__ uint32_t s_warp[kScanThreads / 32];
   const int64_t lo = blockIdx.x * span, hi = min(lo + span, m);
   uint32_t carry = 0, total;
@@ -374,30 +377,92 @@ __device__ __forceinline__ void load_box(const float4* box, float3& lo, float3& 
 
 // Each leaf writes its triangle record and box, then climbs: the first of two
 // children to reach a node stops, the second merges both boxes, stores the
-// node's box and goes on.  A path to the root has at most n_int nodes; the
-// bound guards a corrupt tree.
-__global__ void k_refit(const float* __restrict__ V, const int32_t* __restrict__ F, int32_t nf, BvhView B,
-                        uint32_t* __restrict__ arrive) {
-  const int n_int = B.hdr->n_int;
-  if (blockIdx.x == 0 && threadIdx.x == 0) B.hdr->coarse = 0;  // counted by k_node2_boxes
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nf; i += gridDim.x * blockDim.x) {
-    const int tri = B.leaf_tri[i];
-    const float3 v0 = load3(V + 3 * F[3 * tri]), v1 = load3(V + 3 * F[3 * tri + 1]), v2 = load3(V + 3 * F[3 * tri + 2]);
-    B.tris[3 * i + 0] = make_float4(v0.x, v0.y, v0.z, __int_as_float(tri));
-    const float3 e1 = v1 - v0, e2 = v2 - v0;
-    B.tris[3 * i + 1] = make_float4(e1.x, e1.y, e1.z, 0.f);
-    B.tris[3 * i + 2] = make_float4(e2.x, e2.y, e2.z, 0.f);
-    float3 lo = mk(fminf(v0.x, fminf(v1.x, v2.x)), fminf(v0.y, fminf(v1.y, v2.y)), fminf(v0.z, fminf(v1.z, v2.z)));
-    float3 hi = mk(fmaxf(v0.x, fmaxf(v1.x, v2.x)), fmaxf(v0.y, fmaxf(v1.y, v2.y)), fmaxf(v0.z, fmaxf(v1.z, v2.z)));
-    store_box(B.box_leaf + 2 * i, lo, hi);
+// node's box and goes on.  Through global memory a step of the climb is a fence,
+// an atomic and a read, two microseconds in a chain as long as the tree is deep.
+// A node is numbered by a position inside its range of leaves (but the root), so
+// a CTA takes kRefitLeaves leaves in a row, and the nodes numbered alike climb in
+// shared memory first; where only one child came that way, it goes on to the
+// second climb, through global memory, as do the nodes numbered outside the CTA's
+// leaves: every node has its two arrivals in one of the two.  (With
+// the nodes' boxes: 120k triangles 67 -> 56 us, 5k 47 -> 37, of which the climb
+// through global memory is still most.)  A path to the root has at most n_int nodes; the bounds guard a
+// corrupt tree.
+constexpr int kRefitLeaves = 512;
+
+// A node of the climb with its links; those of the next one are read while the
+// arrival at this one is awaited.
+struct ClimbNode {
+  int node, up;
+  int2 child;
+};
+__device__ __forceinline__ ClimbNode climb_node(const BvhView& B, int node, int n_int) {
+  ClimbNode c{node, -1, make_int2(kNoChild, kNoChild)};
+  if (node >= 0 && node < n_int) {
+    c.up = B.parent[node];
+    c.child = B.bin_child[node];
+  }
+  return c;
+}
+
+__global__ void __launch_bounds__(kRefitLeaves) k_refit(const float* __restrict__ V, const int32_t* __restrict__ F,
+                                                        int32_t nf, BvhView B, uint32_t* arrive) {
+  chain_begin();
+  __shared__ int s_arrive[kRefitLeaves];
+  __shared__ float s_box[2][6][kRefitLeaves];  // of the left and the right child
+  const int n_int = B.hdr->n_int, tid = threadIdx.x;
+  if (blockIdx.x == 0 && tid == 0) B.hdr->coarse = 0;  // counted by k_node_boxes
+  for (int64_t tile = (int64_t)blockIdx.x * kRefitLeaves; tile < nf; tile += (int64_t)gridDim.x * kRefitLeaves) {
+    __syncthreads();
+    s_arrive[tid] = 0;
+    __syncthreads();
+    const int first = (int)tile, i = first + min(tid, nf - 1 - first);
+    const bool on = tile + tid < nf;
+    float3 lo = mk(0.f, 0.f, 0.f), hi = lo;
     int me = ~i;
-    int node = B.parent[n_int + i];
-    for (int hops = 0; node >= 0 && node < n_int && hops <= n_int; ++hops) {
-      const int2 ch = B.bin_child[node];
-      const int sib = (ch.x == me) ? ch.y : ch.x;
+    ClimbNode at{-1, -1, make_int2(kNoChild, kNoChild)};
+    bool parked = false;
+    if (on) {
+      const int tri = B.leaf_tri[i];
+      const float3 v0 = load3(V + 3 * F[3 * tri]), v1 = load3(V + 3 * F[3 * tri + 1]), v2 = load3(V + 3 * F[3 * tri + 2]);
+      B.tris[3 * i + 0] = make_float4(v0.x, v0.y, v0.z, __int_as_float(tri));
+      const float3 e1 = v1 - v0, e2 = v2 - v0;
+      B.tris[3 * i + 1] = make_float4(e1.x, e1.y, e1.z, 0.f);
+      B.tris[3 * i + 2] = make_float4(e2.x, e2.y, e2.z, 0.f);
+      lo = mk(fminf(v0.x, fminf(v1.x, v2.x)), fminf(v0.y, fminf(v1.y, v2.y)), fminf(v0.z, fminf(v1.z, v2.z)));
+      hi = mk(fmaxf(v0.x, fmaxf(v1.x, v2.x)), fmaxf(v0.y, fmaxf(v1.y, v2.y)), fmaxf(v0.z, fmaxf(v1.z, v2.z)));
+      store_box(B.box_leaf + 2 * i, lo, hi);
+      at = climb_node(B, B.parent[n_int + i], n_int);
+      for (int hops = 0; at.node >= first && at.node < n_int && at.node - first < kRefitLeaves && hops < kRefitLeaves;
+           ++hops) {
+        const int side = at.child.x == me ? 0 : 1, slot = at.node - first;
+        if ((side ? at.child.x : at.child.y) == kNoChild) break;  // the root of a single leaf
+        const ClimbNode next = climb_node(B, at.up, n_int);
+        s_box[side][0][slot] = lo.x;
+        s_box[side][1][slot] = lo.y;
+        s_box[side][2][slot] = lo.z;
+        s_box[side][3][slot] = hi.x;
+        s_box[side][4][slot] = hi.y;
+        s_box[side][5][slot] = hi.z;
+        __threadfence_block();
+        parked = atomicAdd(&s_arrive[slot], 1) == 0;
+        if (parked) break;  // the sibling is still on its way, or comes from another CTA
+        __threadfence_block();
+        const float(*o)[kRefitLeaves] = s_box[1 - side];
+        lo = mk(fminf(lo.x, o[0][slot]), fminf(lo.y, o[1][slot]), fminf(lo.z, o[2][slot]));
+        hi = mk(fmaxf(hi.x, o[3][slot]), fmaxf(hi.y, o[4][slot]), fmaxf(hi.z, o[5][slot]));
+        store_box(B.box_int + 2 * at.node, lo, hi);
+        me = at.node;
+        at = next;
+      }
+    }
+    __syncthreads();
+    if (!on || (parked && s_arrive[at.node - first] > 1)) continue;
+    for (int hops = 0; at.node >= 0 && at.node < n_int && hops <= n_int; ++hops) {
+      const ClimbNode next = climb_node(B, at.up, n_int);
+      const int sib = (at.child.x == me) ? at.child.y : at.child.x;
       if (sib != kNoChild) {
         __threadfence();
-        const uint32_t prev = atomicAdd(arrive + node, 1u);
+        const uint32_t prev = atomicAdd(arrive + at.node, 1u);
         if (prev == 0) break;  // the sibling is still on its way
         __threadfence();
         float3 olo, ohi;
@@ -405,9 +470,9 @@ __global__ void k_refit(const float* __restrict__ V, const int32_t* __restrict__
         lo = mk(fminf(lo.x, olo.x), fminf(lo.y, olo.y), fminf(lo.z, olo.z));
         hi = mk(fmaxf(hi.x, ohi.x), fmaxf(hi.y, ohi.y), fmaxf(hi.z, ohi.z));
       }
-      store_box(B.box_int + 2 * node, lo, hi);
-      me = node;
-      node = B.parent[node];
+      store_box(B.box_int + 2 * at.node, lo, hi);
+      me = at.node;
+      at = next;
     }
   }
 }
@@ -508,7 +573,8 @@ __device__ __forceinline__ float comp3(const float3& v, int k) { return k == 0 ?
 // (validation catches any link a build leaves unset, and the depth walks stop
 // at an unset parent).
 __global__ void __launch_bounds__(256) k_sah_prims(const float* __restrict__ V, const int32_t* __restrict__ F, int32_t nf,
-                                                   uint32_t* __restrict__ bounds, SahView S, BvhView B) {
+                                                   uint32_t* bounds, SahView S, BvhView B) {
+  chain_begin();
   __shared__ uint32_t s_b[6];
   if (threadIdx.x < 6) s_b[threadIdx.x] = threadIdx.x < 3 ? 0xffffffffu : 0u;
   __syncthreads();
@@ -1142,6 +1208,7 @@ __device__ __forceinline__ void sah_tiny_split(SahSmallShared& sh, int cur, bool
 }
 
 __global__ void __launch_bounds__(32 * kSahSmallWarps) k_sah_small(SahView S, BvhView B) {
+  chain_begin();
   static_assert(kSahTiny == 4, "a tiny range has four lanes");
   __shared__ SahSmallShared sh;
   const int n_int = B.hdr->n_int;
@@ -1196,8 +1263,10 @@ __global__ void __launch_bounds__(32 * kSahSmallWarps) k_sah_small(SahView S, Bv
 }
 
 // ---- the 4-wide BVH ----------------------------------------------------------
-// flag[j] = 1 when binary node j sits at even depth (walks up to the root)
-__global__ void k_even_depth(BvhView B, uint32_t* __restrict__ flag) {
+// flag[j] = 1 and bin_to4[j] = 0 when binary node j sits at even depth (walks up
+// to the root), else 0 and -1; also clears the arrivals of the refit that follows
+__global__ void k_even_depth(BvhView B, uint32_t* flag, uint32_t* arrive) {
+  chain_begin();
   const int n_int = B.hdr->n_int;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n_int; j += gridDim.x * blockDim.x) {
     int d = 0, p = j;
@@ -1206,26 +1275,26 @@ __global__ void k_even_depth(BvhView B, uint32_t* __restrict__ flag) {
       ++d;
     }
     flag[j] = (d & 1) ? 0u : 1u;
+    B.bin_to4[j] = (d & 1) ? -1 : 0;
+    arrive[j] = 0u;
   }
 }
 
 // after an exclusive scan of the flags: node4 index per even-depth node, -1 else
-__global__ void k_bin_to4(BvhView B, const uint32_t* __restrict__ scanned) {
+__global__ void k_bin_to4(BvhView B, const uint32_t* scanned) {
+  chain_begin();
   const int n_int = B.hdr->n_int;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n_int; j += gridDim.x * blockDim.x) {
-    int d = 0, p = j;
-    for (int hops = 0; hops <= n_int && p > 0; ++hops) {
-      p = B.parent[p];
-      ++d;
-    }
-    B.bin_to4[j] = (d & 1) ? -1 : (int)scanned[j];
-    if (j == n_int - 1) B.hdr->n4 = (int)scanned[j] + ((d & 1) ? 0 : 1);
+    const bool even = B.bin_to4[j] >= 0;
+    if (even) B.bin_to4[j] = (int)scanned[j];
+    if (j == n_int - 1) B.hdr->n4 = (int)scanned[j] + (even ? 1 : 0);
   }
 }
 
 // children of 4-wide node bin_to4[j] = the grandchildren of binary node j (a
 // leaf child stays as it is); refs in row 6, binary sources in row 7
 __global__ void k_node4_topology(BvhView B) {
+  chain_begin();
   const int n_int = B.hdr->n_int;
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n_int; j += gridDim.x * blockDim.x) {
     const int m = B.bin_to4[j];
@@ -1257,30 +1326,27 @@ __global__ void k_node4_topology(BvhView B) {
   }
 }
 
-// child boxes of every 4-wide node from the binary boxes (after each refit)
-__global__ void k_node4_boxes(BvhView B) {
-  const int n4 = B.hdr->n4;
-  for (int m = blockIdx.x * blockDim.x + threadIdx.x; m < n4; m += gridDim.x * blockDim.x) {
-    const int4 sv = reinterpret_cast<const int4*>(B.node4)[8 * m + 7];
-    const int srcs[4] = {sv.x, sv.y, sv.z, sv.w};
-    float r[6][4];
-    for (int k = 0; k < 4; ++k) {
-      float3 lo = mk(INFINITY, INFINITY, INFINITY), hi = mk(-INFINITY, -INFINITY, -INFINITY);
-      const int x = srcs[k];
-      if (x != kNoChild) {
-        const float4* bx = x >= 0 ? B.box_int + 2 * x : B.box_leaf + 2 * (~x);
-        const float4 a = bx[0], b = bx[1];
-        lo = mk(a.x, a.y, a.z);
-        hi = mk(b.x, b.y, b.z);
-      }
-      r[0][k] = lo.x; r[1][k] = hi.x; r[2][k] = lo.y; r[3][k] = hi.y; r[4][k] = lo.z; r[5][k] = hi.z;
+// child boxes of 4-wide node m from the binary boxes
+__device__ __forceinline__ void node4_boxes(const BvhView& B, int m) {
+  const int4 sv = reinterpret_cast<const int4*>(B.node4)[8 * m + 7];
+  const int srcs[4] = {sv.x, sv.y, sv.z, sv.w};
+  float r[6][4];
+  for (int k = 0; k < 4; ++k) {
+    float3 lo = mk(INFINITY, INFINITY, INFINITY), hi = mk(-INFINITY, -INFINITY, -INFINITY);
+    const int x = srcs[k];
+    if (x != kNoChild) {
+      const float4* bx = x >= 0 ? B.box_int + 2 * x : B.box_leaf + 2 * (~x);
+      const float4 a = bx[0], b = bx[1];
+      lo = mk(a.x, a.y, a.z);
+      hi = mk(b.x, b.y, b.z);
     }
-    for (int row = 0; row < 6; ++row) B.node4[8 * m + row] = make_float4(r[row][0], r[row][1], r[row][2], r[row][3]);
+    r[0][k] = lo.x; r[1][k] = hi.x; r[2][k] = lo.y; r[3][k] = hi.y; r[4][k] = lo.z; r[5][k] = hi.z;
   }
+  for (int row = 0; row < 6; ++row) B.node4[8 * m + row] = make_float4(r[row][0], r[row][1], r[row][2], r[row][3]);
 }
 
-// Binary nodes for the 2-wide traversal, from the binary boxes (after each
-// refit): the grid over the scene's box (the union of the root's two child
+// The nodes' child boxes after each refit, from the binary boxes: the 4-wide
+// nodes', and the binary nodes' for the 2-wide traversal: the grid over the scene's box (the union of the root's two child
 // boxes) and every child box coded on it, rounded outward.  The 0.02 steps
 // cover the rounding of (x - lo) inv, at most 65000 steps times 2^-23.
 __device__ __forceinline__ uint32_t code_planes(float lo, float hi, float base, float inv) {
@@ -1297,8 +1363,9 @@ __device__ __forceinline__ const float4* child_box(const BvhView& B, int c) {
 
 constexpr int kQCluster = 6;  // levels: a cluster below the grid's resolution holds dozens of triangles
 
-__global__ void k_node2_boxes(BvhView B) {
-  const int n_int = B.hdr->n_int;
+__global__ void k_node_boxes(BvhView B) {
+  chain_begin();
+  const int n_int = B.hdr->n_int, n4 = B.hdr->n4;
   float3 rlo = mk(INFINITY, INFINITY, INFINITY), rhi = mk(-INFINITY, -INFINITY, -INFINITY);
   const int2 root = B.bin_child[0];
   for (int k = 0; k < 2; ++k) {
@@ -1315,6 +1382,7 @@ __global__ void k_node2_boxes(BvhView B) {
       B.hdr->q[0] = rlo.x; B.hdr->q[1] = rlo.y; B.hdr->q[2] = rlo.z; B.hdr->q[3] = step;
       B.hdr->hi[0] = rhi.x; B.hdr->hi[1] = rhi.y; B.hdr->hi[2] = rhi.z;
     }
+    if (j < n4) node4_boxes(B, j);
     const int2 ch = B.bin_child[j];
     uint32_t w[6];
     for (int k = 0; k < 2; ++k) {
@@ -1341,6 +1409,7 @@ __global__ void k_node2_boxes(BvhView B) {
 // link consistent with the child lists.  The traversal reads `corrupt` once
 // and refuses to run on a tree that failed.
 __global__ void k_validate(BvhView B) {
+  chain_begin();
   const int n_int = B.hdr->n_int, n4 = B.hdr->n4, nf = B.hdr->nf;
   bool bad = (n4 < 1 || n4 > n_int);
   for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < n_int; j += gridDim.x * blockDim.x) {
@@ -1434,15 +1503,18 @@ static int grid_for(int64_t n, int threads) {
   return b < 1 ? 1 : (int)b;
 }
 
+// The boxes of a tree whose arrivals are cleared, by the kernel before on the stream.
+static void launch_boxes(const float* V, const int32_t* F, int32_t nf, BvhView& B, BuildScratch& S, cudaStream_t s) {
+  ProfScope ps("k_refit", s);
+  launch_chained(k_refit, grid_for(nf, kRefitLeaves), kRefitLeaves, 0, s, V, F, nf, B, S.arrive);
+  launch_chained(k_node_boxes, grid_for(nf, 256), 256, 0, s, B);
+}
+
 void launch_refit(const float* V, const int32_t* F, int32_t nf, void* bvh, void* scratch, cudaStream_t s) {
   BvhView B = bvh_view(bvh, nf);
   BuildScratch S(scratch, nf);
-  const size_t n_int = nf > 1 ? (size_t)nf - 1 : 1;
-  ProfScope ps("k_refit", s);
-  cudaMemsetAsync(S.arrive, 0, sizeof(uint32_t) * n_int, s);
-  k_refit<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, B, S.arrive);
-  k_node2_boxes<<<grid_for((int64_t)n_int, 256), 256, 0, s>>>(B);
-  k_node4_boxes<<<grid_for((int64_t)n_int, 256), 256, 0, s>>>(B);
+  cudaMemsetAsync(S.arrive, 0, sizeof(uint32_t) * (nf > 1 ? (size_t)nf - 1 : 1), s);
+  launch_boxes(V, F, nf, B, S, s);
 }
 
 // Binned SAH topology (see above).  Large levels: kSahFreeDepth levels of
@@ -1453,7 +1525,7 @@ void launch_refit(const float* V, const int32_t* F, int32_t nf, void* bvh, void*
 // traversal's 64-entry stack.
 static void launch_sah_topology(const float* V, const int32_t* F, int32_t nf, BvhView& B, BuildScratch& S,
                                 cudaStream_t s) {
-  k_sah_prims<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, S.bounds, S.sah, B);
+  launch_chained(k_sah_prims, grid_for(nf, 256), 256, 0, s, V, F, nf, S.bounds, S.sah, B);
   int levels = 0;
   if (nf > kSahSmall) {
     int lg = 0;
@@ -1475,15 +1547,15 @@ static void launch_sah_topology(const float* V, const int32_t* F, int32_t nf, Bv
   }
   ProfScope ps("sah_small", s);
   // at most one task per two triangles, a CTA each; about kSahSmall / 2 in practice
-  k_sah_small<<<grid_for(nf / 32 + 1, 1), 32 * kSahSmallWarps, 0, s>>>(S.sah, B);
+  launch_chained(k_sah_small, grid_for(nf / 32 + 1, 1), 32 * kSahSmallWarps, 0, s, S.sah, B);
 }
 
 void launch_scan_exclusive(const uint32_t* src, uint32_t* dst, int32_t m, uint32_t* totals, cudaStream_t s) {
   const int64_t tiles = ((int64_t)m + kScanTile - 1) / kScanTile;
   const int64_t per = (tiles + kScanBlocks - 1) / kScanBlocks;  // tiles per span
   const int blocks = (int)((tiles + per - 1) / per);
-  if (blocks > 1) k_scan_totals<<<blocks, kScanThreads, 0, s>>>(src, m, per * kScanTile, totals);
-  k_scan_apply<<<blocks, kScanThreads, 0, s>>>(src, dst, m, per * kScanTile, totals);
+  if (blocks > 1) launch_chained(k_scan_totals, blocks, kScanThreads, 0, s, src, m, per * kScanTile, totals);
+  launch_chained(k_scan_apply, blocks, kScanThreads, 0, s, src, dst, m, per * kScanTile, totals);
 }
 
 void launch_build(const float* V, const int32_t* F, int32_t nf, void* bvh, void* scratch, cudaStream_t s) {
@@ -1518,13 +1590,13 @@ void launch_build(const float* V, const int32_t* F, int32_t nf, void* bvh, void*
     }
     // 4-wide topology: even-depth nodes, numbered by a scan
     uint32_t* flag = S.keys_b;  // free after the sort (unused by the SAH build)
-    k_even_depth<<<grid_for(n_int, 256), 256, 0, s>>>(B, flag);
+    launch_chained(k_even_depth, grid_for(n_int, 256), 256, 0, s, B, flag, S.arrive);
     launch_scan_exclusive(flag, flag, n_int, S.totals, s);
-    k_bin_to4<<<grid_for(n_int, 256), 256, 0, s>>>(B, flag);
-    k_node4_topology<<<grid_for(n_int, 256), 256, 0, s>>>(B);
-    k_validate<<<grid_for(n_int, 256), 256, 0, s>>>(B);
+    launch_chained(k_bin_to4, grid_for(n_int, 256), 256, 0, s, B, flag);
+    launch_chained(k_node4_topology, grid_for(n_int, 256), 256, 0, s, B);
+    launch_chained(k_validate, grid_for(n_int, 256), 256, 0, s, B);
   }
-  launch_refit(V, F, nf, bvh, scratch, s);
+  launch_boxes(V, F, nf, B, S, s);
 }
 
 }  // namespace dt

@@ -29,7 +29,7 @@ namespace dt {
 // the kernels of dt_vertex_normals (dt_bvh.cu), given this file's scratch
 __global__ void k_face_normals_scatter(const float* __restrict__ V, const int32_t* __restrict__ F, int32_t nf,
                                        unsigned long long* __restrict__ acc);
-__global__ void k_normals_finish(const unsigned long long* __restrict__ acc, int64_t n3, float* __restrict__ N);
+__global__ void k_normals_finish(const unsigned long long* acc, int64_t n3, float* __restrict__ N);
 
 constexpr int32_t kNoAllocMaxVertices = 1 << 20;
 
