@@ -126,7 +126,11 @@ struct SceneSums {
 // true: each segment looks its scene up.  kGrid: 1 = some scene has an
 // absorption grid (dt_medium.cuh), whose optical depth interior segments add;
 // 2 = some scene's is a hash texture.
-constexpr int kAdjointMinBlocks = 3;  // CTAs of 256 per SM the register budget is sized for (80 registers)
+// CTAs of 256 per SM the register budget is sized for: 80 registers, and 64 for a
+// batch without media, whose scene lookups leave more to hide (40 meshes: 2.70 ->
+// 2.58 ms; one scene of 48 views at 64 registers: 2.84 -> 3.08).
+template <bool kBatch, int kGrid>
+constexpr int kAdjointMinBlocks = kBatch && kGrid == 0 ? 4 : 3;
 
 // The attenuation A of an interior segment with an absorption grid, without
 // marching its optical depth again: the forward gave each child the
@@ -157,9 +161,8 @@ __device__ __forceinline__ float3 recovered_absorption(const WsView& W, const Sc
 }
 
 template <bool kBatch, int kGrid>
-__global__ void __launch_bounds__(256, kAdjointMinBlocks) k_adjoint(WsView W, int k, const AdjRecords out_next,
-                                                                   const AdjRecords out_cur, const SceneEntry E0,
-                                                                   float4* med_side) {
+__global__ void __launch_bounds__(256, kAdjointMinBlocks<kBatch, kGrid>)
+    k_adjoint(WsView W, int k, const AdjRecords out_next, const AdjRecords out_cur, const SceneEntry E0, float4* med_side) {
   chain_begin();
   using Sum = typename std::conditional<kBatch, float, double>::type;
   extern __shared__ double sums_buffer[];
@@ -708,7 +711,8 @@ void launch_backward_table(const TableHeader& th, const SceneEntry* entries, con
     ProfScope ps("k_zero_grads", s);
     launch_chained(k_zero_grads, dim3(zb, n), 256, 0, s, W);
   }
-  const int blocks = kAdjointMinBlocks * num_sms();  // one wave of the resident CTAs
+  const int blocks =  // one wave of the resident CTAs
+      (n > 1 && !th.any_medium ? kAdjointMinBlocks<true, 0> : kAdjointMinBlocks<false, 0>) * num_sms();
   const size_t smem = sizeof(double) * 4 * (size_t)n;
   float4* side = reinterpret_cast<float4*>((char*)bws + L.off_med);
   for (int k = th.max_depth; k >= 0; --k) {
