@@ -38,7 +38,7 @@ UNIT = "segments/s"
 RAY_RECORD = 48          # origin+sample, direction+node, throughput+source tri
 HIT_RECORD = 16          # t, b1, b2, tri
 LINK_RECORD = 8          # child index + flags
-NODE_BYTES = 64          # one internal node: two child boxes + child ids
+NODE_BYTES = 32          # one internal node: two child boxes in 16-bit codes + child ids
 TRI_BYTES = 48           # v0, e1, e2 of a leaf triangle
 ORDER_ENTRY = 4          # a level's traversal-order entry / a child's order bucket
 HIT_SCENE = 84           # 3 indices + 3 positions + 3 vertex normals

@@ -453,8 +453,11 @@ dt_status dt_edge_loss_grad(const void* d_topo, int32_t nv, int32_t nf, const fl
  * of 256 resident threads per SM (CTAs of 128 threads; 5 runs nine of them).
  * shade_blocks_per_sm sizes the grid of the shading and adjoint kernels.
  * bvh_width selects the node format the traversal reads: 2 (binary nodes,
- * 32 B: boxes in 16-bit codes, rounded outward) or 4 (4-wide nodes, 128 B: the binary nodes at even depth with
- * their grandchildren as children); both are kept current by build/refit.
+ * 32 B: boxes in 16-bit codes, rounded outward; renders and batches of up to
+ * 40,960 camera rays share a ray among four lanes on the 4-wide nodes
+ * instead) or 4 (4-wide nodes, 128 B: the binary nodes at even depth with
+ * their grandchildren as children, a lane per ray); both are kept current by
+ * build/refit.
  * bvh_builder selects the topology dt_build_bvh builds: 0 = LBVH (Morton
  * codes, radix sort, Karras 2012 hierarchy), 1 = top-down binned surface
  * area heuristic (32 centroid bins per axis, 16 for ranges of at most 128

@@ -87,8 +87,8 @@ constexpr int kTraceStack = 64;
 //    half; the plane of code c is at q[axis] + (c - kQOffset) q[3] (the
 //    header's grid over the scene's box), rounded outward, so a coded box
 //    contains the exact one (empty: lower code 65535, upper 0).
-//    One 32-byte sector per visit instead of two: the traversal waits on its
-//    node reads (half of them miss L1), and the tree's footprint halves.  The
+//    One 32-byte sector per visit instead of two: half of the traversal's
+//    node reads miss L1, and the tree's footprint halves.  The
 //    grid's step is 1/65000 of the scene's longest side, 3e-5 of a unit-sphere
 //    object against 5e-3 for the edges of a million-triangle mesh (node visits
 //    per ray 27.93 -> 28.00 on the 52k-triangle genus-2 mesh, 47.8 -> 48.0 on
@@ -296,7 +296,8 @@ struct WsView {
   uint32_t* sflag;
   unsigned long long cap;
   uint32_t ring;  // 0: hit[a] for arena index a; else hit[(k & 1) ring + i] for position i in level k
-  uint32_t* order_count;  // traversal order: kOrderCounters bucket counters, then the scan's span totals
+  uint32_t* order_count;  // traversal order: kOrderCounters bucket counters, then the scan's span totals; in a
+                          // backward pass the scenes' IoR and sigma sums
   float* mom;     // tape_mode 2: kMomFloats arrays of cap floats (medium moments, see below); else null
 };
 

@@ -1214,7 +1214,7 @@ void launch_forward_table(const TableHeader& th, const SceneEntry* entries, void
   const int order_bits = th.n_samples >= (uint32_t)g_tuning.order_min_rays ? g_tuning.trace_order : 0;
   // Four lanes per ray while the rays do not fill the lanes.  Whole passes, one
   // lane per ray against four, of a convex object of 1280 triangles, two tori
-  // of 20k and a genus-2 body of 67k: 64x64 140 -> 131, 499 -> 357, 589 -> 456
+  // of 52k and a bumpy sphere of 203k: 64x64 140 -> 131, 499 -> 357, 589 -> 456
   // us; 128x128 173 -> 145, 535 -> 409, 671 -> 529; 200x200 195 -> 183, 619 ->
   // 467, 795 -> 618; 250x250 205 -> 214, 656 -> 485, 856 -> 754: the line is
   // drawn below the first that loses.  (Whether a level is ordered does not

@@ -105,3 +105,25 @@ def test_captured_passes():
     torch.cuda.synchronize()
     _near([out], [gs.render()[0]])
     assert float((out - want).abs().max()) > 1e-3
+
+
+def test_captured_build_and_refit():
+    V, F = S.icosphere(4)  # more triangles than one small task of the builder
+    V, F = torch.from_numpy(V).cuda(), torch.from_numpy(F).cuda()
+    o = torch.randn(2000, 3, device="cuda") * 3.0
+    d = -o / o.norm(dim=1, keepdim=True)
+    built, refitted = dt.build_bvh(V, F), dt.build_bvh(V, F)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        built.build(V, F)
+        refitted.refit(V, F)
+        N = dt.vertex_normals(V, F)
+    for scale in (0.7, 1.2):
+        V.mul_(scale)  # replays read the vertices anew
+        graph.replay()
+        want = dt.closest_hit(dt.build_bvh(V, F), o, d)
+        for bvh in (built, refitted):
+            got = dt.closest_hit(bvh, o, d)
+            assert torch.equal(got[0], want[0]) and torch.equal(got[1], want[1])
+        assert torch.equal(N, dt.vertex_normals(V, F))
