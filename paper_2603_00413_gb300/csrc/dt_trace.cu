@@ -805,9 +805,9 @@ __device__ __forceinline__ bool marches(const WsView& W, int k, const SceneEntry
 // (NaN: it needs none, or the moments pass has it).  Marched by each
 // segment's own thread, with 11 to 13 of 32 lanes busy and the CTA waiting for
 // its longest segment, the shading of 8 views of 360x360 with an 8-level hash
-// texture took 11.7 ms; it takes 6.0, at 90 % of L1's data pipe (eight 16-byte
-// reads per sample and level; reading a corner once for all the samples around
-// it, with the adjoint's walk, was slower: 8.4 ms).
+// texture took 11.7 ms; it takes 6.4 (eight 16-byte reads per sample and level;
+// reading a corner once for all the samples around it, with the adjoint's walk,
+// was slower: 8.4 ms).
 template <bool kBatch, int kGrid>
 __device__ __forceinline__ float3 shade_march(const WsView& W, int k, const SceneEntry& E0, int n_scenes, uint32_t n,
                                               uint32_t start, uint32_t tile, uint32_t& c_med) {
@@ -831,19 +831,22 @@ __device__ __forceinline__ float3 shade_march(const WsView& W, int k, const Scen
   s_S[0][threadIdx.x] = NAN;
   march_list(T, tile, size, [&](uint32_t, int&) { return steps; });
   for (int at; march_group<kDepthLanes>(T, at);) {
-    float3 S = mk(0.f, 0.f, 0.f);
+    const bool on = at < T.n;
     uint32_t i = 0;
-    if (at < T.n) {
+    float4 ro = make_float4(0.f, 0.f, 0.f, 0.f), rd = ro;
+    float t = 0.f;
+    int sc = 0;
+    if (on) {
       i = T.pos[at];
       const uint32_t a = start + i;
-      const float4 ro = W.ray_o[a], rd = W.ray_d[a];
-      const int sc = kBatch ? find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w)) : 0;
-      const SceneEntry& E = kBatch ? W.ent[sc] : E0;
-      S = medium_depth_part<kGrid == 2>(medium_view(E, W.ent + sc), xyz(ro), xyz(rd), W.hit[hit_slot(W, k, a, i)].x,
-                                        threadIdx.x & (kDepthLanes - 1), kDepthLanes);
+      ro = W.ray_o[a];
+      rd = W.ray_d[a];
+      t = W.hit[hit_slot(W, k, a, i)].x;
+      sc = kBatch ? find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w)) : 0;
     }
-    S = mk(group_sum<kDepthLanes>(S.x), group_sum<kDepthLanes>(S.y), group_sum<kDepthLanes>(S.z));
-    if (at < T.n && (threadIdx.x & (kDepthLanes - 1)) == 0) {
+    const SceneEntry& E = kBatch ? W.ent[sc] : E0;
+    const float3 S = medium_depth_warp<kGrid == 2>(medium_view(E, W.ent + sc), xyz(ro), xyz(rd), t, on);
+    if (on && (threadIdx.x & (kDepthLanes - 1)) == 0) {
       s_S[0][i - tile] = S.x;
       s_S[1][i - tile] = S.y;
       s_S[2][i - tile] = S.z;
@@ -1046,7 +1049,7 @@ __global__ void __launch_bounds__(kShadeThreads, kShadeMinBlocks) k_shade(WsView
 // it itself.  A pass of its own: the march's accumulators need more
 // registers than the shading pass runs with.  March tiles, as in shade_march.
 // (Queued 32 at a time by each warp, a lane per segment, 16 views of 384x384
-// with a 64^3 grid took 2.07 ms; 1.51 now.)
+// with a 64^3 grid took 2.07 ms; 1.66 now.)
 template <bool kBatch, bool kHash>
 __global__ void __launch_bounds__(kTileThreads, 2) k_medium_forward(WsView W, int k, const SceneEntry E0) {
   chain_begin();
@@ -1072,29 +1075,43 @@ __global__ void __launch_bounds__(kTileThreads, 2) k_medium_forward(WsView W, in
       c_med += (uint32_t)steps + 1u;
       return steps;
     });
-    for (int at; march_group<kMomentLanes<kHash>>(T, at);) {
-      const int p = threadIdx.x & (kMomentLanes<kHash> - 1);
-      MediumMoments m;
-      m.S = m.dt = m.ox = m.oy = m.oz = m.dx = m.dy = m.dz = mk(0.f, 0.f, 0.f);
+    constexpr int kLanes = kMomentLanes<kHash>, kCols = 4 / kLanes;
+    for (int at; march_group<kLanes>(T, at);) {
+      const int p = threadIdx.x & (kLanes - 1);
+      const bool on = at < T.n;
       uint32_t a = 0;
-      if (at < T.n) {
+      float4 ro = make_float4(0.f, 0.f, 0.f, 0.f), rd = ro;
+      float t = 0.f;
+      int scene = 0;
+      if (on) {
         const uint32_t i = T.pos[at];
         a = start + i;
-        const float4 ro = W.ray_o[a], rd = W.ray_d[a];
-        const int scene = kBatch ? find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w)) : 0;
-        const SceneEntry& E = kBatch ? W.ent[scene] : E0;
-        m = medium_moments<kHash>(medium_view(E, W.ent + scene), xyz(ro), xyz(rd), W.hit[hit_slot(W, k, a, i)].x, p,
-                                  kMomentLanes<kHash>);
+        ro = W.ray_o[a];
+        rd = W.ray_d[a];
+        t = W.hit[hit_slot(W, k, a, i)].x;
+        scene = kBatch ? find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w)) : 0;
       }
-      float v[kMomFloats] = {m.S.x,  m.S.y,  m.S.z,  m.dt.x, m.dt.y, m.dt.z, m.ox.x, m.oy.x,
-                             m.oz.x, m.ox.y, m.oy.y, m.oz.y, m.ox.z, m.oy.z, m.oz.z, m.dx.x,
-                             m.dy.x, m.dz.x, m.dx.y, m.dy.y, m.dz.y, m.dx.z, m.dy.z, m.dz.z};
+      const SceneEntry& E = kBatch ? W.ent[scene] : E0;
+      const MomentSums<kLanes> v = medium_moments<kHash>(medium_view(E, W.ent + scene), xyz(ro), xyz(rd), t, on);
+      if (!on) continue;
+      const float vt[3] = {v.dt.x, v.dt.y, v.dt.z};
 #pragma unroll
-      for (int j = 0; j < kMomFloats; ++j) v[j] = group_sum<kMomentLanes<kHash>>(v[j]);
-      if (at < T.n) {
+      for (int j = 0; j < kCols; ++j) {
+        const float va[3] = {v.a[j].x, v.a[j].y, v.a[j].z}, vb[3] = {v.b[j].x, v.b[j].y, v.b[j].z};
+        const int col = kCols * p + j;
 #pragma unroll
-        for (int j = 0; j < kMomFloats; ++j)
-          if (j % kMomentLanes<kHash> == p) M[j * cap + a] = v[j];
+        for (int c = 0; c < 3; ++c) {
+          if (col == 0) {
+            M[(kMomS + c) * cap + a] = va[c];
+          } else {
+            M[(kMomDo + 3 * c + col - 1) * cap + a] = va[c];
+            M[(kMomDd + 3 * c + col - 1) * cap + a] = vb[c];
+          }
+        }
+      }
+      if (p == (medium_full_steps(t, E.gstep) & (kLanes - 1))) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) M[(kMomDt + c) * cap + a] = vt[c];
       }
     }
     __syncthreads();  // the list is made anew
