@@ -497,7 +497,8 @@ __global__ void __launch_bounds__(kCgThreads, 1) k_cg(const int32_t* __restrict_
   }
 }
 
-static void launch_cg(const TopoView& T, int32_t nv, float lam, const float* b, float* x, int iters, void* scratch,
+// Whether it was launched.
+static bool launch_cg(const TopoView& T, int32_t nv, float lam, const float* b, float* x, int iters, void* scratch,
                       cudaStream_t s) {
   CgView c = cg_view(scratch, nv);
   cudaMemsetAsync(c.word, 0, kCgWords * sizeof(ulonglong2), s);
@@ -515,8 +516,11 @@ static void launch_cg(const TopoView& T, int32_t nv, float lam, const float* b, 
   const int32_t *row = T.row, *col = T.col;
   void* args[] = {&row, &col, &nv, &chunk, &room, &lam, &b, &x, &c, &iters};
   const void* f = chunk <= kCgThreads ? (const void*)k_cg<true> : (const void*)k_cg<false>;
-  cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(words * sizeof(int32_t)));
-  cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(kCgThreads), args, (size_t)words * sizeof(int32_t), s);
+  // the same value from every thread and for every mesh: the attribute is the kernel's, not the launch's
+  if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgListWords * (int)sizeof(int32_t)) != cudaSuccess)
+    return false;
+  return cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(kCgThreads), args, (size_t)words * sizeof(int32_t), s) ==
+         cudaSuccess;
 }
 
 size_t smooth_scratch_bytes(int32_t nv, int32_t iters) {
@@ -611,7 +615,8 @@ void launch_large_steps_update(const void* topo, int32_t nv, int32_t nf, float l
   const int64_t n = 3 * (int64_t)nv;
   k_apply_m<<<g, 256, 0, s>>>(T.row, T.col, nv, lam, V, u);  // u = M V
   cudaMemsetAsync(gu, 0, (size_t)n * sizeof(float), s);
-  launch_cg(T, nv, lam, grad, gu, iters, cg, s);              // g_u = M^-1 dJ/dV
+  // g_u = M^-1 dJ/dV; without it the optimiser's state stays as it was (the caller reads the launch's error)
+  if (!launch_cg(T, nv, lam, grad, gu, iters, cg, s)) return;
   k_max_sq<<<g, 256, 0, s>>>(gu, n, sc);
   k_adam_uniform<<<g, 256, 0, s>>>(n, gu, m, u, sc, lr, b1, b2, eps);
   k_adam_scalars<<<1, 1, 0, s>>>(sc, b2);
