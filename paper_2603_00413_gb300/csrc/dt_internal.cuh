@@ -274,12 +274,13 @@ constexpr int kOrderBits = 22;
 constexpr uint32_t kOrderCounters = 1u << kOrderBits;
 constexpr size_t kOrderBytes = (((size_t)kOrderCounters + 1024) * sizeof(uint32_t) + 255) / 256 * 256;
 
-// index i with starts[i] <= x < starts[i+1] (n >= 1)
+// index i with starts[i] <= x < starts[i+1] (n >= 1); starts may be a table
+// that an earlier kernel of the chain writes, so no read-only loads
 __device__ __forceinline__ int find_scene(const uint32_t* starts, int n, uint32_t x) {
   int lo = 0, hi = n - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (__ldg(starts + mid) <= x) lo = mid; else hi = mid - 1;
+    if (starts[mid] <= x) lo = mid; else hi = mid - 1;
   }
   return lo;
 }

@@ -82,10 +82,11 @@ struct MediumSteps {
 // 32-bit arithmetic; the level keeps its low bits (tables are powers of two).
 constexpr uint32_t kHashPrimeY = 2654435761u, kHashPrimeZ = 805459861u;
 
+// (ordinary loads: the table is written by an earlier kernel of the chain)
 __device__ __forceinline__ GridLevel load_level(const GridLevel* p) {
   GridLevel L;
-  const int4 a = __ldg(reinterpret_cast<const int4*>(p));
-  const int4 b = __ldg(reinterpret_cast<const int4*>(p) + 1);
+  const int4 a = *reinterpret_cast<const int4*>(p);
+  const int4 b = *(reinterpret_cast<const int4*>(p) + 1);
   L.n = a.x;
   L.mask = (uint32_t)a.y;
   L.off = (uint32_t)a.z;
