@@ -384,19 +384,25 @@ __global__ void __launch_bounds__(kTileThreads, 3) k_medium_adjoint(WsView W, in
     for (int i = threadIdx.x; i < 6 * kTileMax; i += kTileThreads) (&s_motion[0][0])[i] = 0.f;
     __syncthreads();
     for (int at, l, part; march_unit(T, at, l, part);) {
-      if (at >= T.n) continue;
-      const uint32_t i = T.pos[at], a = start + i;
-      const float4 sv = med_side[i], ro = W.ray_o[a], rd = W.ray_d[a];
-      const int sc = kBatch ? scene_of(a) : 0;
+      bool on = at < T.n, gather = false;
+      float4 sv = make_float4(0.f, 0.f, 0.f, 0.f), ro = sv, rd = sv;
+      int sc = 0;
+      if (on) {
+        const uint32_t i = T.pos[at], a = start + i;
+        sv = med_side[i];
+        ro = W.ray_o[a];
+        rd = W.ray_d[a];
+        sc = kBatch ? scene_of(a) : 0;
+        // tape_mode 2: the samples' motion comes from the forward's moments
+        gather = k > 0 && !(W.mom && !isnan(W.mom[kMomS * W.cap + a]));
+      }
       const SceneEntry& E = kBatch ? W.ent[sc] : E0;
-      if (kBatch && l >= (kHash && E.glevels ? E.glevels : 1)) continue;
-      // tape_mode 2: the samples' motion comes from the forward's moments
-      const bool gather = k > 0 && !(W.mom && !isnan(W.mom[kMomS * W.cap + a]));
-      if (!gather && !E.dmu) continue;
+      if (kBatch && l >= (kHash && E.glevels ? E.glevels : 1)) on = false;
+      if (!gather && !E.dmu) on = false;
       float3 ob = mk(0.f, 0.f, 0.f), db = ob;
-      medium_level_adjoint<kHash>(medium_view(E, W.ent + sc), E.dmu, l, part, T.levels > kPartLevels, xyz(ro), xyz(rd), sv.w,
-                                  mk(sv.x, sv.y, sv.z), gather, ob, db);
-      if (gather) {
+      medium_level_adjoint<kHash>(medium_view(E, W.ent + sc), E.dmu, l, part, T.levels > kPartLevels, on, xyz(ro), xyz(rd),
+                                  sv.w, mk(sv.x, sv.y, sv.z), gather, ob, db);
+      if (on && gather) {
         atomicAdd(&s_motion[0][at], ob.x);
         atomicAdd(&s_motion[1][at], ob.y);
         atomicAdd(&s_motion[2][at], ob.z);

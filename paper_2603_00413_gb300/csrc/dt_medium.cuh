@@ -736,17 +736,19 @@ __device__ __forceinline__ void adjoint_walk(const float4* __restrict__ mu, floa
 
 // adjoint_walk over part `part` of a segment's samples (kPartSteps of them, or
 // all with `whole`) on level l of the hash texture, or on the dense grid (l =
-// 0): adds dJ/do and dJ/dd.
+// 0): adds dJ/do and dJ/dd.  Every lane of the warp calls (`on`: the lane has a
+// segment on level l).
 template <bool kHash>
-__device__ __forceinline__ void medium_level_adjoint(const MediumView& g, float4* dmu, int l, int part, bool whole,
+__device__ __forceinline__ void medium_level_adjoint(const MediumView& g, float4* dmu, int l, int part, bool whole, bool on,
                                                      float3 o, float3 d, float t, float3 sbar, bool gather, float3& ob,
                                                      float3& db) {
   const MediumSteps st(t, g, kHash && g.levels);
-  const int i0 = whole ? 0 : part * kPartSteps, i1 = whole ? st.m + 1 : min(i0 + kPartSteps, st.m + 1);
-  if (i0 >= i1) return;
+  const int i0 = whole ? 0 : part * kPartSteps;
+  const int i1 = !on ? i0 : whole ? st.m + 1 : min(i0 + kPartSteps, st.m + 1);
   const Lattice T = lattice_of<kHash>(g, l, o, d);
   float3 uo = mk(0.f, 0.f, 0.f), ud = uo;
-  if (__all_sync(__activemask(), lattice_inside(T, t))) adjoint_walk<true>(g.mu, dmu, T, st, i0, i1, sbar, gather, uo, ud);
+  // one copy of the walk for the warp, whichever its lanes need
+  if (__all_sync(kFull, i0 >= i1 || lattice_inside(T, t))) adjoint_walk<true>(g.mu, dmu, T, st, i0, i1, sbar, gather, uo, ud);
   else adjoint_walk<false>(g.mu, dmu, T, st, i0, i1, sbar, gather, uo, ud);
   ob = ob + mul(uo, T.scale);
   db = db + mul(ud, T.scale);
