@@ -348,6 +348,13 @@ __device__ __forceinline__ uint32_t ray_order_key(float3 o, float3 d, float3 lo,
 __device__ __forceinline__ uint32_t order_bucket(uint32_t key24, int bits, bool batch, uint32_t scene) {
   return batch ? (scene << (bits - 8)) | (key24 >> (32 - bits)) : key24 >> (24 - bits);
 }
+// The position in a level of n segments that entry i < n of its traversal order
+// names (order == nullptr: append order); false when the order is not one of the
+// level's, which a traversal reports (ST_STACK_OVERFLOW) instead of tracing.
+__host__ __device__ inline bool order_position(const uint32_t* order, uint32_t i, uint32_t n, uint32_t& pos) {
+  pos = order ? order[i] : i;
+  return pos < n;
+}
 // Counts a child in its bucket and stores the bucket at its position p of
 // the next level; b == ~0u: no child.
 __device__ __forceinline__ void order_count_child(uint32_t* count, uint32_t* kb, uint32_t b, uint32_t p) {

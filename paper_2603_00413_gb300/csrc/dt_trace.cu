@@ -366,8 +366,8 @@ __device__ __noinline__ void trace_level_exact(const WsView W, int k, int sorted
   uint32_t nvis = 0, ntest = 0;
   bool ok = true;
   for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    const uint32_t pos = sorted ? W.sflag[start + i] : i;
-    if (pos >= n) {
+    uint32_t pos;
+    if (!order_position(sorted ? W.sflag + start : nullptr, i, n, pos)) {
       ok = false;
       continue;
     }
@@ -526,8 +526,8 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
       if (qb > qe) qb = qe;
       if (cursor_done && qb >= qe) exhausted = true;
       if (!active && i < n) {
-        const uint32_t pos = order ? order[i] : i;
-        if (pos >= n) overflow = true;  // not a permutation of the level: reported, not traced
+        uint32_t pos;
+        if (!order_position(order, i, n, pos)) overflow = true;
         else {
           const uint32_t a = start + pos;
           // read once here: not allocated in L1, so they do not evict BVH
@@ -644,7 +644,7 @@ __global__ void __launch_bounds__(kSmallThreads) k_trace_small(WsView W, int k, 
   for (uint32_t w0 = ((threadIdx.x >> 5) * gridDim.x + blockIdx.x) * per; w0 < n; w0 += warps * per) {
     const uint32_t slot = (uint32_t)(lane >> 2);
     uint32_t pos = slot < per ? w0 + slot : n;
-    if (sorted && pos < n) pos = W.sflag[start + pos];
+    if (pos < n && !order_position(sorted ? W.sflag + start : nullptr, pos, n, pos)) overflow = true;
     const uint32_t a = start + pos;
     int node = -1, sp = 0, visits = 0, max_iter = 0, src = -1;
     float tmin = 0.f;
