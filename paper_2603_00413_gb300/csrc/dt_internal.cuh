@@ -93,6 +93,10 @@ constexpr int kTraceStack = 64;
 //    object against 5e-3 for the edges of a million-triangle mesh (node visits
 //    per ray 27.93 -> 28.00 on the 52k-triangle genus-2 mesh, 47.8 -> 48.0 on
 //    a 1.08M-triangle sphere).
+//  - node2x[4j .. 4j+3]: the same node with exact boxes in 64 bytes, for scenes
+//    that the grid cannot resolve (BvhHeader::coarse): child 0's box (lo.x, hi.x,
+//    lo.y, hi.y), child 1's, (c0 lo.z, hi.z, c1 lo.z, hi.z), the children as int
+//    bits.
 //  - tris[3i..3i+2] = leaf i's triangle: (v0, id), (e1, 0), (e2, 0).
 //  - leaf_tri[i] = triangle of leaf i.
 // ---------------------------------------------------------------------------
@@ -108,13 +112,12 @@ struct alignas(16) BvhHeader {
   int32_t corrupt;  // set by the build's validation pass when a reference is out of range
   float q[4];       // grid of the coded boxes: lower corner of the scene's box, step
   float hi[3];      // upper corner of the scene's box
-  // Nodes deep inside a cluster that the grid cannot resolve (counted by
-  // each refit): a scene that holds a detailed part some 1e-4 of its own
-  // size.  Above kQCoarse the rays use the exact boxes (see closest_hit_exact):
-  // coded, the part's boxes all look alike and a ray would test every triangle.
+  // Nodes inside clusters of triangles a few grid steps in size (counted by
+  // each refit, see k_node_boxes): a scene that holds a detailed part some 1e-2
+  // of its own size or less.  Above kQCoarse its rays use the exact boxes.
   int32_t coarse;
 };
-constexpr int kQCoarse = 16;
+constexpr int kQCoarse = 64;
 
 struct BvhView {
   BvhHeader* hdr;
@@ -124,6 +127,7 @@ struct BvhView {
   float4* box_leaf;  // [2 nf]
   float4* node4;     // [8 n_int] (at most n_int 4-wide nodes)
   uint4* node2;      // [2 n_int]
+  float4* node2x;    // [4 n_int]
   int32_t* bin_to4;  // [n_int]
   float4* tris;      // [3 nf]
   int32_t* leaf_tri; // [nf]
@@ -132,8 +136,8 @@ struct BvhView {
 __host__ __device__ inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
 struct BvhLayout {
-  size_t off_child, off_parent, off_box_int, off_box_leaf, off_node4, off_node2, off_bin_to4, off_tris, off_leaf,
-      total;
+  size_t off_child, off_parent, off_box_int, off_box_leaf, off_node4, off_node2, off_node2x, off_bin_to4, off_tris,
+      off_leaf, total;
   __host__ __device__ explicit BvhLayout(int32_t nf) {
     const size_t n_int = nf > 1 ? (size_t)nf - 1 : 1;
     size_t o = 256;
@@ -147,6 +151,7 @@ struct BvhLayout {
     off_box_leaf = take((size_t)nf * 2 * sizeof(float4));
     off_bin_to4 = take(n_int * sizeof(int32_t));
     off_leaf = take((size_t)nf * sizeof(int32_t));
+    off_node2x = take(n_int * 4 * sizeof(float4));
     total = o;
   }
 };
@@ -156,7 +161,7 @@ __host__ __device__ inline BvhView bvh_view(const void* base, int32_t nf) {
   char* b = (char*)base;
   return BvhView{(BvhHeader*)b, (int2*)(b + L.off_child), (int32_t*)(b + L.off_parent),
                  (float4*)(b + L.off_box_int), (float4*)(b + L.off_box_leaf), (float4*)(b + L.off_node4),
-                 (uint4*)(b + L.off_node2), (int32_t*)(b + L.off_bin_to4), (float4*)(b + L.off_tris),
+                 (uint4*)(b + L.off_node2), (float4*)(b + L.off_node2x), (int32_t*)(b + L.off_bin_to4), (float4*)(b + L.off_tris),
                  (int32_t*)(b + L.off_leaf)};
 }
 
@@ -182,7 +187,7 @@ struct WsHeader {
   unsigned long long counters[16];   // see CNT_*
   uint32_t ring;                     // level capacity of the hit ring (tape_mode 1), 0 = every hit kept
   uint32_t mom;                      // 1: the medium moments of tape_mode 2 follow the hit records
-  uint32_t exact;                    // 1: some scene's BvhHeader::coarse is above kQCoarse
+  uint32_t exact;                    // 1: some scene's rays use the exact boxes (BvhHeader::coarse)
 };
 
 enum { CNT_HITS = 0, CNT_MISSES, CNT_DISCARDED, CNT_BACKFACING, CNT_TIR, CNT_NODES, CNT_TRIS, CNT_MEDIUM };

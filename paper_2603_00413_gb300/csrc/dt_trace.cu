@@ -261,24 +261,66 @@ __device__ __forceinline__ bool slab_q(const RayQ& r, uint32_t x, uint32_t y, ui
   return tnear <= fminf(fminf(far_plane(r.x, x), far_plane(r.y, y)), fminf(far_plane(r.z, z), tmax));
 }
 
-// One visit of binary node `node`: of the children whose boxes are hit the
-// nearer is returned and the other pushed, and with none the stack is popped
-// (its bottom entry is kNoChild, the end of the search).  Leaves (~index, < 0)
-// go through the stack like nodes.  Selects and predicated accesses instead of
-// branches, as in test_leaf.
-__device__ __forceinline__ int visit_node2(const uint4* __restrict__ node2, int node, const RayQ& r, float tmin,
-                                           float tmax, int* stack, int& sp) {
-  uint4 a, b;
-  ld_node2(node2 + 2 * node, a, b);
-  const int c0 = (int)b.z, c1 = (int)b.w;
-  float t0, t1;
-  const bool h0 = slab_q(r, a.x, a.y, a.z, tmin, tmax, t0), h1 = slab_q(r, a.w, b.x, b.y, tmin, tmax, t1);
+// Of the children whose boxes are hit the nearer is returned and the other
+// pushed, and with none the stack is popped (its bottom entry is kNoChild, the end
+// of the search).  Leaves (~index, < 0) go through the stack like nodes.  Selects
+// and predicated accesses instead of branches, as in test_leaf.
+__device__ __forceinline__ int descend(bool h0, float t0, int c0, bool h1, float t1, int c1, int* stack, int& sp) {
   const bool swap = !h0 || (h1 && t1 < t0);
   int next = swap ? c1 : c0;
   if (h0 && h1) stack[sp] = swap ? c0 : c1;
   sp += h0 && h1 ? 1 : 0;
   if (!h0 && !h1) next = stack[--sp];
   return next;
+}
+
+// One visit of binary node `node` with coded boxes.
+__device__ __forceinline__ int visit_node2(const uint4* __restrict__ node2, int node, const RayQ& r, float tmin,
+                                           float tmax, int* stack, int& sp) {
+  uint4 a, b;
+  ld_node2(node2 + 2 * node, a, b);
+  float t0, t1;
+  const bool h0 = slab_q(r, a.x, a.y, a.z, tmin, tmax, t0), h1 = slab_q(r, a.w, b.x, b.y, tmin, tmax, t1);
+  return descend(h0, t0, (int)b.z, h1, t1, (int)b.w, stack, sp);
+}
+
+// The same with the exact boxes.
+__device__ __forceinline__ int visit_node2x(const float4* __restrict__ node2x, int node, float3 o, float3 idir, float tmin,
+                                            float tmax, int* stack, int& sp) {
+  float4 a, b, c, e;
+  ld_nc_v8(node2x + 4 * (size_t)node, a, b);
+  ld_nc_v8(node2x + 4 * (size_t)node + 2, c, e);
+  float t0, t1;
+  const bool h0 = slab(o, idir, a.x, a.y, a.z, a.w, c.x, c.y, tmin, tmax, t0);
+  const bool h1 = slab(o, idir, b.x, b.y, b.z, b.w, c.z, c.w, tmin, tmax, t1);
+  return descend(h0, t0, __float_as_int(e.x), h1, t1, __float_as_int(e.y), stack, sp);
+}
+
+// What a ray's search reads: the coded boxes, or the exact ones (node2x), for
+// which the x, y and z of `r` hold the reciprocal direction.  kNodes: known to
+// be one of them, or each ray's own.
+enum NodeKind { kCodedNodes, kExactNodes, kEitherNodes };
+struct RayNodes {
+  const uint4* node2;
+  const float4* node2x;
+  RayQ r;
+  bool exact;
+};
+template <int kNodes>
+__device__ __forceinline__ void ray_begin(RayNodes& q, float3 o, float3 d, const BvhHeader* __restrict__ bh) {
+  if (kNodes == kExactNodes || (kNodes == kEitherNodes && q.exact)) {
+    q.r.x.s = safe_inv(d.x);
+    q.r.y.s = safe_inv(d.y);
+    q.r.z.s = safe_inv(d.z);
+  } else {
+    q.r = ray_q(o, d, bh);
+  }
+}
+template <int kNodes>
+__device__ __forceinline__ int visit(const RayNodes& q, int node, float3 o, float tmin, float tmax, int* stack, int& sp) {
+  if (kNodes == kExactNodes || (kNodes == kEitherNodes && q.exact))
+    return visit_node2x(q.node2x, node, o, mk(q.r.x.s, q.r.y.s, q.r.z.s), tmin, tmax, stack, sp);
+  return visit_node2(q.node2, node, q.r, tmin, tmax, stack, sp);
 }
 
 // Up to kLeafEvery visits, until the next reference is a leaf, then up to
@@ -296,12 +338,12 @@ __device__ __forceinline__ int visit_node2(const uint4* __restrict__ node2, int 
 // pushes, which are checked here.
 constexpr int kLeafEvery = 6, kLeafTests = 2;
 constexpr int kStackWords = 1 + kTraceStack + kLeafEvery;
-__device__ __forceinline__ bool visit_group(const uint4* __restrict__ node2, const float4* __restrict__ tris,
-                                            const RayQ& r, float3 o, float3 d, int src, float tmin, int* stack,
-                                            int& sp, int& node, HitSoFar& h, int& visits, uint32_t& ntest,
-                                            bool& overflow) {
+template <int kNodes>
+__device__ __forceinline__ bool visit_group(const RayNodes& q, const float4* __restrict__ tris, float3 o, float3 d, int src,
+                                            float tmin, int* stack, int& sp, int& node, HitSoFar& h, int& visits,
+                                            uint32_t& ntest, bool& overflow) {
   for (const int end = visits + kLeafEvery; node >= 0 && visits < end; ++visits)
-    node = visit_node2(node2, node, r, tmin, h.t, stack, sp);
+    node = visit<kNodes>(q, node, o, tmin, h.t, stack, sp);
   for (int q = 0; q < kLeafTests && node < 0 && node != kNoChild; ++q) {
     test_leaf(tris, ~node, o, d, src, tmin, h, ntest);
     node = stack[--sp];
@@ -313,80 +355,9 @@ __device__ __forceinline__ bool visit_group(const uint4* __restrict__ node2, con
   return node == kNoChild;
 }
 
-// Closest hit through the exact boxes of the refit, for scenes that the coded
-// boxes' grid cannot resolve (BvhHeader::coarse); the same hits, slower.  A
-// tree traversal visits every node at most once, so more than max_iter = 2
-// n_int + 8 visits means a corrupt hierarchy: give up and flag it.
-__device__ __forceinline__ bool closest_hit_exact(const BvhHeader* bh, int32_t nf, float3 o, float3 d, int src,
-                                                  float tmin, int max_iter, HitSoFar& h, uint32_t& nvis,
-                                                  uint32_t& ntest) {
-  const BvhView B = bvh_view(bh, nf);
-  const float3 idir = mk(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
-  int stack[kTraceStack];
-  int sp = 0, node = 0, it = 0;
-  bool ok = true;
-  while (node >= 0) {
-    if (it >= max_iter) {
-      ok = false;
-      break;
-    }
-    ++it;
-    const int2 ch = B.bin_child[node];
-    int c[2] = {ch.x, ch.y};
-    float tn[2];
-    bool in[2];
-    for (int k = 0; k < 2; ++k) {
-      in[k] = false;
-      if (c[k] == kNoChild) continue;
-      const float4* bx = c[k] >= 0 ? B.box_int + 2 * c[k] : B.box_leaf + 2 * (~c[k]);
-      const float4 lo = bx[0], hi = bx[1];
-      const bool hb = slab(o, idir, lo.x, hi.x, lo.y, hi.y, lo.z, hi.z, tmin, h.t, tn[k]);
-      if (hb && c[k] < 0) test_leaf(B.tris, ~c[k], o, d, src, tmin, h, ntest);
-      in[k] = hb && c[k] >= 0;
-    }
-    if (in[0] && in[1]) {
-      const int first = tn[1] < tn[0] ? 1 : 0;
-      if (sp < kTraceStack) stack[sp++] = c[1 - first]; else ok = false;
-      node = c[first];
-    } else {
-      node = in[0] ? c[0] : in[1] ? c[1] : sp > 0 ? stack[--sp] : -1;
-    }
-  }
-  nvis += (uint32_t)it;
-  return ok;
-}
-
-// Level k of a render one of whose scenes needs the exact boxes
-// (WsHeader::exact): a function of its own, called before the traversal's
-// loop, so that the loop's registers need not live across the call.
-__device__ __noinline__ void trace_level_exact(const WsView W, int k, int sorted) {
-  WsHeader* H = W.hdr;
-  const uint32_t n = level_size(H, k), start = H->level_start[k];
-  const int n_scenes = W.th->n;
-  uint32_t nvis = 0, ntest = 0;
-  bool ok = true;
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    uint32_t pos;
-    if (!order_position(sorted ? W.sflag + start : nullptr, i, n, pos)) {
-      ok = false;
-      continue;
-    }
-    const uint32_t a = start + pos;
-    const float4 ro = W.ray_o[a], rd = W.ray_d[a], rw = W.ray_w[a];
-    const SceneEntry& E = W.ent[find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w))];
-    HitSoFar h{INFINITY, -1, W.hit + hit_slot(W, k, a, pos)};
-    if (E.bh->corrupt) ok = false;
-    else ok &= closest_hit_exact(E.bh, E.nf, xyz(ro), xyz(rd), __float_as_int(rw.w), E.t_min, E.max_iter, h, nvis, ntest);
-    if (h.tri < 0) *h.rec = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-  }
-  warp_add_u64(&H->counters[CNT_NODES], nvis);
-  warp_add_u64(&H->counters[CNT_TRIS], ntest);
-  if (__any_sync(kFull, !ok) && (threadIdx.x & 31) == 0) atomicOr(&H->status, ST_STACK_OVERFLOW);
-}
-
-// The 4-wide visit of the persistent traversal, with hit leaves queued as
-// in visit_node2_deferred (the caller visits only while nothing is pending,
-// so four slots suffice).
+// The 4-wide visit of the persistent traversal.  A leaf that is hit is queued in
+// the lane's pending slots, whose triangles the warp tests together after a few
+// visits (the caller visits only while nothing is pending, so four slots suffice).
 __device__ __forceinline__ void push_pending4(int leaf, int& p0, int& p1, int& p2, int& p3) {
   if (p0 < 0) p0 = leaf;
   else if (p1 < 0) p1 = leaf;
@@ -451,15 +422,15 @@ __device__ __forceinline__ int visit_node4_deferred(const float4* __restrict__ n
 constexpr int kTraceClaim = 32;  // segments a warp claims from the level cursor at once (at least its lanes)
 constexpr int kTraceThreads = 128;
 
-template <int kMinBlocks, int kWidth, bool kBatch>
-__global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, int k, int steps, int refill,
-                                                           const SceneEntry E0, int sorted) {
-  chain_begin();
+struct TraceCounts {
+  uint32_t nvis, ntest;
+  bool overflow;
+};
+
+template <int kWidth, bool kBatch, int kNodes>
+__device__ __forceinline__ TraceCounts trace_level(const WsView& W, int k, int steps, int refill, const SceneEntry& E0,
+                                                   int sorted) {
   WsHeader* H = W.hdr;
-  if (kWidth == 2 && H->exact) {
-    trace_level_exact(W, k, sorted);
-    return;
-  }
   uint32_t* cursor = &H->fetch[k];
   const int n_scenes = kBatch ? W.th->n : 1;
   const uint32_t n = level_size(H, k);
@@ -472,12 +443,11 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
   bool overflow = false;
   bool active = false, exhausted = false;
   float3 o = mk(0.f, 0.f, 0.f), d = o, idir = o;  // idir: the 4-wide nodes' slab tests
-  RayQ rq = {};                                   // the binary nodes'
+  RayNodes rn = {E0.node2, nullptr, {}, false};  // the binary nodes'
   int src = -1, node = 0, sp = 0, iters = 0;
   int max_iter = kBatch ? 0 : (E0.bh->corrupt ? 0 : E0.max_iter);  // a tree that failed validation is not traced
   float tmin = E0.t_min;
   const BvhHeader* bh = E0.bh;
-  const uint4* node2 = E0.node2;
   const float4* node4 = E0.node4;
   const float4* tris = E0.tris;
   HitSoFar h{INFINITY, -1, nullptr};
@@ -536,7 +506,7 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
           if (kBatch) {
             const SceneEntry& E = W.ent[find_scene(W.th->starts, n_scenes, __float_as_uint(ro.w))];
             bh = E.bh;
-            node2 = E.node2;
+            rn.node2 = E.node2;
             node4 = E.node4;
             tris = E.tris;
             max_iter = bh->corrupt ? 0 : E.max_iter;
@@ -545,7 +515,13 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
           o = xyz(ro);
           d = xyz(rd);
           if (kWidth == 4) idir = mk(safe_inv(d.x), safe_inv(d.y), safe_inv(d.z));
-          else rq = ray_q(o, d, bh);
+          else {
+            if (kNodes == kEitherNodes) {
+              rn.exact = bh->coarse > kQCoarse;
+              rn.node2x = bvh_view(bh, bh->nf).node2x;
+            }
+            ray_begin<kNodes>(rn, o, d, bh);
+          }
           src = __float_as_int(rw.w);
           h = HitSoFar{INFINITY, -1, W.hit + hit_slot(W, k, a, pos)};
           node = 0;
@@ -565,7 +541,7 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
     if (!done) {
       if (kWidth == 2) {
         while (st < steps && !done)
-          done = visit_group(node2, tris, rq, o, d, src, tmin, stack, sp, node, h, st, ntest, overflow);
+          done = visit_group<kNodes>(rn, tris, o, d, src, tmin, stack, sp, node, h, st, ntest, overflow);
       } else {
         int p0 = -1, p1 = -1, p2 = -1, p3 = -1;
         while (st < steps) {
@@ -592,18 +568,44 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, i
       active = false;
     }
   }
+  return TraceCounts{nvis, ntest, overflow};
+}
+
+// Level k of a render one of whose scenes needs the exact boxes
+// (WsHeader::exact): every ray searches its own scene's kind of nodes.  A function
+// of its own, so that the common case keeps its registers (inlined: 40 meshes 1 %
+// slower), and a copy of it per register budget.
+template <int kMinBlocks, bool kBatch>
+__device__ __noinline__ void trace_level_either(const WsView W, int k, int steps, int refill, int sorted) {
+  const TraceCounts c = trace_level<2, kBatch, kEitherNodes>(W, k, steps, refill, W.ent[0], sorted);
+  warp_add_u64(&W.hdr->counters[CNT_NODES], c.nvis);
+  warp_add_u64(&W.hdr->counters[CNT_TRIS], c.ntest);
+  if (__any_sync(kFull, c.overflow) && (threadIdx.x & 31) == 0) atomicOr(&W.hdr->status, ST_STACK_OVERFLOW);
+}
+
+template <int kMinBlocks, int kWidth, bool kBatch>
+__global__ void __launch_bounds__(kTraceThreads, kMinBlocks) k_trace(WsView W, int k, int steps, int refill,
+                                                           const SceneEntry E0, int sorted) {
+  chain_begin();
+  WsHeader* H = W.hdr;
+  if (kWidth == 2 && H->exact) {
+    trace_level_either<kMinBlocks, kBatch>(W, k, steps, refill, sorted);
+    return;
+  }
+  const TraceCounts c = trace_level<kWidth, kBatch, kCodedNodes>(W, k, steps, refill, E0, sorted);
+  const uint32_t lane = threadIdx.x & 31;
   // the visit and test counts, summed over the CTA first: with a small level
   // spread over every warp, one atomic per warp on these two addresses would
   // queue thousands of atomics at the end of the launch
   __shared__ unsigned long long s_count[2];
   if (threadIdx.x == 0) s_count[0] = s_count[1] = 0ull;
   __syncthreads();
-  const unsigned wv = __reduce_add_sync(kFull, nvis), wt = __reduce_add_sync(kFull, ntest);
+  const unsigned wv = __reduce_add_sync(kFull, c.nvis), wt = __reduce_add_sync(kFull, c.ntest);
   if (lane == 0) {
     if (wv) atomicAdd(&s_count[0], (unsigned long long)wv);
     if (wt) atomicAdd(&s_count[1], (unsigned long long)wt);
   }
-  if (__any_sync(kFull, overflow) && lane == 0) atomicOr(&H->status, ST_STACK_OVERFLOW);
+  if (__any_sync(kFull, c.overflow) && lane == 0) atomicOr(&H->status, ST_STACK_OVERFLOW);
   __syncthreads();
   if (threadIdx.x == 0 && s_count[0]) atomicAdd(&H->counters[CNT_NODES], s_count[0]);
   if (threadIdx.x == 1 && s_count[1]) atomicAdd(&H->counters[CNT_TRIS], s_count[1]);
@@ -737,16 +739,30 @@ __global__ void __launch_bounds__(kSmallThreads) k_trace_small(WsView W, int k, 
   if (__any_sync(kFull, overflow) && lane == 0) atomicOr(&H->status, ST_STACK_OVERFLOW);
 }
 
+// Closest hit of one ray; false when the search gave up.
+template <int kNodes>
+__device__ __forceinline__ bool closest_hit(RayNodes& q, const float4* __restrict__ tris, float3 o, float3 d, int src,
+                                            const BvhHeader* bh, float tmin, int max_iter, HitSoFar& h) {
+  ray_begin<kNodes>(q, o, d, bh);
+  int stack[kStackWords];
+  stack[0] = kNoChild;
+  int sp = 1, node = 0, visits = 0;
+  uint32_t ntest = 0;
+  bool overflow = false;
+  while (!visit_group<kNodes>(q, tris, o, d, src, tmin, stack, sp, node, h, visits, ntest, overflow))
+    if (visits >= max_iter) return false;
+  return !overflow;
+}
+
 // Closest hit of arbitrary rays (tooling and tests).
-__global__ void __launch_bounds__(128) k_closest_hit_rays(const uint4* __restrict__ nodes,
+__global__ void __launch_bounds__(128) k_closest_hit_rays(const uint4* __restrict__ nodes, const float4* __restrict__ exact,
                                                           const float4* __restrict__ tris, const float* __restrict__ o,
                                                           const float* __restrict__ d, const int32_t* __restrict__ src,
                                                           int32_t n, const BvhHeader* bh, float tmin, int max_iter,
                                                           int32_t* __restrict__ tri, float* __restrict__ tbb) {
-  const bool corrupt = bh->corrupt != 0, exact = bh->coarse > kQCoarse;
+  const bool corrupt = bh->corrupt != 0, coarse = bh->coarse > kQCoarse;
+  RayNodes q = {nodes, exact, {}, coarse};
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    uint32_t nv = 0, nt = 0;
-    bool ovf = false;
     if (corrupt) {
       tri[i] = -2;
       continue;
@@ -755,20 +771,9 @@ __global__ void __launch_bounds__(128) k_closest_hit_rays(const uint4* __restric
     const int s = src ? src[i] : -1;
     float4 rec = make_float4(0.f, 0.f, 0.f, 0.f);
     HitSoFar h{INFINITY, -1, &rec};
-    if (exact) {
-      ovf = !closest_hit_exact(bh, bh->nf, ro, rd, s, tmin, max_iter, h, nv, nt);
-    } else {
-      const RayQ rq = ray_q(ro, rd, bh);
-      int stack[kStackWords];
-      stack[0] = kNoChild;
-      int sp = 1, node = 0, visits = 0;
-      while (!visit_group(nodes, tris, rq, ro, rd, s, tmin, stack, sp, node, h, visits, nt, ovf))
-        if (visits >= max_iter) {
-          ovf = true;
-          break;
-        }
-    }
-    tri[i] = ovf ? -2 : h.tri;
+    const bool ok = coarse ? closest_hit<kExactNodes>(q, tris, ro, rd, s, bh, tmin, max_iter, h)
+                           : closest_hit<kCodedNodes>(q, tris, ro, rd, s, bh, tmin, max_iter, h);
+    tri[i] = ok ? h.tri : -2;
     tbb[3 * i] = rec.x;
     tbb[3 * i + 1] = rec.y;
     tbb[3 * i + 2] = rec.z;
@@ -1366,7 +1371,7 @@ void launch_closest_hit(const void* bvh, int32_t nf, const float* o, const float
   BvhView B = bvh_view(bvh, nf);
   int b = (n + 127) / 128;
   if (b > 8 * num_sms()) b = 8 * num_sms();
-  k_closest_hit_rays<<<b > 0 ? b : 1, 128, 0, s>>>(B.node2, B.tris, o, d, src, n, B.hdr, tmin,
+  k_closest_hit_rays<<<b > 0 ? b : 1, 128, 0, s>>>(B.node2, B.node2x, B.tris, o, d, src, n, B.hdr, tmin,
                                                     traversal_limit(nf), tri, tbb);
 }
 
