@@ -409,6 +409,7 @@ __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float* __restrict_
   chain_begin();
   __shared__ int s_arrive[kRefitLeaves];
   __shared__ float s_box[2][6][kRefitLeaves];  // of the left and the right child
+  if (B.hdr->corrupt) return;  // a tree that failed validation: its leaves may be unset
   const int n_int = B.hdr->n_int, tid = threadIdx.x;
   if (blockIdx.x == 0 && tid == 0) B.hdr->coarse = 0;  // counted by k_node_boxes
   for (int64_t tile = (int64_t)blockIdx.x * kRefitLeaves; tile < nf; tile += (int64_t)gridDim.x * kRefitLeaves) {
@@ -1211,6 +1212,7 @@ __global__ void __launch_bounds__(32 * kSahSmallWarps) k_sah_small(SahView S, Bv
   chain_begin();
   static_assert(kSahTiny == 4, "a tiny range has four lanes");
   __shared__ SahSmallShared sh;
+  if (B.hdr->corrupt) return;  // the large levels gave up: their permutation is incomplete
   const int n_int = B.hdr->n_int;
   const int tid = threadIdx.x, w = tid >> 5;
   const int nsmall = min(S.st->n_small, S.max_small);
@@ -1375,6 +1377,7 @@ constexpr float kQPatch = 26.0f;
 
 __global__ void k_node_boxes(BvhView B) {
   chain_begin();
+  if (B.hdr->corrupt) return;
   const int n_int = B.hdr->n_int, n4 = B.hdr->n4;
   float3 rlo = mk(INFINITY, INFINITY, INFINITY), rhi = mk(-INFINITY, -INFINITY, -INFINITY);
   const int2 root = B.bin_child[0];
