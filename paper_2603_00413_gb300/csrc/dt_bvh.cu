@@ -1545,7 +1545,8 @@ void launch_refit(const float* V, const int32_t* F, int32_t nf, void* bvh, void*
 // tasks take free splits to depth kSahSmallFreeDepth, then at most
 // log2(kSahSmall) median levels: the tree is at most 63 deep, within the
 // traversal's 64-entry stack.
-static void launch_sah_topology(const float* V, const int32_t* F, int32_t nf, BvhView& B, BuildScratch& S,
+// False when it could not be launched: the tree is then marked corrupt.
+static bool launch_sah_topology(const float* V, const int32_t* F, int32_t nf, BvhView& B, BuildScratch& S,
                                 cudaStream_t s) {
   launch_chained(k_sah_prims, grid_for(nf, 256), 256, 0, s, V, F, nf, S.bounds, S.sah, B);
   int levels = 0;
@@ -1565,11 +1566,18 @@ static void launch_sah_topology(const float* V, const int32_t* F, int32_t nf, Bv
     if (blocks > most) blocks = most;
     const uint32_t* bounds = S.bounds;
     void* args[] = {&nf, &levels, &bounds, &S.sah, &B};
-    cudaLaunchCooperativeKernel((const void*)k_sah_levels, dim3(blocks), dim3(kSahThreads), args, 0, s);
+    const bool launched = launch_cooperative(blocks, [&](int n) {
+      return cudaLaunchCooperativeKernel((const void*)k_sah_levels, dim3(n), dim3(kSahThreads), args, 0, s);
+    });
+    if (!launched) {
+      cudaMemsetAsync(&B.hdr->corrupt, 1, sizeof(B.hdr->corrupt), s);
+      return false;
+    }
   }
   ProfScope ps("sah_small", s);
   // at most one task per two triangles, a CTA each; about kSahSmall / 2 in practice
   launch_chained(k_sah_small, grid_for(nf / 32 + 1, 1), 32 * kSahSmallWarps, 0, s, S.sah, B);
+  return true;
 }
 
 void launch_scan_exclusive(const uint32_t* src, uint32_t* dst, int32_t m, uint32_t* totals, cudaStream_t s) {
@@ -1589,7 +1597,7 @@ void launch_build(const float* V, const int32_t* F, int32_t nf, void* bvh, void*
     ProfScope ps(sah ? "sah_build" : "lbvh_build", s);
     k_bvh_header<<<1, 256, 0, s>>>(B.hdr, nf, S.bounds, S.sah.st);
     if (sah) {
-      launch_sah_topology(V, F, nf, B, S, s);
+      if (!launch_sah_topology(V, F, nf, B, S, s)) return;
     } else {
       k_centroid_bounds<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, S.bounds);
       k_morton<<<grid_for(nf, 256), 256, 0, s>>>(V, F, nf, S.bounds, S.keys_a, S.vals_a);

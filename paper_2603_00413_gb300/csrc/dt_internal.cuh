@@ -535,6 +535,21 @@ inline void launch_chained(void (*kernel)(P...), dim3 grid, int threads, size_t 
   cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// Cooperative launch of at most `blocks` CTAs of a kernel that works with any
+// number of them; try_launch(blocks) launches that many.  Where the stream's
+// context has not the SMs to hold them at once (a green context, an MPS share: the
+// device's SM count does not tell), half as many are tried, down to one.
+template <class Launch>
+inline bool launch_cooperative(int blocks, const Launch& try_launch) {
+  cudaError_t e = try_launch(blocks);
+  while (e == cudaErrorCooperativeLaunchTooLarge && blocks > 1) {
+    cudaGetLastError();  // not an error of the call: a smaller grid follows
+    blocks = (blocks + 1) / 2;
+    e = try_launch(blocks);
+  }
+  return e == cudaSuccess;
+}
+
 // Per-kernel event timing (dt_profile_enable).  Scoped: records a start event
 // on construction and a stop event on destruction when profiling is on.
 struct ProfScope {

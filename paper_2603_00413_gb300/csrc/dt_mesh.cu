@@ -505,22 +505,24 @@ static bool launch_cg(const TopoView& T, int32_t nv, float lam, const float* b, 
   int blocks = (nv + kCgThreads - 1) / kCgThreads;
   const int most = num_sms() < kCgMaxBlocks ? num_sms() : kCgMaxBlocks;
   if (blocks > most) blocks = most;
-  int32_t chunk = (nv + blocks - 1) / blocks;
-  // list starts and room for lists of eight neighbours a vertex (a closed mesh
-  // has six on average), as far as they fit; the starts alone exceed shared
-  // memory past 7.7M vertices, and are then read where they are (room -1)
-  int64_t words = (int64_t)chunk * 9 + 1;
-  if (words > kCgListWords) words = kCgListWords;
-  int32_t room = words > chunk ? (int32_t)(words - (chunk + 1)) : -1;
-  if (room < 0) words = 0;
-  const int32_t *row = T.row, *col = T.col;
-  void* args[] = {&row, &col, &nv, &chunk, &room, &lam, &b, &x, &c, &iters};
-  const void* f = chunk <= kCgThreads ? (const void*)k_cg<true> : (const void*)k_cg<false>;
-  // the same value from every thread and for every mesh: the attribute is the kernel's, not the launch's
-  if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgListWords * (int)sizeof(int32_t)) != cudaSuccess)
-    return false;
-  return cudaLaunchCooperativeKernel(f, dim3(blocks), dim3(kCgThreads), args, (size_t)words * sizeof(int32_t), s) ==
-         cudaSuccess;
+  return launch_cooperative(blocks, [&](int n) {
+    int32_t chunk = (nv + n - 1) / n;
+    // list starts and room for lists of eight neighbours a vertex (a closed mesh
+    // has six on average), as far as they fit; the starts alone exceed shared
+    // memory past 7.7M vertices, and are then read where they are (room -1)
+    int64_t words = (int64_t)chunk * 9 + 1;
+    if (words > kCgListWords) words = kCgListWords;
+    int32_t room = words > chunk ? (int32_t)(words - (chunk + 1)) : -1;
+    if (room < 0) words = 0;
+    const int32_t *row = T.row, *col = T.col;
+    void* args[] = {&row, &col, &nv, &chunk, &room, &lam, &b, &x, &c, &iters};
+    const void* f = chunk <= kCgThreads ? (const void*)k_cg<true> : (const void*)k_cg<false>;
+    // the same value from every thread and for every mesh: the attribute is the kernel's, not the launch's
+    const cudaError_t e =
+        cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kCgListWords * (int)sizeof(int32_t));
+    if (e != cudaSuccess) return e;
+    return cudaLaunchCooperativeKernel(f, dim3(n), dim3(kCgThreads), args, (size_t)words * sizeof(int32_t), s);
+  });
 }
 
 size_t smooth_scratch_bytes(int32_t nv, int32_t iters) {
