@@ -568,7 +568,11 @@ __global__ void k_zero_grads(WsView W) {
     for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < ne; i += (size_t)gridDim.x * blockDim.x)
       E.denv[i] = 0.f;
   }
-  if (blockIdx.x == 0 && threadIdx.x < 4) scene_sums(W, blockIdx.y)[threadIdx.x] = 0.0;
+  if (blockIdx.x == 0 && threadIdx.x < 4) {
+    scene_sums(W, blockIdx.y)[threadIdx.x] = 0.0;
+    if (threadIdx.x == 0) E.dior[0] = 0.f;
+    else E.dsigma[threadIdx.x - 1] = 0.f;
+  }
 }
 
 // Eq. 13 backward for every scene (blockIdx.y = scene): dN -> dV, on the
@@ -596,14 +600,13 @@ __global__ void k_face_normals_backward_table(const SceneEntry* ent) {
 }
 
 // the caller's dV [nv][3], dIoR and dsigma from the accumulators (blockIdx.y =
-// scene)
+// scene); scenes that share an IoR or sigma gradient add up in it
 __global__ void k_finish_grads_table(WsView W) {
   chain_begin();
   const SceneEntry& E = W.ent[blockIdx.y];
   if (blockIdx.x == 0 && threadIdx.x < 4) {
     const float g = (float)scene_sums(W, blockIdx.y)[threadIdx.x];
-    if (threadIdx.x == 0) E.dior[0] = g;
-    else E.dsigma[threadIdx.x - 1] = g;
+    atomicAdd(threadIdx.x == 0 ? E.dior : E.dsigma + (threadIdx.x - 1), g);
   }
   const float4* dV4 = acc_dV4(E);
   for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < E.nv; v += gridDim.x * blockDim.x) {
