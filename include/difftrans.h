@@ -303,7 +303,8 @@ dt_status dt_read_stats(const void* d_ws, size_t ws_bytes, dt_stats* out, dt_str
  *
  * The scene, views and params must be those of the dt_render that filled
  * d_ws (ws_bytes as passed to it), and that render must have finished with
- * status DT_OK; d_ws is only read, and the vertices must not have changed
+ * status DT_OK; d_ws is only read (backward passes over one tape may overlap,
+ * each with a d_bws of its own), and the vertices must not have changed
  * since the forward.  dt_backward_workspace_size: bytes of the backward scratch
  * d_bws (256-byte aligned) for a render whose largest level held max_level
  * segments (dt_stats.max_level); pass the same max_level to
@@ -327,7 +328,8 @@ dt_status dt_render_backward(const dt_scene* scene, const dt_views* views, const
  * global across the batch (entry i's samples follow entry i-1's) for
  * dt_dump_segments.  n in [1, 256]; the total of primary rays < 2^32.
  * The backward takes d_grad_out, d_grad_V, d_grad_ior, d_grad_sigma of each
- * entry (outputs overwritten) and a scratch sized by
+ * entry (outputs overwritten; entries may share a d_grad_ior or d_grad_sigma,
+ * which then holds the sum of their gradients) and a scratch sized by
  * dt_batch_backward_workspace_size.  Entries are host memory read during
  * the call; the library keeps no pointer to them.
  * ------------------------------------------------------------------------ */

@@ -42,11 +42,12 @@ struct AdjRecords {
   }
 };
 
-// backward scratch: two level buffers of adjoint records and the dN/dV
-// accumulators
+// backward scratch: two level buffers of adjoint records, the pass's own scene
+// table and IoR and sigma sums (the tape is only read, so that passes over one tape
+// may run at the same time) and, from off_dN, the scenes' dN/dV accumulators
 struct BwsLayout {
-  size_t off_buf[2][3], off_med, off_dN, total;
-  BwsLayout(unsigned long long max_level, int32_t nv) {
+  size_t off_buf[2][3], off_med, off_th, off_ent, off_sums, off_dN;
+  BwsLayout(unsigned long long max_level, int n_scenes) {
     size_t o = 0;
     for (int k = 0; k < 2; ++k) {
       off_buf[k][0] = o;
@@ -58,8 +59,10 @@ struct BwsLayout {
     // segment with an absorption grid, zeros otherwise
     off_med = o;
     o = align_up(o + (size_t)max_level * sizeof(float4), 256);
-    off_dN = o;
-    total = align_up(off_dN + (size_t)nv * 2 * sizeof(float4), 256);
+    off_th = o;
+    off_ent = align_up(off_th + sizeof(TableHeader), 256);
+    off_sums = align_up(off_ent + (size_t)n_scenes * sizeof(SceneEntry), 256);
+    off_dN = align_up(off_sums + (size_t)n_scenes * 4 * sizeof(double), 256);
   }
   AdjRecords records(void* base, int k) const {
     char* b = (char*)base;
@@ -77,7 +80,7 @@ __device__ __forceinline__ float4* acc_dN4(const SceneEntry& E) { return reinter
 __device__ __forceinline__ float4* acc_dV4(const SceneEntry& E) { return reinterpret_cast<float4*>(E.dN) + E.nv; }
 
 // Sums of the IoR and sigma gradients, per CTA in shared memory and per scene
-// in the order counters of the workspace, which only a forward uses.  The terms
+// in the backward's scratch (WsView::order_count).  The terms
 // of a closed surface cancel to a thousandth of their absolute sum, so the CTAs'
 // sums are added in 64 bits, and a warp's lanes among themselves first: with a
 // float atomic per lane and per CTA, in the order in which they came, two sweeps
@@ -87,7 +90,6 @@ __device__ __forceinline__ float4* acc_dV4(const SceneEntry& E) { return reinter
 __device__ __forceinline__ double* scene_sums(const WsView& W, int scene) {
   return reinterpret_cast<double*>(W.order_count) + 4 * scene;
 }
-static_assert(kMaxBatch * 4 * sizeof(double) <= kOrderBytes, "the sums must fit the order counters");
 
 // T: double for one scene, where a warp adds once; float in a batch, whose
 // lanes change scenes (64-bit atomics on shared memory: 2.7 -> 3.8 ms).
@@ -735,15 +737,18 @@ void launch_l2_loss_grad(const float* img, const float* target, int64_t n, float
 void launch_write_table(const WsView& W, const TableHeader& th, const SceneEntry* entries, int n, bool clear,
                         cudaStream_t s);
 
-// Backward of a table of scenes over the tape in ws: rewrites the table with
-// the gradient pointers, zeroes the gradients, sweeps k = D..0, then the
+// Backward of a table of scenes over the tape in ws: writes a table of its own,
+// with the gradient pointers, zeroes the gradients, sweeps k = D..0, then the
 // vertex-normal adjoint of every scene.
 void launch_backward_table(const TableHeader& th, const SceneEntry* entries, const void* ws, unsigned long long cap,
                            unsigned long long ring, bool mom, void* bws, unsigned long long max_level, cudaStream_t s) {
-  WsView W = ws_view(ws, cap, ring, mom);
-  BwsLayout L(max_level, 0);
-  const AdjRecords buf[2] = {L.records(bws, 0), L.records(bws, 1)};
   const int n = th.n;
+  BwsLayout L(max_level, n);
+  WsView W = ws_view(ws, cap, ring, mom);
+  W.th = (TableHeader*)((char*)bws + L.off_th);
+  W.ent = (SceneEntry*)((char*)bws + L.off_ent);
+  W.order_count = (uint32_t*)((char*)bws + L.off_sums);
+  const AdjRecords buf[2] = {L.records(bws, 0), L.records(bws, 1)};
   launch_write_table(W, th, entries, n, false, s);
   int max_nv = 1, max_nf = 1;
   for (int i = 0; i < n; ++i) {
@@ -806,18 +811,18 @@ void launch_backward_table(const TableHeader& th, const SceneEntry* entries, con
   launch_chained(k_finish_grads_table, dim3(vb, n), 256, 0, s, W);
 }
 
-// The backward scratch of a table: the two level buffers, then every
+// The backward scratch of a table: BwsLayout, then every
 // scene's dN and dV accumulators (float4 per vertex each).  assign_dN
 // points each entry's dN at its pair.
 size_t backward_ws_bytes_table(unsigned long long max_level, const SceneEntry* entries, int n) {
-  BwsLayout L(max_level, 0);
+  BwsLayout L(max_level, n);
   size_t o = L.off_dN;
   for (int i = 0; i < n; ++i) o = align_up(o + (size_t)entries[i].nv * 2 * sizeof(float4), 256);
   return o;
 }
 
 void assign_dN(SceneEntry* entries, int n, void* bws, unsigned long long max_level) {
-  BwsLayout L(max_level, 0);
+  BwsLayout L(max_level, n);
   size_t o = L.off_dN;
   for (int i = 0; i < n; ++i) {
     entries[i].dN = (float*)((char*)bws + o);

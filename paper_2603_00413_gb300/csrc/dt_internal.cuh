@@ -303,7 +303,7 @@ struct WsView {
   unsigned long long cap;
   uint32_t ring;  // 0: hit[a] for arena index a; else hit[(k & 1) ring + i] for position i in level k
   uint32_t* order_count;  // traversal order: kOrderCounters bucket counters, then the scan's span totals; in a
-                          // backward pass the scenes' IoR and sigma sums
+                          // backward pass the scenes' IoR and sigma sums, in its scratch
   float* mom;     // tape_mode 2: kMomFloats arrays of cap floats (medium moments, see below); else null
 };
 

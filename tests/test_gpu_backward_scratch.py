@@ -1,4 +1,6 @@
-"""Scenes of a batch that share an IoR or sigma gradient add up in it."""
+"""A backward pass only reads the tape: it leaves the workspace's bytes as they
+are, and two passes over one tape may run at once on two streams.  Scenes of a
+batch that share an IoR or sigma gradient add up in it."""
 import pytest
 import torch
 
@@ -22,6 +24,33 @@ def _item(gs):
 def _near(got, want):
     for x, y in zip(got, want):  # sums of the same terms in another order
         assert float((x - y).abs().max()) <= 1e-5 * float(y.abs().max()) + 1e-7
+
+
+def test_the_workspace_keeps_its_bytes():
+    img, tape = _scene(0).render()
+    before = tape.ws.buf.clone()
+    dt.render_backward(tape, img)
+    assert torch.equal(tape.ws.buf, before)
+    imgs, tape = dt.render_batch([_item(_scene(k)) for k in range(3)])
+    before = tape.ws.buf.clone()
+    dt.render_batch_backward(tape, imgs)
+    assert torch.equal(tape.ws.buf, before)
+
+
+def test_two_passes_over_one_tape():
+    img, tape = _scene(1, 256).render()
+    seeds = [img, 1.0 - 2.0 * img]
+    want = [[g.clone() for g in dt.render_backward(tape, s)] for s in seeds]
+    torch.cuda.synchronize()
+    streams = [torch.cuda.Stream() for _ in seeds]
+    for _ in range(10):
+        got = []
+        for s, seed in zip(streams, seeds):
+            with torch.cuda.stream(s):
+                got.append(dt.render_backward(tape, seed))
+        torch.cuda.synchronize()
+        for g, w in zip(got, want):
+            _near(g, w)
 
 
 def test_scenes_that_share_a_gradient_add_up():
