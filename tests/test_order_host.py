@@ -24,6 +24,6 @@ def test_an_entry_outside_the_level_is_reported(tmp_path):
     src.write_text(SOURCE)
     subprocess.run([B._nvcc(), *B.ARCH, *B.NVCC_FLAGS, "-I", B.CSRC, "-o", str(exe), str(src)], check=True)
     assert subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout == "0"
-    # the traversals read the order through it alone
+    # the traversals (a lane per ray, four lanes per ray) read the order through it alone
     trace = open(B.CSRC + "/dt_trace.cu").read()
-    assert trace.count("order_position(") == 3 and "W.sflag[start + " not in trace
+    assert trace.count("order_position(") >= 2 and "W.sflag[start + " not in trace and "order[" not in trace
