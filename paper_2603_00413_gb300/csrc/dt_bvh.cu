@@ -1371,9 +1371,15 @@ __device__ __forceinline__ const float4* child_box(const BvhView& B, int c) {
 // traced with coded and exact boxes, took 1477 and 1614 us (edges of 15 steps),
 // 1589 and 1623 (10), 1777 and 1609 (6), 2672 and 1606 (2.6), 14970 and 1458 (0.5);
 // 200k queries of it 156 and 157, 168 and 155, 188 and 158, 283 and 156, 1189 and
-// 160 us.  Meshes of 19k and 307k triangles cross at the same edge length.
+// 160 us.  Meshes of 19k and 307k triangles cross at the same edge length.  A scene
+// of few triangles has no such patches, and its rays would test all of a part that
+// one grid step holds: there one node shorter than kQTinyNode steps decides (80
+// triangles of unit size above a ground triangle of 1e4 and 1e5, a frame of 512x512:
+// coded 861 and 1492 us, exact 372 and 374; float boxes of before 478).
 constexpr int kQCluster = 4;
 constexpr float kQPatch = 26.0f;
+constexpr int kQTiny = 1024;  // nodes of a scene of few triangles
+constexpr float kQTinyNode = 8.0f;
 
 __global__ void k_node_boxes(BvhView B) {
   chain_begin();
@@ -1419,7 +1425,9 @@ __global__ void k_node_boxes(BvhView B) {
     X[1] = make_float4(lo[1].x, hi[1].x, lo[1].y, hi[1].y);
     X[2] = make_float4(lo[0].z, hi[0].z, lo[1].z, hi[1].z);
     X[3] = make_float4(__int_as_float(ch.x), __int_as_float(ch.y), 0.f, 0.f);
-    if (n_int > 256 && longest_side(B.box_int + 2 * j) < kQPatch * step) {
+    if (n_int <= kQTiny) {
+      if (j > 0 && longest_side(B.box_int + 2 * j) < kQTinyNode * step) atomicAdd(&B.hdr->coarse, kQCoarse + 1);
+    } else if (longest_side(B.box_int + 2 * j) < kQPatch * step) {
       int p = j;
       for (int l = 0; l < kQCluster && p > 0; ++l) p = B.parent[p];
       if (p > 0 && p < n_int && longest_side(B.box_int + 2 * p) < kQPatch * step) atomicAdd(&B.hdr->coarse, 1);

@@ -21,6 +21,11 @@ def _scene(kind, checkpoint=False):
     if kind == "resolved":
         V, F = S.two_tori_mesh(36)
         cams, t_min = S.fibonacci_views(VIEWS, 3.0, W, H), 1e-5
+    elif kind == "ground":  # few triangles, and one 1e5 times their size
+        V, F = S.icosphere(1)
+        V = np.concatenate([V, np.float32([[-1e5, -2, -1e5], [1e5, -2, -1e5], [0, -2, 1e5]])])
+        F = np.concatenate([F, np.int32([[len(V) - 3, len(V) - 1, len(V) - 2]])])
+        cams, t_min = [S.camera((0.3 + 0.01 * k, 0.5, 3.0), (0, 0, 0), (0, 1, 0), 45.0, W, H) for k in range(VIEWS)], 1e-5
     else:  # a large sphere, and beside it a small one with edges of two steps of the codes' grid
         scale = 1e-3
         V, F = S.icosphere(2)
@@ -83,8 +88,9 @@ def test_a_batch_traces_each_scene_with_its_own_nodes():
         np.testing.assert_allclose(img.cpu().numpy(), a[0][0].cpu().numpy(), rtol=1e-6, atol=1e-6)
 
 
-def test_an_unresolved_part_costs_what_float_boxes_do():
-    gs = _scene("unresolved")
+@pytest.mark.parametrize("kind", ["unresolved", "ground"])
+def test_an_unresolved_part_costs_what_float_boxes_do(kind):
+    gs = _scene(kind)
     got = {}
     for width in (2, 4):
         old = dt.set_tuning(bvh_width=width)
@@ -99,5 +105,6 @@ def test_an_unresolved_part_costs_what_float_boxes_do():
     # arbitrary rays: the camera rays, asked again
     si, sf = dt.dump_segments(tape)
     cam = si[:, 1] == 1
-    tri, tbb = dt.closest_hit(gs.bvh, sf[cam][:, 3:6].contiguous(), sf[cam][:, 6:9].contiguous(), t_min=1e-8)
+    tri, tbb = dt.closest_hit(gs.bvh, sf[cam][:, 3:6].contiguous(), sf[cam][:, 6:9].contiguous(),
+                              t_min=gs.params.t_min)
     assert torch.equal(tri, si[cam][:, 2]) and torch.equal(tbb, sf[cam][:, :3])
