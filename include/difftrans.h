@@ -453,10 +453,11 @@ dt_status dt_edge_loss_grad(const void* d_topo, int32_t nv, int32_t nf, const fl
  * refills its idle lanes from the level's queue once trace_refill of them
  * are idle; trace_blocks_per_sm sizes its grid and register budget in units
  * of 256 resident threads per SM (CTAs of 128 threads; 5 runs nine of them).
- * shade_blocks_per_sm sizes the grid of the shading and adjoint kernels.
+ * shade_blocks_per_sm sizes the grid of the shading kernel.
  * bvh_width selects the node format the traversal reads: 2 (binary nodes,
- * 32 B: boxes in 16-bit codes, rounded outward; renders and batches of up to
- * 40,960 camera rays share a ray among four lanes on the 4-wide nodes
+ * 32 B: boxes in 16-bit codes, rounded outward, or 64 B with exact boxes for
+ * a scene with parts that the codes cannot resolve; renders and batches of
+ * up to 40,960 camera rays share a ray among four lanes on the 4-wide nodes
  * instead) or 4 (4-wide nodes, 128 B: the binary nodes at even depth with
  * their grandchildren as children, a lane per ray); both are kept current by
  * build/refit.
@@ -478,8 +479,13 @@ dt_status dt_edge_loss_grad(const void* d_topo, int32_t nv, int32_t nf, const fl
  * traces every level in append order: its levels are a few thousand
  * segments, where the order's three launches per level cost more than the
  * coherence gains.
- * Defaults {192, 8, 5, 4, 2, 1, 20, 65536}; results do not depend on them
- * (the same closest hit is found).  dt_set_tuning rejects values outside
+ * Defaults {192, 8, 5, 4, 2, 1, 20, 65536}; results do not depend on them:
+ * the same closest hit is found, but for a ray that meets an edge in its
+ * last bits, where exact boxes (bvh_width 4, unresolved scenes) may leave out
+ * one of the edge's two triangles and coded ones (and those of small
+ * renders, which are widened by 84 roundings) test both and keep the nearer
+ * or the smaller one; so may a render differ from the same views in one of
+ * more than 40,960 rays.  dt_set_tuning rejects values outside
  * steps 1..256, refill 1..32, trace 1..8, shade 1..16, width 2 or 4,
  * builder 0 or 1, order 0 or 12..22, order_min_rays >= 0.
  * ------------------------------------------------------------------------ */

@@ -357,10 +357,11 @@ __global__ void __launch_bounds__(256, kAdjointMinBlocks<kBatch, kGrid>)
 // texture.  March tiles (dt_medium.cuh), a unit being 32 segments on one level;
 // the levels' parts of dJ/do and dJ/dd meet in shared memory.
 // (A lane per segment over all levels, 32 at a time as they came, 8 views of
-// 360x360 with an 8-level hash texture took 24.5 ms at 9 lanes per instruction;
-// 8.1 now, of which the atomics are about 3 and the reads 2.  The same, moments
-// tape: 6.7.  16 views of 384x384 with a 64^3 grid: 2.56 -> 2.08 ms, half of it
-// the atomics.)
+// 360x360 with an 8-level hash texture took 23.7 ms at 9 lanes per instruction;
+// 9.2 now, moments tape 16.4 and 8.5.  16 views of 384x384 with a 64^3 grid: 3.26 ->
+// 2.30 ms, moments tape 2.48 -> 1.97.  At 100 views of 512x512 the atomics in L2
+// bound it and the forms come closer: grid 24.6 and 24.1, moments tape 20 and 22,
+// each within a fifth with where the gradient lies in memory.)
 template <bool kBatch, bool kHash>
 __global__ void __launch_bounds__(kTileThreads, 3) k_medium_adjoint(WsView W, int k, const AdjRecords out_cur,
                                                                     const float4* med_side,

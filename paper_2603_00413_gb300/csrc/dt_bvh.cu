@@ -1,7 +1,7 @@
 // Geometry kernels: vertex normals (DiffTrans Sec. 3.4, Eq. 13) and their
 // backward, and the LBVH (Morton codes, a stable LSD radix sort, the Karras
-// 2012 hierarchy, bottom-up bounds written straight into the float4 node
-// layout that the traversal reads).
+// 2012 hierarchy, bottom-up bounds, and from them the nodes that the traversal
+// reads), with a binned SAH builder beside it.
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -481,7 +481,7 @@ __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float* __restrict_
 // ---- binned SAH build (top-down) ---------------------------------------------
 // A second builder of the same binary layout.  Top-down: each task is a
 // contiguous range of a primitive permutation; its split is the bin boundary
-// (of 32 centroid bins per axis; 16 in the warp builder) with the least
+// (of 32 centroid bins per axis; 16 in the small builder) with the least
 // surface area cost area(left box) * left count + area(right box) * right
 // count, and the range
 // is partitioned stably into [left | right].  Tasks larger than kSahSmall
@@ -496,7 +496,7 @@ __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float* __restrict_
 // knowing how many there are, this took 1.18 ms for 120k triangles and 0.67
 // ms for 5k, most of it launches; now 212
 // and 89 us.)  Smaller tasks are built
-// down to their leaves by one warp each, in shared memory.  An internal node
+// down to their leaves by one CTA each, in shared memory.  An internal node
 // is numbered by its split position s (the last position of its left child),
 // which is unique in [0, nf - 2]; the root's number is swapped with 0 so the
 // root is node 0.  Splits deeper than kSahFreeDepth (large tasks) or
@@ -505,7 +505,7 @@ __global__ void __launch_bounds__(kRefitLeaves) k_refit(const float* __restrict_
 // the geometry: bins are integer sums, minima and maxima, and partitions are
 // stable.
 constexpr int kSahBins = 32;       // bins per axis of the large-task levels
-constexpr int kSahSmallBins = 16;  // of the warp builder
+constexpr int kSahSmallBins = 16;  // of the small builder
 constexpr int kSahTiny = 4;        // ranges up to this size split at the centroid median
 constexpr int kSahSmall = 128;
 constexpr int kSahFreeDepth = 24;

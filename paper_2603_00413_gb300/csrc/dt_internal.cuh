@@ -1,8 +1,9 @@
 // Internal definitions shared by the CUDA translation units of libdifftrans:
 // float3 arithmetic, the device layouts of the BVH buffer and of the render
 // workspace (the segment "tape"), segment and status flag bits, and the
-// launch helpers.  FP32 throughout; no fast-math approximations (divisions
-// and square roots are IEEE round-to-nearest).
+// launch helpers.  FP32 throughout; divisions and square roots are IEEE
+// round-to-nearest, but for the coded boxes' planes (16-bit codes, approximate
+// reciprocal), which only choose the triangles to test and are rounded outward.
 #pragma once
 
 #include <cuda_runtime.h>

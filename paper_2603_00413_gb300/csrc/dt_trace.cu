@@ -166,9 +166,8 @@ struct HitSoFar {
 // Moller-Trumbore on a leaf; keeps the smallest t > tmin, ties to the smaller
 // triangle id, skipping the triangle the ray starts on.  No early returns:
 // the lanes of a warp test different triangles, and a branch per condition
-// runs the block's pieces one after another with a few lanes each (with the
-// branches in visit_node2 below gone as well: 13.2 -> 11.1 ms of traversal per
-// 48-view genus-2 step, then).
+// runs the block's pieces one after another with a few lanes each (with those of
+// the visits gone as well: 13.2 -> 11.1 ms of traversal per 48-view genus-2 step).
 __device__ __forceinline__ void test_leaf(const float4* __restrict__ tris, int leaf, float3 o, float3 d, int src,
                                           float tmin, HitSoFar& h, uint32_t& ntest) {
   const float4 a = __ldg(tris + 3 * leaf), b = __ldg(tris + 3 * leaf + 1), c = __ldg(tris + 3 * leaf + 2);
