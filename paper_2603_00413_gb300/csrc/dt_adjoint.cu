@@ -659,8 +659,12 @@ __device__ __forceinline__ float3 paper_loss_pixel(float3 ch, float3 c, float kc
 // kVec: all three arrays are 16-byte aligned, and a thread takes four pixels as
 // three 16-byte words of each; the last n mod 4 pixels go one by one.  It is
 // then bound by HBM: 6.3M pixels (226 MB) took 72 us with 4-byte accesses and
-// an atomic per warp, this takes 37.
+// an atomic per warp, this takes 37.  Fewer than kLossVecPixels go one by one, a
+// thread each, since four in a row are a longer chain than the atomics of so few
+// CTAs (device time of the call, four and one: 4,000 pixels 6.2 and 5.2 us, 1,000 6.2
+// and 4.2, 24,000 6.2 and 5.4, 50,000 to 100,000 6.2 both, 150,000 6.2 and 8.2).
 constexpr int kLossThreads = 256;
+constexpr int64_t kLossVecPixels = 65536;
 template <bool kVec>
 __global__ void __launch_bounds__(kLossThreads) k_paper_loss_grad(const float* __restrict__ img,
                                                                   const float* __restrict__ target, int64_t n,
@@ -717,7 +721,7 @@ void launch_paper_loss_grad(const float* img, const float* target, int64_t n, fl
   cudaMemsetAsync(loss, 0, 3 * sizeof(float), s);
   if (n == 0) return;
   ProfScope ps("k_paper_loss_grad", s);
-  const bool vec = (((uintptr_t)img | (uintptr_t)target | (uintptr_t)grad) & 15) == 0 && n >= 4;
+  const bool vec = (((uintptr_t)img | (uintptr_t)target | (uintptr_t)grad) & 15) == 0 && n >= kLossVecPixels;
   int64_t b = ((vec ? n / 4 : n) + kLossThreads - 1) / kLossThreads;
   if (b > 8 * num_sms()) b = 8 * num_sms();
   const float inv_n = 1.0f / (float)n;
