@@ -1328,6 +1328,15 @@ __global__ void k_node4_topology(BvhView B) {
   }
 }
 
+// 256-bit store of a whole sector (p 32-byte aligned).  With stores of 128 bits, which
+// write each sector in halves, keeping the exact nodes cost a refit of 82k triangles
+// 4.7 us of 49; it is 1.9 with every kind of node stored so.
+__device__ __forceinline__ void st_v8(float4* p, float4 a, float4 b) {
+  asm volatile("st.global.v8.f32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "f"(a.x), "f"(a.y), "f"(a.z), "f"(a.w), "f"(b.x),
+               "f"(b.y), "f"(b.z), "f"(b.w)
+               : "memory");
+}
+
 // child boxes of 4-wide node m from the binary boxes
 __device__ __forceinline__ void node4_boxes(const BvhView& B, int m) {
   const int4 sv = reinterpret_cast<const int4*>(B.node4)[8 * m + 7];
@@ -1344,7 +1353,10 @@ __device__ __forceinline__ void node4_boxes(const BvhView& B, int m) {
     }
     r[0][k] = lo.x; r[1][k] = hi.x; r[2][k] = lo.y; r[3][k] = hi.y; r[4][k] = lo.z; r[5][k] = hi.z;
   }
-  for (int row = 0; row < 6; ++row) B.node4[8 * m + row] = make_float4(r[row][0], r[row][1], r[row][2], r[row][3]);
+#pragma unroll
+  for (int row = 0; row < 6; row += 2)
+    st_v8(B.node4 + 8 * (size_t)m + row, make_float4(r[row][0], r[row][1], r[row][2], r[row][3]),
+          make_float4(r[row + 1][0], r[row + 1][1], r[row + 1][2], r[row + 1][3]));
 }
 
 // The nodes' child boxes after each refit, from the binary boxes: the 4-wide
@@ -1418,13 +1430,13 @@ __global__ void k_node_boxes(BvhView B) {
       w[3 * k + 1] = code_planes(a.y, b.y, rlo.y, inv);
       w[3 * k + 2] = code_planes(a.z, b.z, rlo.z, inv);
     }
-    B.node2[2 * j] = make_uint4(w[0], w[1], w[2], w[3]);
-    B.node2[2 * j + 1] = make_uint4(w[4], w[5], (uint32_t)ch.x, (uint32_t)ch.y);
+    st_v8(reinterpret_cast<float4*>(B.node2) + 2 * (size_t)j,
+          make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3])),
+          make_float4(__uint_as_float(w[4]), __uint_as_float(w[5]), __int_as_float(ch.x), __int_as_float(ch.y)));
     float4* X = B.node2x + 4 * (size_t)j;
-    X[0] = make_float4(lo[0].x, hi[0].x, lo[0].y, hi[0].y);
-    X[1] = make_float4(lo[1].x, hi[1].x, lo[1].y, hi[1].y);
-    X[2] = make_float4(lo[0].z, hi[0].z, lo[1].z, hi[1].z);
-    X[3] = make_float4(__int_as_float(ch.x), __int_as_float(ch.y), 0.f, 0.f);
+    st_v8(X, make_float4(lo[0].x, hi[0].x, lo[0].y, hi[0].y), make_float4(lo[1].x, hi[1].x, lo[1].y, hi[1].y));
+    st_v8(X + 2, make_float4(lo[0].z, hi[0].z, lo[1].z, hi[1].z),
+          make_float4(__int_as_float(ch.x), __int_as_float(ch.y), 0.f, 0.f));
     if (n_int <= kQTiny) {
       if (j > 0 && longest_side(B.box_int + 2 * j) < kQTinyNode * step) atomicAdd(&B.hdr->coarse, kQCoarse + 1);
     } else if (longest_side(B.box_int + 2 * j) < kQPatch * step) {
